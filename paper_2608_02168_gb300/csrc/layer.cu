@@ -251,7 +251,7 @@ extern "C" hg_status hg_layer_fwd(const hg_graph* graph, const hg_layer_params* 
   } else {
     HG_TRY(aggregate_forward(graph, p->dtype, d, H_in, L.M, L.agg_part, L.work, s));
   }
-  return project_forward(graph, p, H_in, H_out, L, true, s);
+  return project_forward(graph, p, H_in, H_out, L, s);
 }
 
 namespace hg {
@@ -259,7 +259,7 @@ namespace hg {
 // Eq. 7 and Eq. 11 from the relation rows in L.M: U = sum_r M_r W_r W_agg + b, activation,
 // residual, optional LayerNorm.
 hg_status project_forward(const hg_graph* graph, const hg_layer_params* p, const void* H_in, void* H_out,
-                          const LayerLayout& L, bool compact, cudaStream_t s) {
+                          const LayerLayout& L, cudaStream_t s) {
   const GraphMeta& m = graph->meta;
   const int d = p->d;
   const size_t b = elem_size(p->dtype);
@@ -275,10 +275,10 @@ hg_status project_forward(const hg_graph* graph, const hg_layer_params* p, const
         ++a.nrel;
       }
       a.type = t;
-      a.mrow = compact ? graph->mrow : nullptr;
+      a.mrow = graph->mrow;
       a.msent = graph->csr_rows;
-      a.perm = compact ? graph->nperm + m.type_off[t] : nullptr;
-      a.tmask = compact ? graph->tmask + graph->tile_base[t] : nullptr;
+      a.perm = graph->nperm + m.type_off[t];
+      a.tmask = graph->tmask + graph->tile_base[t];
       a.b = (const __nv_bfloat16*)p->b_agg + (size_t)t * d;
       a.gamma = p->layernorm ? (const __nv_bfloat16*)p->ln_gamma + (size_t)t * d : nullptr;
       a.beta = p->layernorm ? (const __nv_bfloat16*)p->ln_beta + (size_t)t * d : nullptr;
@@ -310,7 +310,7 @@ hg_status project_forward(const hg_graph* graph, const hg_layer_params* p, const
   for (int t = 0; t < m.num_types; ++t) {
     FwdArgs a{};
     a.M = L.M;
-    a.mrow = compact ? graph->mrow : nullptr;
+    a.mrow = graph->mrow;
     a.msent = graph->csr_rows;
     for (int r = 0; r < m.num_rels; ++r) {
       if (m.rel_dst[r] != t) continue;
@@ -356,7 +356,7 @@ extern "C" hg_status hg_layer_bwd(const hg_graph* graph, const hg_layer_params* 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   LayerLayout L;
   carve_layer(graph, p->d, p->dtype, const_cast<void*>(saved), scratch, &L, nullptr, nullptr, p->fused != 0);
-  HG_TRY(project_backward(graph, p, H_in, dH_out, grads, L, true, true, s));
+  HG_TRY(project_backward(graph, p, H_in, dH_out, grads, L, true, s));
   if (dH_in) HG_TRY(aggregate_backward(graph, p->dtype, p->d, L.dMs, L.dY, dH_in, L.agg_part, L.work, s));
   return HG_OK;
 }
@@ -366,7 +366,7 @@ namespace hg {
 // Backward of project_forward: L.dY = the residual path's dL/dH_in, L.dMs = dL/dM_r (divided by
 // deg_r when deg_scale is set, for the mean's transposed gather), and every weight gradient.
 hg_status project_backward(const hg_graph* graph, const hg_layer_params* p, const void* H_in, const void* dH_out,
-                           const hg_layer_grads* grads, const LayerLayout& L, bool deg_scale, bool compact,
+                           const hg_layer_grads* grads, const LayerLayout& L, bool deg_scale,
                            cudaStream_t s) {
   const GraphMeta& m = graph->meta;
   const int d = p->d;
@@ -405,8 +405,8 @@ hg_status project_backward(const hg_graph* graph, const hg_layer_params* p, cons
       a.gamma = p->layernorm ? (const __nv_bfloat16*)p->ln_gamma + (size_t)t * d : nullptr;
       a.b = (const __nv_bfloat16*)p->b_agg + (size_t)t * d;
       a.csr_ptr = deg_scale ? graph->csr_ptr : nullptr;
-      a.mlist = compact ? graph->mlist : nullptr;
-      a.mbase = compact ? graph->mbase : nullptr;
+      a.mlist = graph->mlist;
+      a.mbase = graph->mbase;
       a.dY = (__nv_bfloat16*)L.dY;
       a.dU = (__nv_bfloat16*)L.dU;
       a.dMs = (__nv_bfloat16*)L.dMs;
@@ -433,7 +433,7 @@ hg_status project_backward(const hg_graph* graph, const hg_layer_params* p, cons
         ++a.nrel;
       }
       a.csr_ptr = deg_scale ? graph->csr_ptr : nullptr;
-      a.mrow = compact ? graph->mrow : nullptr;
+      a.mrow = graph->mrow;
       a.msent = graph->csr_rows;
       a.dY = L.dY;
       a.dU = L.dU;
@@ -461,38 +461,19 @@ hg_status project_backward(const hg_graph* graph, const hg_layer_params* p, cons
                                    m.type_off[t + 1] - m.type_off[t], L.wpart, L.G + (size_t)r * d * d, L.rtmp,
                                    s));
     }
-  } else if (tc && compact) {  // G_r = M_r^T dU over each relation's stored rows (dU rows gathered)
+  } else if (tc) {  // G_r = M_r^T dU over each relation's stored rows (dU rows gathered)
     for (int r = 0; r < m.num_rels; ++r) {
       const int t = m.rel_dst[r];
       HG_TRY(tc_weight_grad_rows(d, L.M, graph->csr_rows, graph->mlist, graph->mbase, r, m.row_base[r], L.dU,
                                  m.type_off[t], m.type_off[t + 1] - m.type_off[t], L.wpart, L.G + (size_t)r * d * d,
                                  L.rtmp, s));
     }
-  } else if (tc) {  // G_r = M_r^T dU, the relations into one type sharing the loads of dU
-    for (int t = 0; t < m.num_types; ++t) {
-      const int64_t n = m.type_off[t + 1] - m.type_off[t];
-      int64_t x0[kMaxRels];
-      float* outs[kMaxRels];
-      int R = 0;
-      for (int r = 0; r <= m.num_rels; ++r) {
-        if (r < m.num_rels && m.rel_dst[r] == t) {
-          x0[R] = m.row_base[r];
-          outs[R] = L.G + (size_t)r * d * d;
-          ++R;
-        }
-        if (R > 0 && (R == wgrad_tc_max_rels(d) || r == m.num_rels)) {
-          HG_TRY(tc_weight_grad(d, L.M, x0, R, L.dU, m.type_off[t], n, L.wpart, outs, L.rtmp, s));
-          R = 0;
-        }
-      }
-    }
   } else {
     for (int r = 0; r < m.num_rels; ++r) {
       const int t = m.rel_dst[r];
       const int64_t n = m.type_off[t + 1] - m.type_off[t];
       HG_TRY(weight_grad(p->dtype, d, L.M, m.row_base[r], L.dZ, m.type_off[t], n, L.wpart,
-                         grads->dW_rel + (size_t)r * d * d, L.rtmp, s, compact ? graph->mrow : nullptr,
-                         graph->csr_rows));
+                         grads->dW_rel + (size_t)r * d * d, L.rtmp, s, graph->mrow, graph->csr_rows));
     }
   }
   if (tc)  // dW_r = G_r W_agg^T, dW_agg[t] = sum_{r -> t} W_r^T G_r

@@ -164,15 +164,26 @@ size_t reduce_tmp_floats(int splits, int64_t count);
 hg_status reduce_partials3(const float* part, int64_t stride, int splits, int64_t seg, float* out0, float* out1,
                            float* out2, cudaStream_t s);
 int wgrad_splits(int64_t n);
+// The stored (non-empty) rows of relation `rel`: compact rows k = base[rel] .. base[rel + 1] (device),
+// each at node list[k] - row0 of its destination type.  list null: no map.
+struct RowMap {
+  const int32_t* list = nullptr;
+  const int32_t* base = nullptr;
+  int rel = 0;
+  int64_t row0 = 0;
+  int scatter = 0;  // 0: A indexed by node, out by compact row; 1: A by compact row, out by node
+};
 // Tensor-core row product (bf16): out[r][ocol0 + c] (=, or += when accumulate) scale A[r] B + bias,
 // A: n x d rows (row stride d), B: d x d row-major, bias: d or null; out row stride ldo; scale =
-// scale_mul * (*scale_ptr), scale_ptr a device fp32 scalar or null (1).
+// scale_mul * (*scale_ptr), scale_ptr a device fp32 scalar or null (1).  With a map, over the stored
+// rows only (at most n of them).
 hg_status rows_gemm_tc(int d, const void* A, int64_t n, const void* B, const void* bias, void* out, int64_t ldo,
-                       int ocol0, int accumulate, const float* scale_ptr, float scale_mul, cudaStream_t s);
+                       int ocol0, int accumulate, const float* scale_ptr, float scale_mul, cudaStream_t s,
+                       const RowMap& map = RowMap{});
 
 // Buffers of one layer (saved for the backward, and scratch).
 struct LayerLayout {
-  void* M;        // saved: csr_rows x d relation rows (means, or attention-weighted sums)
+  void* M;        // saved: relation rows (means, or attention-weighted sums), up to csr_rows x d, compact
   void* Mlong;    // saved (fused mean layer): long_cap x d means of the rows above kFuseRuns runs
   void* Z;        // saved (fp32 storage only): N x d
   void* U;        // saved: N x d pre-activation
@@ -197,14 +208,13 @@ void carve_layer(const hg_graph* g, int d, hg_dtype dt, void* saved, void* scrat
                  size_t* saved_bytes, size_t* scratch_bytes, bool fused = false);
 RelDst rel_dst_of(const GraphMeta& m);
 // Eq. 7 and Eq. 11 from the relation rows in L.M (bias, activation, residual, optional LayerNorm).
-// compact: L.M holds the non-empty CSR rows only, in the graph's compact order (the mean layer);
-// otherwise one row per CSR row (the attention layer's weighted sums).
+// L.M holds the non-empty CSR rows only, in the graph's compact order.
 hg_status project_forward(const hg_graph* graph, const hg_layer_params* p, const void* H_in, void* H_out,
-                          const LayerLayout& L, bool compact, cudaStream_t s);
-// Its backward: L.dY (residual path), L.dMs (dL/dM_r, divided by deg_r when deg_scale; compact rows
-// when compact), the weight gradients into grads.
+                          const LayerLayout& L, cudaStream_t s);
+// Its backward: L.dY (residual path), L.dMs (dL/dM_r, divided by deg_r when deg_scale; compact rows),
+// the weight gradients into grads.
 hg_status project_backward(const hg_graph* graph, const hg_layer_params* p, const void* H_in, const void* dH_out,
-                           const hg_layer_grads* grads, const LayerLayout& L, bool deg_scale, bool compact,
+                           const hg_layer_grads* grads, const LayerLayout& L, bool deg_scale,
                            cudaStream_t s);
 
 }  // namespace hg

@@ -80,3 +80,34 @@ def test_hgt_is_bitwise_repeatable():
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     for k in KEYS:
         assert np.array_equal(a[2][k], b[2][k]), k
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("rows", [1, 128, 129])
+def test_hgt_few_stored_rows(dtype, rows):
+    """Only `rows` targets of relation 0 have in-edges and relation 1 has none: products over the stored rows at the
+    edges of a 128-row tile, and over no rows at all."""
+    need_gpu()
+    hg = lib()
+    sp = hgsynth.spec("tiny-10k", n_user=401, n_risk=103, num_edges=6_000, n_overlap=10, dtype=dtype)
+    w = hgsynth.make_workload(sp, random_affine=True, with_ids=False)
+    p = hgsynth.make_hgt_params(sp, 4, bias_margin=BF16_RELU_MARGIN if dtype == "bf16" else None)
+    g = w.graph
+    keep = np.flatnonzero(g["rel"] == 0)
+    for k in ("src", "dst", "rel"):
+        g[k] = np.ascontiguousarray(g[k][keep])
+    lo = g["type_offsets"][g["rels"][0][1]]
+    g["dst"] = (lo + np.arange(keep.size) % rows).astype(g["dst"].dtype)
+    out, dH, gr = run_gpu(hg, w, p, 4, True, w.dH_top)
+    args = (g["src"], g["dst"], g["rel"], g["type_offsets"], g["rels"], p, w.X)
+    ref, _ = OH.hgt_forward(*args, 4, layernorm=True)
+    dref, gref = OH.hgt_backward(*args, w.dH_top, 4, layernorm=True)
+    assert relerr(out, ref) <= TOL[dtype] and relerr(dH, dref) <= TOL[dtype]
+    for k in KEYS:
+        # with one relation b_K shifts all scores of a softmax alike: its gradient is zero, what is left is rounding;
+        # dmu = <W_att, dW_att> / mu, a sum of cancelling terms, is off by at most |W_att| |error of dW_att| / mu
+        scale = np.abs(gref["W_K" if k == "b_K" else k]).max()
+        if k == "mu":
+            scale = np.linalg.norm(p["W_att"][0]) * np.linalg.norm(gref["W_att"][0]) / abs(p["mu"][0])
+        assert np.abs(gr[k] - gref[k]).max() <= TOL[dtype] * scale, k
+    assert hg.hg_device_status() == 0
