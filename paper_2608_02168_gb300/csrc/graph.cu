@@ -692,10 +692,13 @@ __global__ void __launch_bounds__(256) order_scatter(const int32_t* __restrict__
   }
 }
 
+// *nzero = nodes of the type with mask 0 (the scan's entry of mask 1, block 0);
 // tmask[q] = OR of the masks at positions kProjTileRows q .. + kProjTileRows - 1 (one warp per tile)
 __global__ void __launch_bounds__(256) order_tiles(const int32_t* __restrict__ csr_ptr, TypeRels tr, int64_t n,
                                                    const int32_t* __restrict__ perm, int64_t tiles,
-                                                   int32_t* __restrict__ tmask) {
+                                                   int32_t* __restrict__ tmask, const int32_t* __restrict__ nz_src,
+                                                   int32_t* __restrict__ nzero) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *nzero = *nz_src;
   const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (q >= tiles) return;
@@ -728,7 +731,7 @@ struct GraphLayout {
   int32_t *agg_ptr, *agg_col, *agg_cnt, *agg_chunk_ofs, *agg_chunk_row;
   int32_t *bagg_ptr, *bagg_col, *bagg_cnt, *bagg_chunk_ofs, *bagg_chunk_row;
   int32_t *mrow, *mlist, *mbase;  // non-empty CSR rows: compact index per row, row per index, per relation
-  int32_t *nperm, *tmask, *ohist, *oofs;  // node order by relation mask, tile masks, the sort's counts
+  int32_t *nperm, *tmask, *nzero, *ohist, *oofs;  // node order by relation mask, tile masks, the sort's counts
   int32_t *long_ofs, *long_list;          // the fused layer's long rows
   SortBuffers sort;
 };
@@ -760,6 +763,7 @@ static size_t carve_graph(void* ws, int64_t E, int64_t rows, int64_t crows, int6
   L->mbase = c.take<int32_t>(kMaxRels + 1);
   L->nperm = c.take<int32_t>(std::max<int64_t>(N, 1));
   L->tmask = c.take<int32_t>(order_tiles_cap(N));
+  L->nzero = c.take<int32_t>(kMaxTypes);
   L->long_ofs = c.take<int32_t>(rows + 1);
   L->long_list = c.take<int32_t>(long_cap(E));
   L->ohist = c.take<int32_t>(order_hist_cap(N) + 1);
@@ -983,7 +987,8 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
                   nblk, (const int32_t*)L.oofs, perm));
     const int64_t tiles = tile_base[t + 1] - tile_base[t];
     HG_TRY(launch("order_tiles", order_tiles, dim3((unsigned)ceil_div(tiles * 32, 256)), dim3(256), 0, s,
-                  (const int32_t*)L.csr_ptr, tr, n, (const int32_t*)perm, tiles, L.tmask + tile_base[t]));
+                  (const int32_t*)L.csr_ptr, tr, n, (const int32_t*)perm, tiles, L.tmask + tile_base[t],
+                  (const int32_t*)L.oofs + nblk, L.nzero + t));
   }
   // chunk tables over runs for rows above the hub degree (mean and attention layers)
   HG_TRY(chunk_table(L.agg_ptr, rows, L.agg_chunk_ofs, L.agg_chunk_row, L, s));
@@ -1021,6 +1026,7 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
   gh->mbase = L.mbase;
   gh->nperm = L.nperm;
   gh->tmask = L.tmask;
+  gh->nzero = L.nzero;
   gh->long_ofs = L.long_ofs;
   gh->long_list = L.long_list;
   gh->long_cap = long_cap(E);

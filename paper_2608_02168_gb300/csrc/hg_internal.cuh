@@ -157,6 +157,7 @@ struct hg_graph {
   int32_t* nperm;           // [N]
   int32_t* tmask;           // [tile_base[num_types]]
   int64_t tile_base[hg::kMaxTypes + 1];
+  int32_t* nzero;           // [kMaxTypes], device: positions of each type's order with mask 0 (unset for an empty type)
   // CSR rows with more than kFuseRuns runs (the fused layer's long rows): long_ofs = exclusive scan
   // of the flags (row is long iff long_ofs[row + 1] > long_ofs[row]; long_ofs[row] is its compact
   // slot, long_ofs[csr_rows] their number), long_list[k] = the CSR row of slot k.

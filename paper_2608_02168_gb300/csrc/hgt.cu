@@ -22,7 +22,8 @@
 //   to the weights.
 // Edge work is warp per row (a lane holds d / 32 consecutive features, the 32 / S lanes of a head
 // reduce by shuffles); rows above the hub degree are split into chunks whose partial results are
-// merged in chunk order, so every reduction has a fixed order (deterministic, atomic-free).  The
+// merged in chunk order, so every reduction has a fixed order (the only atomics are the claim
+// counters, which decide who computes a row and not the order of its terms).  The
 // dense row products run on the tensor cores for bf16 (rows_gemm_tc.cu) and on CUDA cores for fp32.
 #include <cuda_bf16.h>
 
@@ -73,10 +74,57 @@ __device__ __forceinline__ void load_slice(const T* __restrict__ p, float (&f)[E
   }
 }
 
+// The same slice kept as loaded (bf16 pairs stay packed until they are used: half the registers of
+// the rows in flight).
+template <typename T, int E>
+struct RawSlice {
+  static constexpr int kWords = E * (int)sizeof(T) / 4;
+  uint32_t w[kWords];
+  __device__ __forceinline__ void load(const T* __restrict__ p) {
+    if constexpr (kWords == 1) {
+      w[0] = __ldg(reinterpret_cast<const unsigned int*>(p));
+    } else if constexpr (kWords == 2) {
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+      w[0] = v.x;
+      w[1] = v.y;
+    } else {
+#pragma unroll
+      for (int i = 0; i < kWords; i += 4) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p) + i / 4);
+        w[i] = v.x;
+        w[i + 1] = v.y;
+        w[i + 2] = v.z;
+        w[i + 3] = v.w;
+      }
+    }
+  }
+  __device__ __forceinline__ void get(float (&f)[E]) const {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) f[e] = __uint_as_float(w[e]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; e += 2) {
+        f[e] = __uint_as_float(w[e / 2] << 16);
+        f[e + 1] = __uint_as_float(w[e / 2] & 0xFFFF0000u);
+      }
+    }
+  }
+};
+
 template <typename T, int E>
 __device__ __forceinline__ void store_slice(T* __restrict__ p, const float (&f)[E]) {
+  if constexpr (sizeof(T) == 2 && E == 4) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(pack2_bf16(f[0], f[1]), pack2_bf16(f[2], f[3]));
+  } else if constexpr (sizeof(T) == 2 && E == 2) {
+    *reinterpret_cast<uint32_t*>(p) = pack2_bf16(f[0], f[1]);
+  } else if constexpr (E * sizeof(T) % 16 == 0) {
 #pragma unroll
-  for (int e = 0; e < E; ++e) p[e] = from_f32<T>(f[e]);
+    for (int e = 0; e < E; e += VecTraits<T>::kElems) st16(p + e, pack(f + e, T()));
+  } else {
+#pragma unroll
+    for (int e = 0; e < E; ++e) p[e] = from_f32<T>(f[e]);
+  }
 }
 
 // Sum over the lanes of this lane's head (lpw = 32 / S consecutive lanes).
@@ -215,7 +263,13 @@ struct HgtArgs {
   const int32_t* scnt;
   const int32_t* schunk_ofs;
   const int32_t* schunk_row;
-  const int32_t* mrow;  // compact row of each CSR row (>= csr_rows: the row has no in-edge)
+  const int32_t* mrow;   // compact row of each CSR row (>= csr_rows: the row has no in-edge)
+  const int32_t* mlist;  // CSR row of each compact row
+  const int32_t* mcount; // device: number of compact rows
+  // nodes by relation mask, per type: positions below nzero[t] have no in-edge at all
+  const int32_t* nperm;
+  const int32_t* nzero;
+  int32_t* work;         // claim counters of the node and row kernels (zeroed before each pass)
   const void* KV;       // N x 2d: K then V of each node
   // compact rows
   const void* Qp;    // d: relation-scaled queries
@@ -229,15 +283,50 @@ struct HgtArgs {
   float* part;       // chunk partials
 };
 
-constexpr int kBatch = 4;       // edges of a row in flight per warp (node kernels)
-constexpr int kBatchChunk = 4;  // the same for the chunk kernels (eight was slower: registers)
+// Edge passes.  All of them are bound by the latency of the row gathers (a run's two rows, 2 d bytes
+// each, from L2 or HBM) and by the uneven rows, so
+//  - warps claim work from a counter, a few nodes or rows at a time (a warp per node in grid order
+//    left the SMs waiting for the blocks that held the longest rows);
+//  - the bounds of everything claimed are loaded at once, one (node, relation) or row per lane;
+//  - a row's run entries are loaded 32 at a time, one per lane, and handed out by shuffles, and the
+//    first window is loaded together with the row's own slices;
+//  - hub chunks are a whole CTA each, a warp per eighth, merged in warp order.
+// 1M nodes, 20M edges (3.2M runs), d = 128 bf16: fwd nodes 2.01 -> 0.61 ms, target pass 2.32 -> 0.49 ms, source
+// pass 1.77 -> 0.58 ms, the three chunk passes 1.31 -> 0.65 ms; the layer forward + backward 11.05 -> 6.60 ms.
+constexpr int kBatch = 4;        // runs of a row in flight per warp
+constexpr int kEdgeWarps = 4;    // warps per CTA of the node and row kernels
+constexpr int kChunkWarps = 8;   // warps per hub chunk
+constexpr int kChunkPart = kChunkEdges / kChunkWarps;
+constexpr unsigned kAll = 0xffffffffu;
 
-// Online softmax step for one run of w parallel edges (per lane: its head's running maximum m and
-// sum l; the value accumulators are rescaled when the maximum grows).
-template <int E, int NACC>
-__device__ __forceinline__ void online_step(float s, float w, const float (&v)[E], float& m, float& l,
-                                            float (&acc)[NACC][E], int slot) {
-  const float mn = fmaxf(m, s);
+// One window of run entries: lane l holds entry base + l.
+struct RunWindow {
+  int col, cnt;
+  __device__ __forceinline__ void load(const int32_t* __restrict__ c, const int32_t* __restrict__ n, int64_t base,
+                                       int64_t end) {
+    const int64_t e = base + (threadIdx.x & 31);
+    col = e < end ? __ldg(c + e) : 0;
+    cnt = e < end ? __ldg(n + e) : 0;
+  }
+};
+
+// claims `n` consecutive items
+__device__ __forceinline__ int64_t claim(int32_t* counter, int n) {
+  int c = 0;
+  if ((threadIdx.x & 31) == 0) c = atomicAdd(counter, n);
+  return __shfl_sync(kAll, c, 0);
+}
+
+// Online softmax over a batch of nb runs of one row (per lane: its head's running maximum m and sum l;
+// the value accumulators are rescaled when the maximum grows).
+template <typename T, int E, int NACC>
+__device__ __forceinline__ void online_batch(const float (&sc)[kBatch], const float (&w)[kBatch],
+                                             const RawSlice<T, E> (&v)[kBatch], int nb, float& m, float& l,
+                                             float (&acc)[NACC][E], int slot) {
+  float mn = m;
+#pragma unroll
+  for (int u = 0; u < kBatch; ++u)
+    if (u < nb) mn = fmaxf(mn, sc[u]);
   if (mn > m) {
     const float so = expf(m - mn);
     l *= so;
@@ -247,242 +336,352 @@ __device__ __forceinline__ void online_step(float s, float w, const float (&v)[E
       for (int e = 0; e < E; ++e) acc[k][e] *= so;
     m = mn;
   }
-  const float p = w * expf(s - m);  // w edges with this score
-  l += p;
+#pragma unroll
+  for (int u = 0; u < kBatch; ++u) {
+    if (u >= nb) break;
+    const float p = w[u] * expf(sc[u] - m);  // w runs with this score
+    l += p;
+    float f[E];
+    v[u].get(f);
+#pragma unroll
+    for (int k = 0; k < NACC; ++k)
+      if (k == slot)
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[k][e] = fmaf(p, f[e], acc[k][e]);
+  }
+}
+
+// The runs [beg, end) of one CSR row against the query slice q, folded into (m, l, acc[slot]); `win`
+// holds the first window.
+template <typename T, int D, int NACC>
+__device__ __forceinline__ void fwd_edges(const HgtArgs& a, int64_t beg, int64_t end, RunWindow win,
+                                          const float (&q)[D / 32], int lph, float& m, float& l,
+                                          float (&acc)[NACC][D / 32], int slot) {
+  constexpr int E = D / 32;
+  const int lane = threadIdx.x & 31;
+  const T* KV = (const T*)a.KV + lane * E;
+  for (int64_t w0 = beg; w0 < end; w0 += 32) {
+    if (w0 > beg) win.load(a.dcol, a.dcnt, w0, end);
+    const int n = (int)min((int64_t)32, end - w0);
+    for (int b = 0; b < n; b += kBatch) {
+      const int nb = min(kBatch, n - b);
+      RawSlice<T, E> k[kBatch], v[kBatch];
+      float w[kBatch], sc[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int64_t src = __shfl_sync(kAll, win.col, b + u);
+        w[u] = (float)__shfl_sync(kAll, win.cnt, b + u);
+        if (u < nb) {
+          k[u].load(KV + src * 2 * D);
+          v[u].load(KV + src * 2 * D + D);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        sc[u] = 0.f;
+        if (u >= nb) break;
+        float f[E];
+        k[u].get(f);
+#pragma unroll
+        for (int e = 0; e < E; ++e) sc[u] = fmaf(f[e], q[e], sc[u]);
+        sc[u] = head_sum(sc[u], lph);
+      }
+      online_batch<T, E, NACC>(sc, w, v, nb, m, l, acc, slot);
+    }
+  }
+}
+
+// (m, l, acc) += (pm, pl, pv) of a later part of the same softmax
+template <int E, int NACC>
+__device__ __forceinline__ void merge_part(float pm, float pl, const float (&pv)[E], float& m, float& l,
+                                           float (&acc)[NACC][E], int slot) {
+  const float mn = fmaxf(m, pm);
+  if (mn > m) {
+    const float so = expf(m - mn);
+    l *= so;
+#pragma unroll
+    for (int k = 0; k < NACC; ++k)
+#pragma unroll
+      for (int e = 0; e < E; ++e) acc[k][e] *= so;
+    m = mn;
+  }
+  const float sp = expf(pm - m);
+  l = fmaf(pl, sp, l);
 #pragma unroll
   for (int k = 0; k < NACC; ++k)
     if (k == slot)
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[k][e] = fmaf(p, v[e], acc[k][e]);
+      for (int e = 0; e < E; ++e) acc[k][e] = fmaf(sp, pv[e], acc[k][e]);
 }
 
-// The edges [beg, end) of one CSR row against the query slice q, folded into (m, l, acc[slot]).
-template <typename T, int D, int NACC, int NB = kBatch>
-__device__ __forceinline__ void fwd_edges(const HgtArgs& a, int64_t beg, int64_t end, const float (&q)[D / 32], int lph,
-                                          float& m, float& l, float (&acc)[NACC][D / 32], int slot) {
-  constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31;
-  const T* KV = (const T*)a.KV;
-  for (int64_t e0 = beg; e0 < end; e0 += NB) {
-    int src[NB];
-    float w[NB];
-#pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      src[u] = e0 + u < end ? __ldg(a.dcol + e0 + u) : -1;
-      w[u] = e0 + u < end ? (float)__ldg(a.dcnt + e0 + u) : 0.f;
-    }
-    float k[NB][E], v[NB][E];
-#pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      if (src[u] >= 0) {
-        load_slice<T, E>(KV + (int64_t)src[u] * 2 * D + lane * E, k[u]);
-        load_slice<T, E>(KV + (int64_t)src[u] * 2 * D + D + lane * E, v[u]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      if (src[u] < 0) break;
-      float s = 0.f;
-#pragma unroll
-      for (int e = 0; e < E; ++e) s = fmaf(k[u][e], q[e], s);
-      s = head_sum(s, lph);
-      online_step<E, NACC>(s, w[u], v[u], m, l, acc, slot);
-    }
-  }
-}
-
-// One warp per chunk of a hub row: (m, l, unnormalised value sum) of the chunk's edges.
+// One CTA per chunk of a hub row: (m, l, unnormalised value sum) of the chunk's runs.  Warp w takes
+// runs [64 w, 64 w + 64) of the chunk; warp 0 merges the warps' parts in order.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) hgt_fwd_chunks(HgtArgs a) {
+__global__ void __launch_bounds__(32 * kChunkWarps) hgt_fwd_chunks(HgtArgs a) {
   constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31, lph = 32 / a.S;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  __shared__ float part[kChunkWarps][32][E + 2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S;
   const int nchunks = a.dchunk_ofs[a.csr_rows];
   const int stride = 2 * a.S + D;
-  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nchunks; c += nw) {
+  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int row = a.dchunk_row[c];
-    const int64_t beg = (int64_t)a.dptr[row] + (int64_t)(c - a.dchunk_ofs[row]) * kChunkEdges;
-    const int64_t end = min((int64_t)a.dptr[row + 1], beg + kChunkEdges);
-    float q[E];
+    const int64_t cb = (int64_t)a.dptr[row] + (int64_t)(c - a.dchunk_ofs[row]) * kChunkEdges;
+    const int64_t ce = min((int64_t)a.dptr[row + 1], cb + kChunkEdges);
+    const int64_t beg = cb + warp * kChunkPart, end = min(ce, beg + kChunkPart);
+    float q[E], m = -INFINITY, l = 0.f, acc[1][E];
     load_slice<T, E>((const T*)a.Qp + (int64_t)a.mrow[row] * D + lane * E, q);
-    float m = -INFINITY, l = 0.f, acc[1][E];
 #pragma unroll
     for (int e = 0; e < E; ++e) acc[0][e] = 0.f;
-    fwd_edges<T, D, 1, kBatchChunk>(a, beg, end, q, lph, m, l, acc, 0);
-    float* p = a.part + c * stride;
-    if (lane % lph == 0) {
-      p[2 * (lane / lph)] = m;
-      p[2 * (lane / lph) + 1] = l;
-    }
+    RunWindow win;
+    win.load(a.dcol, a.dcnt, beg, end);
+    fwd_edges<T, D, 1>(a, beg, end, win, q, lph, m, l, acc, 0);
 #pragma unroll
-    for (int e = 0; e < E; ++e) p[2 * a.S + lane * E + e] = acc[0][e];
+    for (int e = 0; e < E; ++e) part[warp][lane][e] = acc[0][e];
+    part[warp][lane][E] = m;
+    part[warp][lane][E + 1] = l;
+    __syncthreads();
+    if (warp == 0) {
+      for (int w = 1; w < kChunkWarps && cb + w * kChunkPart < ce; ++w) {
+        float pv[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) pv[e] = part[w][lane][e];
+        merge_part<E, 1>(part[w][lane][E], part[w][lane][E + 1], pv, m, l, acc, 0);
+      }
+      float* p = a.part + (int64_t)c * stride;
+      if (lane % lph == 0) {
+        p[2 * (lane / lph)] = m;
+        p[2 * (lane / lph) + 1] = l;
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) p[2 * a.S + lane * E + e] = acc[0][e];
+    }
+    __syncthreads();
   }
 }
 
-// One warp per node j: the softmax over all of j's in-edges (its rows of every relation into its
+// nodes with at least one in-edge
+__device__ __forceinline__ int64_t live_nodes(const HgtArgs& a) {
+  int64_t n = 0;
+  for (int t = 0; t < a.meta.num_types; ++t) {
+    const int64_t nt = a.meta.type_off[t + 1] - a.meta.type_off[t];
+    if (nt > 0) n += nt - a.nzero[t];
+  }
+  return n;
+}
+// The x-th of them as (type, local id), the types in order and each type's masks descending (nodes
+// with in-edges of every relation, which hold the most runs, come first); t = -1 past the last.
+__device__ __forceinline__ void live_node(const HgtArgs& a, int64_t x, int& t, int64_t& jl) {
+  for (t = 0; t < a.meta.num_types; ++t) {
+    const int64_t nt = a.meta.type_off[t + 1] - a.meta.type_off[t];
+    const int64_t live = nt > 0 ? nt - a.nzero[t] : 0;
+    if (x < live) {
+      jl = a.nperm[a.meta.type_off[t] + nt - 1 - x];
+      return;
+    }
+    x -= live;
+  }
+  t = -1;
+  jl = 0;
+}
+
+// A warp per node j: the softmax over all of j's in-edges (its rows of every relation into its
 // type, hub rows through their chunk partials in order), S_r(j) = sum alpha V for each relation.
-// The row bounds and query slices of all of j's rows are loaded before any edge.
+// Lane n KS + k holds the bounds of the claim's node n, relation slot k.
 template <typename T, int D, int KS>
-__global__ void __launch_bounds__(256, (D <= 128 && KS <= 4) ? 3 : 1) hgt_fwd_nodes(HgtArgs a) {
-  constexpr int E = D / 32;
+__global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1) hgt_fwd_nodes(HgtArgs a) {
+  constexpr int E = D / 32, NC = 32 / KS;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
-  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= a.N) return;
-  const int t = node_type_of(a.meta, j);
-  const int64_t jl = j - a.meta.type_off[t];
+  const int64_t total = live_nodes(a);
   const int stride = 2 * a.S + D;
-  int64_t row[KS];
-  int c0[KS], c1[KS];
-  int64_t e0[KS], e1[KS];
-  float q[KS][E];
-#pragma unroll
-  for (int k = 0; k < KS; ++k) {
-    const int r = a.rslot[t][k];
-    row[k] = -1;  // compact row
-    if (r < 0) continue;
-    const int64_t cr = a.meta.row_base[r] + jl;
-    const int64_t mr = a.mrow[cr];
-    if (mr < a.csr_rows) {
-      row[k] = mr;
-      c0[k] = a.dchunk_ofs[cr];
-      c1[k] = a.dchunk_ofs[cr + 1];
-      e0[k] = a.dptr[cr];
-      e1[k] = a.dptr[cr + 1];
-      load_slice<T, E>((const T*)a.Qp + mr * D + lane * E, q[k]);
-    }
-  }
-  float m = -INFINITY, l = 0.f, acc[KS][E];
-#pragma unroll
-  for (int k = 0; k < KS; ++k)
-#pragma unroll
-    for (int e = 0; e < E; ++e) acc[k][e] = 0.f;
-#pragma unroll
-  for (int k = 0; k < KS; ++k) {
-    if (row[k] < 0) continue;
-    if (c1[k] > c0[k]) {
-      for (int c = c0[k]; c < c1[k]; ++c) {
-        const float* p = a.part + (int64_t)c * stride;
-        const float pm = p[2 * (lane / lph)], pl = p[2 * (lane / lph) + 1];
-        const float mn = fmaxf(m, pm);
-        if (mn > m) {
-          const float so = expf(m - mn);
-          l *= so;
-#pragma unroll
-          for (int kk = 0; kk < KS; ++kk)
-#pragma unroll
-            for (int e = 0; e < E; ++e) acc[kk][e] *= so;
-          m = mn;
-        }
-        const float sp = expf(pm - m);
-        l = fmaf(pl, sp, l);
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[k][e] = fmaf(sp, p[2 * a.S + lane * E + e], acc[k][e]);
+  for (int64_t x0 = claim(a.work, NC); x0 < total; x0 = claim(a.work, NC)) {
+    int t = -1, mrow = -1, eb = 0, ee = 0, cb = 0, ce = 0;
+    int64_t jl = 0;
+    if (x0 + lane / KS < total) live_node(a, x0 + lane / KS, t, jl);
+    const int r = t >= 0 ? a.rslot[t][lane % KS] : -1;
+    if (r >= 0) {
+      const int64_t cr = a.meta.row_base[r] + jl;
+      const int mr = a.mrow[cr];
+      if (mr < a.csr_rows) {
+        mrow = mr;
+        eb = a.dptr[cr];
+        ee = a.dptr[cr + 1];
+        cb = a.dchunk_ofs[cr];
+        ce = a.dchunk_ofs[cr + 1];
       }
-    } else {
-      fwd_edges<T, D, KS>(a, e0[k], e1[k], q[k], lph, m, l, acc, k);
+    }
+    const int64_t node = t >= 0 ? a.meta.type_off[t] + jl : 0;
+    const int nn = (int)min((int64_t)NC, total - x0);
+    for (int n = 0; n < nn; ++n) {
+      int row[KS];
+      RawSlice<T, E> q[KS];
+      RunWindow win[KS];
+#pragma unroll
+      for (int k = 0; k < KS; ++k) {
+        row[k] = __shfl_sync(kAll, mrow, n * KS + k);
+        const int b = __shfl_sync(kAll, eb, n * KS + k), e = __shfl_sync(kAll, ee, n * KS + k);
+        if (row[k] >= 0) {
+          q[k].load((const T*)a.Qp + (int64_t)row[k] * D + lane * E);
+          win[k].load(a.dcol, a.dcnt, b, e);
+        }
+      }
+      float m = -INFINITY, l = 0.f, acc[KS][E];
+#pragma unroll
+      for (int k = 0; k < KS; ++k)
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[k][e] = 0.f;
+#pragma unroll
+      for (int k = 0; k < KS; ++k) {
+        const int b = __shfl_sync(kAll, eb, n * KS + k), e = __shfl_sync(kAll, ee, n * KS + k);
+        const int c0 = __shfl_sync(kAll, cb, n * KS + k), c1 = __shfl_sync(kAll, ce, n * KS + k);
+        if (row[k] < 0) continue;
+        if (c1 > c0) {
+          for (int c = c0; c < c1; c += kBatch) {  // kBatch partials loaded before the first is merged
+            float pm[kBatch], pl[kBatch], pv[kBatch][E];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+              if (c + u >= c1) break;
+              const float* p = a.part + (int64_t)(c + u) * stride;
+              pm[u] = p[2 * (lane / lph)];
+              pl[u] = p[2 * (lane / lph) + 1];
+#pragma unroll
+              for (int i = 0; i < E; ++i) pv[u][i] = p[2 * a.S + lane * E + i];
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+              if (c + u >= c1) break;
+              merge_part<E, KS>(pm[u], pl[u], pv[u], m, l, acc, k);
+            }
+          }
+        } else {
+          float qf[E];
+          q[k].get(qf);
+          fwd_edges<T, D, KS>(a, b, e, win[k], qf, lph, m, l, acc, k);
+        }
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+      for (int k = 0; k < KS; ++k) {
+        if (row[k] < 0) continue;
+        float o[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) o[e] = acc[k][e] * inv;
+        store_slice<T, E>((T*)a.Srows + (int64_t)row[k] * D + lane * E, o);
+      }
+      const int64_t j = __shfl_sync(kAll, node, n * KS);
+      if (lane % lph == 0) a.stats[j * a.S + lane / lph] = make_float2(l > 0.f ? m : 0.f, l);
     }
   }
-  const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-  for (int k = 0; k < KS; ++k) {
-    if (row[k] < 0) continue;
-    float o[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) o[e] = acc[k][e] * inv;
-    store_slice<T, E>((T*)a.Srows + row[k] * D + lane * E, o);
-  }
-  if (lane % lph == 0) a.stats[j * a.S + lane / lph] = make_float2(l > 0.f ? m : 0.f, l);
 }
 
 // D^s_j = sum over j's relation rows of <dS_r(j), S_r(j)> on head s, stored with the softmax statistics
-// on every row of j (the source pass reads them by row).  One warp per node.
+// on every row of j (the target and source passes read them by row).  One warp per node with in-edges.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) hgt_bwd_dstats(HgtArgs a) {
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
-  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= a.N) return;
-  const int t = node_type_of(a.meta, j);
-  const int64_t jl = j - a.meta.type_off[t];
-  float s = 0.f;
+  const int64_t total = live_nodes(a), nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < total; x += nw) {
+    int t;
+    int64_t jl;
+    live_node(a, x, t, jl);
+    int row = -1;  // lane k: the compact row of relation slot k
+    if (lane < kMaxRels && a.rslot[t][lane] >= 0) {
+      row = a.mrow[a.meta.row_base[a.rslot[t][lane]] + jl];
+      if (row >= a.csr_rows) row = -1;
+    }
+    float s = 0.f;
 #pragma unroll
-  for (int r = 0; r < kMaxRels; ++r) {
-    if (r >= a.meta.num_rels || a.meta.rel_dst[r] != t) continue;
-    const int64_t row = a.mrow[a.meta.row_base[r] + jl];
-    if (row >= a.csr_rows) continue;
-    float x[E], y[E];
-    load_slice<T, E>((const T*)a.dS + row * D + lane * E, x);
-    load_slice<T, E>((const T*)a.Srows + row * D + lane * E, y);
+    for (int k = 0; k < kMaxRels; ++k) {
+      const int64_t rk = __shfl_sync(kAll, row, k);
+      if (rk < 0) continue;
+      float u[E], v[E];
+      load_slice<T, E>((const T*)a.dS + rk * D + lane * E, u);
+      load_slice<T, E>((const T*)a.Srows + rk * D + lane * E, v);
 #pragma unroll
-    for (int e = 0; e < E; ++e) s = fmaf(x[e], y[e], s);
-  }
-  s = head_sum(s, lph);
-  if (lane % lph == 0) {
-    const float2 st = a.stats[j * a.S + lane / lph];
+      for (int e = 0; e < E; ++e) s = fmaf(u[e], v[e], s);
+    }
+    s = head_sum(s, lph);
+    const float2 st = a.stats[(a.meta.type_off[t] + jl) * a.S + lane / lph];
     const float4 v = make_float4(st.x, st.y > 0.f ? 1.f / st.y : 0.f, s, 0.f);
 #pragma unroll
-    for (int r = 0; r < kMaxRels; ++r) {
-      if (r >= a.meta.num_rels || a.meta.rel_dst[r] != t) continue;
-      const int64_t row = a.mrow[a.meta.row_base[r] + jl];
-      if (row < a.csr_rows) a.rstat[row * a.S + lane / lph] = v;
+    for (int k = 0; k < kMaxRels; ++k) {
+      const int64_t rk = __shfl_sync(kAll, row, k);
+      if (rk >= 0 && lane % lph == 0) a.rstat[rk * a.S + lane / lph] = v;
     }
   }
 }
 
-// sum over the edges [beg, end) of one row (relation r, target j) of de K(i), with
+// sum over the runs [beg, end) of one row (relation r, target j) of de K(i), with
 // de = alpha (<dS_r(j), V(i)> - D_j) and alpha from the saved softmax statistics.
-template <typename T, int D, int NB = kBatch>
-__device__ __forceinline__ void dst_edges(const HgtArgs& a, int64_t beg, int64_t end, const float (&q)[D / 32],
-                                          const float (&g)[D / 32], float m, float inv_l, float Dh, int lph,
-                                          float (&acc)[D / 32]) {
+template <typename T, int D>
+__device__ __forceinline__ void dst_edges(const HgtArgs& a, int64_t beg, int64_t end, RunWindow win,
+                                          const float (&q)[D / 32], const float (&g)[D / 32], float m, float inv_l,
+                                          float Dh, int lph, float (&acc)[D / 32]) {
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31;
-  const T* KV = (const T*)a.KV;
-  for (int64_t e0 = beg; e0 < end; e0 += NB) {
-    int src[NB];
-    float w[NB];
+  const T* KV = (const T*)a.KV + lane * E;
+  for (int64_t w0 = beg; w0 < end; w0 += 32) {
+    if (w0 > beg) win.load(a.dcol, a.dcnt, w0, end);
+    const int n = (int)min((int64_t)32, end - w0);
+    for (int b = 0; b < n; b += kBatch) {
+      const int nb = min(kBatch, n - b);
+      RawSlice<T, E> k[kBatch], v[kBatch];
+      float w[kBatch];
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      src[u] = e0 + u < end ? __ldg(a.dcol + e0 + u) : -1;
-      w[u] = e0 + u < end ? (float)__ldg(a.dcnt + e0 + u) : 0.f;
-    }
-    float k[NB][E], v[NB][E];
-#pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      if (src[u] >= 0) {
-        load_slice<T, E>(KV + (int64_t)src[u] * 2 * D + lane * E, k[u]);
-        load_slice<T, E>(KV + (int64_t)src[u] * 2 * D + D + lane * E, v[u]);
+      for (int u = 0; u < kBatch; ++u) {
+        const int64_t src = __shfl_sync(kAll, win.col, b + u);
+        w[u] = (float)__shfl_sync(kAll, win.cnt, b + u);
+        if (u < nb) {
+          k[u].load(KV + src * 2 * D);
+          v[u].load(KV + src * 2 * D + D);
+        }
       }
-    }
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      if (src[u] < 0) break;
-      float s = 0.f, da = 0.f;
+      for (int u = 0; u < kBatch; ++u) {
+        if (u >= nb) break;
+        float kf[E], vf[E], s = 0.f, da = 0.f;
+        k[u].get(kf);
+        v[u].get(vf);
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        s = fmaf(k[u][e], q[e], s);
-        da = fmaf(g[e], v[u][e], da);
+        for (int e = 0; e < E; ++e) {
+          s = fmaf(kf[e], q[e], s);
+          da = fmaf(g[e], vf[e], da);
+        }
+        s = head_sum(s, lph);
+        da = head_sum(da, lph);
+        const float alpha = expf(s - m) * inv_l;
+        const float de = w[u] * alpha * (da - Dh);  // the run's w edges
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = fmaf(de, kf[e], acc[e]);
       }
-      s = head_sum(s, lph);
-      da = head_sum(da, lph);
-      const float alpha = expf(s - m) * inv_l;
-      const float de = w[u] * alpha * (da - Dh);  // the run's w edges
-#pragma unroll
-      for (int e = 0; e < E; ++e) acc[e] = fmaf(de, k[u][e], acc[e]);
     }
   }
+}
+
+// Adds the warps' sums of N floats per lane in warp order into warp 0's.
+template <int N>
+__device__ __forceinline__ void add_warps(float (&v)[N], float (*part)[32][N], int nwarps) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int e = 0; e < N; ++e) part[warp][lane][e] = v[e];
+  __syncthreads();
+  if (warp == 0)
+    for (int w = 1; w < nwarps; ++w)
+#pragma unroll
+      for (int e = 0; e < N; ++e) v[e] += part[w][lane][e];
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) hgt_bwd_dst_chunks(HgtArgs a) {
+__global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_dst_chunks(HgtArgs a) {
   constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31, lph = 32 / a.S, h = lane / lph;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  __shared__ float part[kChunkWarps][32][E];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S, h = lane / lph;
   const int nchunks = a.dchunk_ofs[a.csr_rows];
-  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nchunks; c += nw) {
+  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int row = a.dchunk_row[c];
-    const int64_t beg = (int64_t)a.dptr[row] + (int64_t)(c - a.dchunk_ofs[row]) * kChunkEdges;
-    const int64_t end = min((int64_t)a.dptr[row + 1], beg + kChunkEdges);
+    const int64_t cb = (int64_t)a.dptr[row] + (int64_t)(c - a.dchunk_ofs[row]) * kChunkEdges;
+    const int64_t ce = min((int64_t)a.dptr[row + 1], cb + kChunkEdges);
+    const int64_t beg = cb + warp * kChunkPart, end = min(ce, beg + kChunkPart);
     const int64_t mr = a.mrow[row];
     const float4 st = a.rstat[mr * a.S + h];
     float q[E], g[E], acc[E];
@@ -490,163 +689,224 @@ __global__ void __launch_bounds__(256) hgt_bwd_dst_chunks(HgtArgs a) {
     load_slice<T, E>((const T*)a.dS + mr * D + lane * E, g);
 #pragma unroll
     for (int e = 0; e < E; ++e) acc[e] = 0.f;
-    dst_edges<T, D, kBatchChunk>(a, beg, end, q, g, st.x, st.y, st.z, lph, acc);
+    RunWindow win;
+    win.load(a.dcol, a.dcnt, beg, end);
+    dst_edges<T, D>(a, beg, end, win, q, g, st.x, st.y, st.z, lph, acc);
+    add_warps<E>(acc, part, kChunkWarps);
+    if (warp == 0)
 #pragma unroll
-    for (int e = 0; e < E; ++e) a.part[c * D + lane * E + e] = acc[e];
+      for (int e = 0; e < E; ++e) a.part[(int64_t)c * D + lane * E + e] = acc[e];
+    __syncthreads();
   }
 }
 
-// dQ'_r(j) for every relation row of node j (hub rows: their chunk partials in order); the row
-// bounds, query and gradient slices of all of j's rows are loaded before any edge.
-template <typename T, int D, int KS>
-__global__ void __launch_bounds__(256, (D <= 128 && KS <= 4) ? 3 : 1) hgt_bwd_dst_nodes(HgtArgs a) {
+// acc += the partials [c0, c1) of one row in order, N floats per lane at p + c * stride; kBatch
+// partials are loaded before the first is added.
+template <int N>
+__device__ __forceinline__ void add_parts(const float* __restrict__ p, int64_t stride, int c0, int c1,
+                                          float (&acc)[N]) {
+  for (int c = c0; c < c1; c += kBatch) {
+    float v[kBatch][N];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u)
+      if (c + u < c1)
+#pragma unroll
+        for (int e = 0; e < N; ++e) v[u][e] = p[(int64_t)(c + u) * stride + e];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u)
+      if (c + u < c1)
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc[e] += v[u][e];
+  }
+}
+
+// dQ'_r(j) for every stored row (hub rows: their chunk partials in order).  A warp claims kRowClaim
+// compact rows; the next row's slices, statistics and first window load while a row is summed.
+constexpr int kRowClaim = 8;
+template <typename T, int D>
+__global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_dst_rows(HgtArgs a) {
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S, h = lane / lph;
-  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= a.N) return;
-  const int t = node_type_of(a.meta, j);
-  const int64_t jl = j - a.meta.type_off[t];
-  int64_t row[KS];
-  int c0[KS], c1[KS];
-  int64_t e0[KS], e1[KS];
-  float q[KS][E], g[KS][E];
-#pragma unroll
-  for (int k = 0; k < KS; ++k) {
-    const int r = a.rslot[t][k];
-    row[k] = -1;  // compact row
-    if (r < 0) continue;
-    const int64_t cr = a.meta.row_base[r] + jl;
-    const int64_t mr = a.mrow[cr];
-    if (mr < a.csr_rows) {
-      row[k] = mr;
-      c0[k] = a.dchunk_ofs[cr];
-      c1[k] = a.dchunk_ofs[cr + 1];
-      e0[k] = a.dptr[cr];
-      e1[k] = a.dptr[cr + 1];
-      load_slice<T, E>((const T*)a.Qp + mr * D + lane * E, q[k]);
-      load_slice<T, E>((const T*)a.dS + mr * D + lane * E, g[k]);
+  const int64_t total = *a.mcount;
+  for (int64_t x0 = claim(a.work + 1, kRowClaim); x0 < total; x0 = claim(a.work + 1, kRowClaim)) {
+    const int nn = (int)min((int64_t)kRowClaim, total - x0);
+    int eb = 0, ee = 0, cb = 0, ce = 0;
+    if (lane < nn) {
+      const int64_t cr = a.mlist[x0 + lane];
+      eb = a.dptr[cr];
+      ee = a.dptr[cr + 1];
+      cb = a.dchunk_ofs[cr];
+      ce = a.dchunk_ofs[cr + 1];
     }
-  }
-  float4 st = make_float4(0.f, 0.f, 0.f, 0.f);  // the same on each of the node's rows
+    RawSlice<T, E> q, g, qn, gn;
+    float4 st, stn;
+    RunWindow win, wn;
+    auto fetch = [&](int i) {
+      const int64_t mr = x0 + i;
+      qn.load((const T*)a.Qp + mr * D + lane * E);
+      gn.load((const T*)a.dS + mr * D + lane * E);
+      stn = __ldg(a.rstat + mr * a.S + h);
+      wn.load(a.dcol, a.dcnt, __shfl_sync(kAll, eb, i), __shfl_sync(kAll, ee, i));
+    };
+    fetch(0);
+    for (int i = 0; i < nn; ++i) {
+      q = qn;
+      g = gn;
+      st = stn;
+      win = wn;
+      if (i + 1 < nn) fetch(i + 1);
+      const int c0 = __shfl_sync(kAll, cb, i), c1 = __shfl_sync(kAll, ce, i);
+      const int b = __shfl_sync(kAll, eb, i), e1 = __shfl_sync(kAll, ee, i);
+      float acc[E];
 #pragma unroll
-  for (int k = KS - 1; k >= 0; --k)
-    if (row[k] >= 0) st = a.rstat[row[k] * a.S + h];
-#pragma unroll
-  for (int k = 0; k < KS; ++k) {
-    if (row[k] < 0) continue;
-    float acc[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = 0.f;
-    if (c1[k] > c0[k]) {
-      for (int c = c0[k]; c < c1[k]; ++c)
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] += a.part[(int64_t)c * D + lane * E + e];
-    } else {
-      dst_edges<T, D>(a, e0[k], e1[k], q[k], g[k], st.x, st.y, st.z, lph, acc);
+      for (int e = 0; e < E; ++e) acc[e] = 0.f;
+      if (c1 > c0) {
+        add_parts<E>(a.part + lane * E, D, c0, c1, acc);
+      } else {
+        float qf[E], gf[E];
+        q.get(qf);
+        g.get(gf);
+        dst_edges<T, D>(a, b, e1, win, qf, gf, st.x, st.y, st.z, lph, acc);
+      }
+      store_slice<T, E>((T*)a.dQp + (x0 + i) * D + lane * E, acc);
     }
-    store_slice<T, E>((T*)a.dQp + row[k] * D + lane * E, acc);
   }
 }
 
-// Out-edges [beg, end) of source i (node-major list; each entry is the compact row of the edge's
-// target): dK(i) += de Q'_r(j), dV(i) += alpha dS_r(j).
-template <typename T, int D, int NB = kBatch>
-__device__ __forceinline__ void src_edges(const HgtArgs& a, int64_t beg, int64_t end, const float (&k)[D / 32],
-                                          const float (&v)[D / 32], int lph, float (&ak)[D / 32],
-                                          float (&av)[D / 32]) {
+// Out-runs [beg, end) of source i (node-major list; each entry is the compact row of the edge's
+// target): dK(i) += de Q'_r(j) in acc[0 .. E), dV(i) += alpha dS_r(j) in acc[E .. 2 E).
+template <typename T, int D>
+__device__ __forceinline__ void src_edges(const HgtArgs& a, int64_t beg, int64_t end, RunWindow win,
+                                          const float (&k)[D / 32], const float (&v)[D / 32], int lph,
+                                          float (&acc)[D / 16]) {
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, h = lane / lph;
-  for (int64_t e0 = beg; e0 < end; e0 += NB) {
-    int row[NB];
-    float w[NB];
+  const T* Qp = (const T*)a.Qp + lane * E;
+  const T* dS = (const T*)a.dS + lane * E;
+  for (int64_t w0 = beg; w0 < end; w0 += 32) {
+    if (w0 > beg) win.load(a.scol, a.scnt, w0, end);
+    const int n = (int)min((int64_t)32, end - w0);
+    for (int b = 0; b < n; b += kBatch) {
+      const int nb = min(kBatch, n - b);
+      RawSlice<T, E> q[kBatch], g[kBatch];
+      float4 st[kBatch];
+      float w[kBatch];
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      row[u] = e0 + u < end ? __ldg(a.scol + e0 + u) : -1;
-      w[u] = e0 + u < end ? (float)__ldg(a.scnt + e0 + u) : 0.f;
-    }
-    float q[NB][E], g[NB][E];
-    float4 st[NB];
-#pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      if (row[u] >= 0) {
-        load_slice<T, E>((const T*)a.Qp + (int64_t)row[u] * D + lane * E, q[u]);
-        load_slice<T, E>((const T*)a.dS + (int64_t)row[u] * D + lane * E, g[u]);
-        st[u] = a.rstat[(int64_t)row[u] * a.S + h];
+      for (int u = 0; u < kBatch; ++u) {
+        const int64_t row = __shfl_sync(kAll, win.col, b + u);
+        w[u] = (float)__shfl_sync(kAll, win.cnt, b + u);
+        if (u < nb) {
+          q[u].load(Qp + row * D);
+          g[u].load(dS + row * D);
+          st[u] = __ldg(a.rstat + row * a.S + h);
+        }
       }
-    }
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      if (row[u] < 0) break;
-      float s = 0.f, da = 0.f;
+      for (int u = 0; u < kBatch; ++u) {
+        if (u >= nb) break;
+        float qf[E], gf[E], s = 0.f, da = 0.f;
+        q[u].get(qf);
+        g[u].get(gf);
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        s = fmaf(k[e], q[u][e], s);
-        da = fmaf(g[u][e], v[e], da);
-      }
-      s = head_sum(s, lph);
-      da = head_sum(da, lph);
-      const float alpha = w[u] * expf(s - st[u].x) * st[u].y;  // the run's w edges
-      const float de = alpha * (da - st[u].z);
+        for (int e = 0; e < E; ++e) {
+          s = fmaf(k[e], qf[e], s);
+          da = fmaf(gf[e], v[e], da);
+        }
+        s = head_sum(s, lph);
+        da = head_sum(da, lph);
+        const float alpha = w[u] * expf(s - st[u].x) * st[u].y;  // the run's w edges
+        const float de = alpha * (da - st[u].z);
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        ak[e] = fmaf(de, q[u][e], ak[e]);
-        av[e] = fmaf(alpha, g[u][e], av[e]);
+        for (int e = 0; e < E; ++e) {
+          acc[e] = fmaf(de, qf[e], acc[e]);
+          acc[E + e] = fmaf(alpha, gf[e], acc[E + e]);
+        }
       }
     }
   }
 }
 
+// Partials of the source pass: lane-major, 2 E floats per lane (dK then dV).
 template <typename T, int D>
-__global__ void __launch_bounds__(256) hgt_bwd_src_chunks(HgtArgs a) {
+__global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_src_chunks(HgtArgs a) {
   constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31, lph = 32 / a.S;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  __shared__ float part[kChunkWarps][32][2 * E];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S;
   const int nchunks = a.schunk_ofs[a.N];
   const T* KV = (const T*)a.KV;
-  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nchunks; c += nw) {
+  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int i = a.schunk_row[c];
-    const int64_t beg = (int64_t)a.sptr[i] + (int64_t)(c - a.schunk_ofs[i]) * kChunkEdges;
-    const int64_t end = min((int64_t)a.sptr[i + 1], beg + kChunkEdges);
-    float k[E], v[E], ak[E], av[E];
+    const int64_t cb = (int64_t)a.sptr[i] + (int64_t)(c - a.schunk_ofs[i]) * kChunkEdges;
+    const int64_t ce = min((int64_t)a.sptr[i + 1], cb + kChunkEdges);
+    const int64_t beg = cb + warp * kChunkPart, end = min(ce, beg + kChunkPart);
+    float k[E], v[E], acc[2 * E];
     load_slice<T, E>(KV + (int64_t)i * 2 * D + lane * E, k);
     load_slice<T, E>(KV + (int64_t)i * 2 * D + D + lane * E, v);
 #pragma unroll
-    for (int e = 0; e < E; ++e) ak[e] = av[e] = 0.f;
-    src_edges<T, D, kBatchChunk>(a, beg, end, k, v, lph, ak, av);
+    for (int e = 0; e < 2 * E; ++e) acc[e] = 0.f;
+    RunWindow win;
+    win.load(a.scol, a.scnt, beg, end);
+    src_edges<T, D>(a, beg, end, win, k, v, lph, acc);
+    add_warps<2 * E>(acc, part, kChunkWarps);
+    if (warp == 0)
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      a.part[c * 2 * D + lane * E + e] = ak[e];
-      a.part[c * 2 * D + D + lane * E + e] = av[e];
-    }
+      for (int e = 0; e < 2 * E; ++e) a.part[((int64_t)c * 32 + lane) * 2 * E + e] = acc[e];
+    __syncthreads();
   }
 }
 
+// dK(i), dV(i) of every node (zeros without out-edges); claims and prefetch as in hgt_bwd_dst_rows.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) hgt_bwd_src_nodes(HgtArgs a) {
+__global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_src_nodes(HgtArgs a) {
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
-  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= a.N) return;
-  float ak[E], av[E];
+  const T* KV = (const T*)a.KV;
+  for (int64_t x0 = claim(a.work + 2, kRowClaim); x0 < a.N; x0 = claim(a.work + 2, kRowClaim)) {
+    const int nn = (int)min((int64_t)kRowClaim, a.N - x0);
+    int eb = 0, ee = 0, cb = 0, ce = 0;
+    if (lane < nn) {
+      eb = a.sptr[x0 + lane];
+      ee = a.sptr[x0 + lane + 1];
+      cb = a.schunk_ofs[x0 + lane];
+      ce = a.schunk_ofs[x0 + lane + 1];
+    }
+    RawSlice<T, E> k, v, kn, vn;
+    RunWindow win, wn;
+    auto fetch = [&](int i) {
+      const int b = __shfl_sync(kAll, eb, i), e = __shfl_sync(kAll, ee, i);
+      if (b == e) return;
+      kn.load(KV + (x0 + i) * 2 * D + lane * E);
+      vn.load(KV + (x0 + i) * 2 * D + D + lane * E);
+      wn.load(a.scol, a.scnt, b, e);
+    };
+    fetch(0);
+    for (int i = 0; i < nn; ++i) {
+      k = kn;
+      v = vn;
+      win = wn;
+      if (i + 1 < nn) fetch(i + 1);
+      const int c0 = __shfl_sync(kAll, cb, i), c1 = __shfl_sync(kAll, ce, i);
+      const int b = __shfl_sync(kAll, eb, i), e1 = __shfl_sync(kAll, ee, i);
+      float acc[2 * E];
 #pragma unroll
-  for (int e = 0; e < E; ++e) ak[e] = av[e] = 0.f;
-  const int c0 = a.schunk_ofs[i], c1 = a.schunk_ofs[i + 1];
-  if (c1 > c0) {
-    for (int c = c0; c < c1; ++c)
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        ak[e] += a.part[(int64_t)c * 2 * D + lane * E + e];
-        av[e] += a.part[(int64_t)c * 2 * D + D + lane * E + e];
+      for (int e = 0; e < 2 * E; ++e) acc[e] = 0.f;
+      if (c1 > c0) {
+        add_parts<2 * E>(a.part + lane * 2 * E, 2 * D, c0, c1, acc);
+      } else if (e1 > b) {
+        float kf[E], vf[E];
+        k.get(kf);
+        v.get(vf);
+        src_edges<T, D>(a, b, e1, win, kf, vf, lph, acc);
       }
-  } else {
-    float k[E], v[E];
-    const T* KV = (const T*)a.KV;
-    load_slice<T, E>(KV + i * 2 * D + lane * E, k);
-    load_slice<T, E>(KV + i * 2 * D + D + lane * E, v);
-    src_edges<T, D>(a, a.sptr[i], a.sptr[i + 1], k, v, lph, ak, av);
+      float o[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) o[e] = acc[e];
+      store_slice<T, E>((T*)a.dK + (x0 + i) * D + lane * E, o);
+#pragma unroll
+      for (int e = 0; e < E; ++e) o[e] = acc[E + e];
+      store_slice<T, E>((T*)a.dV + (x0 + i) * D + lane * E, o);
+    }
   }
-  store_slice<T, E>((T*)a.dK + i * D + lane * E, ak);
-  store_slice<T, E>((T*)a.dV + i * D + lane * E, av);
 }
 
 // dW_msg[r][s] = the diagonal blocks of the dense gradient G[r] (d x d); dW_att[r][s] = c_r times the
@@ -791,6 +1051,11 @@ HgtArgs edge_args(const hg_graph* g, const hg_hgt_params* p, const HgtLayout& H)
   a.schunk_ofs = g->bagg_chunk_ofs;
   a.schunk_row = g->bagg_chunk_row;
   a.mrow = g->mrow;
+  a.mlist = g->mlist;
+  a.mcount = g->mbase + g->meta.num_rels;
+  a.nperm = g->nperm;
+  a.nzero = g->nzero;
+  a.work = H.L.work;
   a.KV = H.KV;
   a.Qp = H.Qp;
   a.Srows = H.L.M;
@@ -816,7 +1081,11 @@ int max_rels_per_type(const GraphMeta& m) {
 }
 
 unsigned grid_of(int64_t threads) { return (unsigned)std::max<int64_t>(1, ceil_div(threads, 256)); }
-unsigned chunk_blocks(int64_t cap) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(cap, 8), 152 * 16)); }
+unsigned chunk_blocks(int64_t cap) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(cap, 152 * 8)); }
+// CTAs of a claiming kernel over at most n items: what the SMs hold, or fewer for few items
+unsigned claim_blocks(int64_t n) {
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, kRowClaim * kEdgeWarps), 152 * 6));
+}
 
 template <typename T, int D>
 hg_status gemm(const void* A, int64_t lda, const void* B, const void* bias, int K, int64_t n, void* out, int64_t ldo,
@@ -894,11 +1163,14 @@ hg_status hgt_fwd_t(const hg_graph* g, const hg_hgt_params* p, const void* H_in,
   }
   // Eq. 6-10: softmax over the in-edges, weighted value sums per relation row
   const HgtArgs a = edge_args(g, p, H);
-  HG_TRY(launch("hgt_fwd_chunks", hgt_fwd_chunks<T, D>, dim3(chunk_blocks(g->chunk_cap_csr)), dim3(256), 0, s, a));
+  HG_TRY(launch("hgt_fwd_chunks", hgt_fwd_chunks<T, D>, dim3(chunk_blocks(g->chunk_cap_csr)), dim3(32 * kChunkWarps), 0,
+                s, a));
+  HG_CUDA(cudaMemsetAsync(a.work, 0, 3 * sizeof(int32_t), s));
+  const dim3 cb(32 * kEdgeWarps);
   if (max_rels_per_type(m) <= 4)
-    HG_TRY(launch("hgt_fwd_nodes", hgt_fwd_nodes<T, D, 4>, dim3(grid_of(N * 32)), dim3(256), 0, s, a));
+    HG_TRY(launch("hgt_fwd_nodes", hgt_fwd_nodes<T, D, 4>, dim3(claim_blocks(N)), cb, 0, s, a));
   else
-    HG_TRY(launch("hgt_fwd_nodes", hgt_fwd_nodes<T, D, kMaxRels>, dim3(grid_of(N * 32)), dim3(256), 0, s, a));
+    HG_TRY(launch("hgt_fwd_nodes", hgt_fwd_nodes<T, D, kMaxRels>, dim3(claim_blocks(N)), cb, 0, s, a));
   // Eq. 11 on S_r with W_rel = blockdiag(W_msg[r])
   const hg_layer_params lp = projection_params(p, H);
   return project_forward(g, &lp, H_in, H_out, H.L, s);
@@ -925,17 +1197,13 @@ hg_status hgt_bwd_t(const hg_graph* g, const hg_hgt_params* p, const void* H_in,
   HG_TRY(project_backward(g, &lp, H_in, dH_out, &lg, H.L, false, s));
   // attention backward: target pass (dQ'), source pass (dK, dV)
   const HgtArgs a = edge_args(g, p, H);
-  HG_TRY(launch("hgt_bwd_dstats", hgt_bwd_dstats<T, D>, dim3(grid_of(N * 32)), dim3(256), 0, s, a));
-  HG_TRY(launch("hgt_bwd_dst_chunks", hgt_bwd_dst_chunks<T, D>, dim3(chunk_blocks(g->chunk_cap_csr)), dim3(256), 0, s,
-                a));
-  if (max_rels_per_type(m) <= 4)
-    HG_TRY(launch("hgt_bwd_dst_nodes", hgt_bwd_dst_nodes<T, D, 4>, dim3(grid_of(N * 32)), dim3(256), 0, s, a));
-  else
-    HG_TRY(launch("hgt_bwd_dst_nodes", hgt_bwd_dst_nodes<T, D, kMaxRels>, dim3(grid_of(N * 32)), dim3(256), 0, s,
-                  a));
-  HG_TRY(launch("hgt_bwd_src_chunks", hgt_bwd_src_chunks<T, D>, dim3(chunk_blocks(g->chunk_cap_node)), dim3(256), 0,
-                s, a));
-  HG_TRY(launch("hgt_bwd_src_nodes", hgt_bwd_src_nodes<T, D>, dim3(grid_of(N * 32)), dim3(256), 0, s, a));
+  const dim3 cb(32 * kEdgeWarps), hb(32 * kChunkWarps);
+  HG_CUDA(cudaMemsetAsync(a.work, 0, 3 * sizeof(int32_t), s));
+  HG_TRY(launch("hgt_bwd_dstats", hgt_bwd_dstats<T, D>, dim3(std::min(grid_of(N * 32), 152u * 16)), dim3(256), 0, s, a));
+  HG_TRY(launch("hgt_bwd_dst_chunks", hgt_bwd_dst_chunks<T, D>, dim3(chunk_blocks(g->chunk_cap_csr)), hb, 0, s, a));
+  HG_TRY(launch("hgt_bwd_dst_rows", hgt_bwd_dst_rows<T, D>, dim3(claim_blocks(g->csr_rows)), cb, 0, s, a));
+  HG_TRY(launch("hgt_bwd_src_chunks", hgt_bwd_src_chunks<T, D>, dim3(chunk_blocks(g->chunk_cap_node)), hb, 0, s, a));
+  HG_TRY(launch("hgt_bwd_src_nodes", hgt_bwd_src_nodes<T, D>, dim3(claim_blocks(N)), cb, 0, s, a));
   // weights of the backward products (exact copies and transposes)
   HG_TRY(launch("hgt_blockdiag", hgt_blockdiag<T>, dim3(grid_of((int64_t)m.num_rels * dd)), dim3(256), 0, s,
                 (const T*)p->W_att, m.num_rels, D, S, 0, (T*)H.BDatt));
