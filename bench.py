@@ -239,7 +239,7 @@ class Clocks:
 # ------------------------------------------------------------------------------------------------
 # algorithmic bytes / flops per step for each kernel (from the graph's own statistics)
 # ------------------------------------------------------------------------------------------------
-HUB, CHUNK = 512, 512
+HUB, CHUNK = 96, 512
 FUSE = 32  # the fused mean layer streams rows of at most this many runs in its projection
 
 

@@ -17,10 +17,15 @@ namespace hg {
 constexpr int kMaxTypes = 4;
 constexpr int kMaxRels = 8;
 constexpr int kProjTileRows = 128;  // output rows per tile of the tensor-core forward projection
-// A CSR/CSC row with more than kHubDegree edges is split into chunks of kChunkEdges edges; each
+// A row with more than kHubDegree runs is split into chunks of kChunkEdges runs, a CTA per chunk; each
 // chunk's fp32 partial sum goes to scratch and the row is finished by adding the chunk partials
-// in chunk order, so the reduction order is fixed (deterministic, atomic-free).
-constexpr int kHubDegree = 512;
+// in chunk order, so the reduction order is fixed.  The degree is a balance: a longer row would hold
+// one warp (about 0.6 us per eight runs, which is the whole kernel's time on a small graph), a shorter
+// one does not fill a CTA and its partial costs more than its gathers.  Layer forward + backward at
+// 512 / 128 / 96 / 64 / 40: 100k nodes fp32 854 / 726 / 717 / 696 / 684 us, 1M-node step 5.89 / 5.47 / 5.50 /
+// 5.43 / 5.44 ms, 10M nodes 11.21 / 10.99 / 11.09 / 11.17 / 11.41 ms; 2M nodes forward 3.05 / 2.65 / 2.67 / 2.69 /
+// 2.92 ms.  Chunks of 128, 256 and 1024 runs were slower on the large graphs (12.30, 11.42, 11.32 ms).
+constexpr int kHubDegree = 96;
 constexpr int kChunkEdges = 512;
 // The fused mean layer (gathers into the projection's operand tiles) sums a CSR row in the
 // projection only up to kFuseRuns runs; the means of longer rows are computed beforehand by the

@@ -3,7 +3,7 @@
 The aggregation models split every layer's work between the row kernels and the hub-chunk kernels
 exactly as the library does: forward rows are the CSR rows of each (relation, destination),
 backward rows are node-major (a node's out-edges of every relation), parallel edges of a node pair
-are one run with their multiplicity, and a row above 512 runs goes through 512-run chunks.  Here
+are one run with their multiplicity, and a row above 96 runs goes through 512-run chunks.  Here
 those rows are rebuilt from the oracle's CSR / CSC, and the roofline figures are recomputed by hand
 from a fake timing report."""
 import numpy as np

@@ -2,7 +2,7 @@
 summed inside the projection and never stored, and summed again for the weight gradient.  Its
 results must equal the unfused layer's bit for bit (the same sums in the same order) and the plain
 definition (Eq. 7, 10, 11 in fp64) within the bf16 tolerance, on graphs whose rows span every path:
-no in-edges, short rows, rows above 32 runs and hub rows above 512 runs."""
+no in-edges, short rows, rows above 32 runs and hub rows above 96 runs."""
 import numpy as np
 import pytest
 import torch
