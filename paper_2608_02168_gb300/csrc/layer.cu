@@ -279,6 +279,7 @@ hg_status project_forward(const hg_graph* graph, const hg_layer_params* p, const
       a.msent = graph->csr_rows;
       a.perm = graph->nperm + m.type_off[t];
       a.tmask = graph->tmask + graph->tile_base[t];
+      a.nzero = graph->nzero + t;
       a.b = (const __nv_bfloat16*)p->b_agg + (size_t)t * d;
       a.gamma = p->layernorm ? (const __nv_bfloat16*)p->ln_gamma + (size_t)t * d : nullptr;
       a.beta = p->layernorm ? (const __nv_bfloat16*)p->ln_beta + (size_t)t * d : nullptr;

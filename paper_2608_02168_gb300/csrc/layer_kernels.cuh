@@ -56,11 +56,12 @@ struct TcFwdArgs {
   int nrel;
   int rel[kMaxRels];          // relation ids into this type (row block of W_rel^T)
   int64_t mrow0[kMaxRels];    // first CSR row of each
-  const int32_t* mrow;        // row of M holding each CSR row (>= msent: an empty row, read as zeros);
-  int64_t msent;              // null: M is indexed by CSR row.  msent = the row extent of M
+  const int32_t* mrow;        // row of M holding each CSR row (>= msent: an empty row, read as zeros)
+  int64_t msent;              // the row extent of M
   const __nv_bfloat16* M;     // relation means, [msent][D]
-  const int32_t* perm;        // tile position -> local node (the type's nodes by relation mask); null: identity
-  const int32_t* tmask;       // per tile, the relations (bit k = rel[k]) with a stored row in it; null: all
+  const int32_t* perm;        // tile position -> local node (the type's nodes by relation mask)
+  const int32_t* tmask;       // per tile, the relations (bit k = rel[k]) with a stored row in it
+  const int32_t* nzero;       // device: first positions of perm whose nodes have no in-edge
   // the fused mean layer (M unused): the means are summed from H_in over the CSR runs in the
   // projection; rows above kFuseRuns runs read theirs from Mlong at slot long_ofs[row]
   const int32_t* agg_ptr;

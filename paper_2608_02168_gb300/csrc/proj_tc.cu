@@ -117,6 +117,100 @@ template <int D>
 __global__ void __launch_bounds__(FwdCfg<D, true>::kThreads, 1)
     proj_fwd_gather_tc(const __grid_constant__ CUtensorMap tm_Vt, TcFwdArgs a);
 
+// Positions of the node order, from the start, whose nodes have no in-edge under any relation, in
+// whole tiles (a tile that mixes them with others belongs to the projection).
+__device__ __forceinline__ int64_t idle_rows(const int32_t* nzero) {
+  return (int64_t)__ldg(nzero) / kTileRows * kTileRows;
+}
+
+// a lane's E consecutive bf16 of a row as one word or vector
+template <int E>
+using RawBf16 = typename std::conditional<E == 2, uint32_t, typename std::conditional<E == 4, uint2, uint4>::type>::type;
+template <int E>
+__device__ __forceinline__ void unpack_raw(const RawBf16<E>& w, float* v) {
+  if constexpr (E == 2) {
+    v[0] = __uint_as_float(w << 16);
+    v[1] = __uint_as_float(w & 0xFFFF0000u);
+  } else if constexpr (E == 4) {
+    v[0] = __uint_as_float(w.x << 16);
+    v[1] = __uint_as_float(w.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(w.y << 16);
+    v[3] = __uint_as_float(w.y & 0xFFFF0000u);
+  } else {
+    unpack(w, v, __nv_bfloat16());
+  }
+}
+template <int E>
+__device__ __forceinline__ void store_raw(__nv_bfloat16* p, const float* v) {
+  if constexpr (E == 2) {
+    *reinterpret_cast<uint32_t*>(p) = pack_bf16x2(v[0], v[1]);
+  } else if constexpr (E == 4) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]));
+  } else {
+    st16(p, pack(v, __nv_bfloat16()));
+  }
+}
+
+// The forward projection of the idle rows: no message, so U = 0 and H_out = LN(act(b) + H_in).  Warp
+// per row, kIdleRows rows in flight, the nodes of the next ones loaded a round ahead.  Bound by HBM
+// (one row in, two out), which the projection's eight epilogue warps per SM did not reach on these
+// rows.  10M nodes, 200M edges (most nodes without in-edges), d = 128: the projection 2.69 ms before,
+// now 1.23 + 0.80 ms.  (Leaving their U out of memory and skipping it in the backward was slower: the scattered
+// 256-byte accesses cost ln_act_bwd more than the saved bytes, 2.32 -> 2.67 ms.)
+constexpr int kIdleRows = 4;
+template <int D>
+__global__ void __launch_bounds__(256) proj_fwd_idle(TcFwdArgs a) {
+  constexpr int E = D / 32;
+  const int lane = threadIdx.x & 31, c0 = lane * E;
+  const int64_t n = idle_rows(a.nzero);
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x / 32) * kIdleRows;
+  float ab[E], g[E], be[E];
+#pragma unroll
+  for (int i = 0; i < E; ++i) {
+    ab[i] = act_apply(__bfloat162float(a.b[c0 + i]), a.act);
+    g[i] = a.ln ? __bfloat162float(a.gamma[c0 + i]) : 1.f;
+    be[i] = a.ln ? __bfloat162float(a.beta[c0 + i]) : 0.f;
+  }
+  int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kIdleRows;  // n is a multiple of kIdleRows
+  int jn = lane < kIdleRows && p < n ? __ldg(a.perm + p + lane) : 0;
+  for (; p < n; p += step) {
+    int64_t j[kIdleRows];
+    RawBf16<E> rh[kIdleRows];
+#pragma unroll
+    for (int k = 0; k < kIdleRows; ++k) {
+      j[k] = a.off + __shfl_sync(0xffffffffu, jn, k);
+      rh[k] = *reinterpret_cast<const RawBf16<E>*>(a.H_in + j[k] * D + c0);
+    }
+    jn = lane < kIdleRows && p + step < n ? __ldg(a.perm + p + step + lane) : 0;
+#pragma unroll
+    for (int k = 0; k < kIdleRows; ++k) {
+      float y[E], sum = 0.f;
+      unpack_raw<E>(rh[k], y);
+#pragma unroll
+      for (int i = 0; i < E; ++i) {
+        y[i] += ab[i];
+        sum += y[i];
+      }
+      if (a.ln) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const float mean = sum * (1.f / D);
+        float qq = 0.f;
+#pragma unroll
+        for (int i = 0; i < E; ++i) qq += (y[i] - mean) * (y[i] - mean);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) qq += __shfl_xor_sync(0xffffffffu, qq, o);
+        const float rstd = rsqrtf(qq * (1.f / D) + a.eps);
+#pragma unroll
+        for (int i = 0; i < E; ++i) y[i] = (y[i] - mean) * rstd * g[i] + be[i];
+        if (lane == 0) a.stats[j[k]] = make_float2(mean, rstd);
+      }
+      store_raw<E>(a.H_out + j[k] * D + c0, y);
+      *reinterpret_cast<RawBf16<E>*>(a.U + j[k] * D + c0) = RawBf16<E>{};
+    }
+  }
+}
+
 template <int D, bool kGather>
 __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const TcFwdArgs& a) {
   using C = FwdCfg<D, kGather>;
@@ -139,16 +233,18 @@ __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const Tc
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t ntiles = (a.n + kTileRows - 1) / kTileRows;
   const int64_t G = gridDim.x;
+  // the tiles of nodes without any in-edge, first in the order, are proj_fwd_idle's
+  const int64_t tile0 = idle_rows(a.nzero) / kTileRows + blockIdx.x;
   const uint32_t all = (1u << a.nrel) - 1u;
   // the relations whose products tile q computes (a relation without a stored row in it is skipped)
   auto rels_of = [&](int64_t q) -> uint32_t {
     if (q >= ntiles) return 0u;
-    return a.tmask ? (uint32_t)__ldg(a.tmask + q) & all : all;
+    return (uint32_t)__ldg(a.tmask + q) & all;
   };
   // local node at position m of the order; -1 past the type
   auto node_at = [&](int64_t m) -> int64_t {
     if (m >= a.n) return -1;
-    return a.perm ? (int64_t)__ldg(a.perm + m) : m;
+    return (int64_t)__ldg(a.perm + m);
   };
   __shared__ int64_t s_row0[kMaxRels];  // gather variant: first CSR row and id of each relation into the type
   __shared__ int s_rel[kMaxRels];
@@ -212,7 +308,7 @@ __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const Tc
       // The relation tiles of this CTA (warp-uniform): tiles blockIdx.x, + G, ..., each with the
       // relations of its mask in ascending order (the MMA warp's order).  Lane k holds the mask of
       // tile wb + G k of a window of 32 tiles.
-      int wb = blockIdx.x;
+      int wb = (int)tile0;
       uint32_t wmask = rels_of(wb + G * lane);
       unsigned wnz = __ballot_sync(0xffffffffu, wmask != 0u);
       int wnext = 0;
@@ -426,11 +522,11 @@ __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const Tc
         for (int h = 0; h < 2; ++h) {
           int64_t x = -1;
           if (((tm >> r) & 1u) && j[h] >= 0)
-            x = a.mrow ? (int64_t)__ldg(a.mrow + a.mrow0[r] + j[h]) : a.mrow0[r] + j[h];
+            x = (int64_t)__ldg(a.mrow + a.mrow0[r] + j[h]);
           v[r][h] = x >= 0 && x < a.msent ? (int32_t)x : -1;
         }
     };
-    int64_t tile = blockIdx.x;
+    int64_t tile = tile0;
     uint32_t tm_c = rels_of(tile), tm_n = rels_of(tile + G);
     int64_t j_c[2], j_n[2];
     int32_t v_c[kMaxRels][2];
@@ -500,8 +596,8 @@ __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const Tc
       bool ok = true;
       uint32_t g = 0;
       int it = 0;
-      uint32_t tm_n = rels_of(blockIdx.x);
-      for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += G, ++it) {
+      uint32_t tm_n = rels_of(tile0);
+      for (int64_t tile = tile0; tile < ntiles && ok; tile += G, ++it) {
         const uint32_t tm = tm_n;
         tm_n = rels_of(tile + G);  // in flight during this tile
         const int b = it & 1;
@@ -598,11 +694,11 @@ __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const Tc
     };
     bool ok = true;
     int it = 0;
-    int64_t j_c = node_at((int64_t)blockIdx.x * kTileRows + row);  // this tile's node at the row
-    int64_t j_n = node_at(((int64_t)blockIdx.x + G) * kTileRows + row);  // the next tile's
-    bool has_n = rels_of(blockIdx.x) != 0;
+    int64_t j_c = node_at(tile0 * kTileRows + row);  // this tile's node at the row
+    int64_t j_n = node_at((tile0 + G) * kTileRows + row);  // the next tile's
+    bool has_n = rels_of(tile0) != 0;
     fetch_h(j_c, 0);
-    for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += G, ++it) {
+    for (int64_t tile = tile0; tile < ntiles && ok; tile += G, ++it) {
       const int b = it & 1;
       const int64_t j = j_c;
       const bool live = j >= 0;
@@ -939,31 +1035,9 @@ __global__ void __launch_bounds__(256, LnCfg<D>::kBlocks) ln_act_bwd(TcBwdArgs a
   float pdb[E], pdg[E], pdbe[E];
 #pragma unroll
   for (int i = 0; i < E; ++i) pdb[i] = pdg[i] = pdbe[i] = 0.f;
-  auto store = [&](__nv_bfloat16* p, const float* v) {
-    if constexpr (E == 2) {
-      *reinterpret_cast<uint32_t*>(p) = pack_bf16x2(v[0], v[1]);
-    } else if constexpr (E == 4) {
-      *reinterpret_cast<uint2*>(p) = make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]));
-    } else {
-      st16(p, pack(v, __nv_bfloat16()));
-    }
-  };
   // kLnRows rows per iteration: all their loads are in flight before any is computed (held as the
   // raw bf16 words, E / 2 registers per tensor and row)
-  using Raw = typename std::conditional<E == 2, uint32_t, typename std::conditional<E == 4, uint2, uint4>::type>::type;
-  auto unpack_raw = [&](const Raw& w, float* v) {
-    if constexpr (E == 2) {
-      v[0] = __uint_as_float(w << 16);
-      v[1] = __uint_as_float(w & 0xFFFF0000u);
-    } else if constexpr (E == 4) {
-      v[0] = __uint_as_float(w.x << 16);
-      v[1] = __uint_as_float(w.x & 0xFFFF0000u);
-      v[2] = __uint_as_float(w.y << 16);
-      v[3] = __uint_as_float(w.y & 0xFFFF0000u);
-    } else {
-      unpack(w, v, __nv_bfloat16());
-    }
-  };
+  using Raw = RawBf16<E>;
   const int64_t step = (int64_t)gridDim.x * 8;
   for (int64_t row0 = (int64_t)blockIdx.x * 8 + warp; row0 < a.n; row0 += kLnRows * step) {
     Raw rd[kLnRows], ru[kLnRows], rh[kLnRows];
@@ -982,9 +1056,9 @@ __global__ void __launch_bounds__(256, LnCfg<D>::kBlocks) ln_act_bwd(TcBwdArgs a
       const int64_t row = row0 + k * step;
       if (row >= a.n) continue;
       float dv[E], uv[E], hv[E], dy[E], du[E], xh[E];
-      unpack_raw(rd[k], dv);
-      unpack_raw(ru[k], uv);
-      unpack_raw(rh[k], hv);
+      unpack_raw<E>(rd[k], dv);
+      unpack_raw<E>(ru[k], uv);
+      unpack_raw<E>(rh[k], hv);
 #pragma unroll
       for (int i = 0; i < E; ++i) uv[i] += bias[i];
       if (a.ln) {
@@ -1019,8 +1093,8 @@ __global__ void __launch_bounds__(256, LnCfg<D>::kBlocks) ln_act_bwd(TcBwdArgs a
         pdbe[i] += dv[i];
       }
       const int64_t o = (a.off + row) * D + c0;
-      store(a.dY + o, dy);
-      store(a.dU + o, du);
+      store_raw<E>(a.dY + o, dy);
+      store_raw<E>(a.dU + o, du);
     }
   }
 #pragma unroll
@@ -1832,6 +1906,14 @@ static hg_status tc_fuse_t(const void* W_rel, const void* W_agg, RelDst rd, int 
 }
 
 template <int D>
+static hg_status fwd_idle_t(const TcFwdArgs& a, cudaStream_t s) {
+  if (a.n < kTileRows) return HG_OK;  // less than a tile of idle rows
+  const int64_t warps = ceil_div(a.n, kIdleRows);
+  return launch("proj_fwd_idle", proj_fwd_idle<D>, dim3((unsigned)std::min<int64_t>(ceil_div(warps, 8), 152 * 8)),
+                dim3(256), 0, s, a);
+}
+
+template <int D>
 static hg_status tc_fwd_t(const TcFwdArgs& a0, const void* M, int64_t m_rows, const void* Vt, int num_rels,
                           cudaStream_t s) {
   HG_TRY(smem_attr_once<D>());
@@ -1844,6 +1926,7 @@ static hg_status tc_fwd_t(const TcFwdArgs& a0, const void* M, int64_t m_rows, co
   HG_CUDA(cudaGetDevice(&dev));
   HG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(a.n, kTileRows), sms));
+  HG_TRY(fwd_idle_t<D>(a, s));
   return launch("proj_fwd_tc", proj_fwd_tc<D>, dim3(grid), dim3(FwdCfg<D>::kThreads), FwdCfg<D>::kSmem, s, tm_V,
                 a);
 }
@@ -1866,6 +1949,7 @@ static hg_status tc_fwd_gather_t(const TcFwdArgs& a, const void* Vt, int num_rel
     HG_CUDA(cudaGetDevice(&dev));
     HG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(a.n, kTileRows), sms));
+    HG_TRY(fwd_idle_t<D>(a, s));
     return launch("proj_fwd_gather_tc", proj_fwd_gather_tc<D>, dim3(grid), dim3(FwdCfg<D, true>::kThreads),
                   FwdCfg<D, true>::kSmem, s, tm_V, a);
   }

@@ -136,3 +136,28 @@ def test_relu_near_zero_pre_activations_bf16():
     for k in ("W_rel", "W_agg", "b_agg"):
         x, y = host(grads[k]), gref[k]
         assert np.linalg.norm(x - y) / np.linalg.norm(y) <= 2e-2, k
+
+
+@pytest.mark.parametrize("d,ln", [(64, True), (128, False), (128, True), (256, True)])
+@pytest.mark.parametrize("idle", [0, 127, 128, 129, 400])
+def test_nodes_without_in_edges_bf16(d, ln, idle):
+    """`idle` of 400 users and every risk node without in-edges: whole 128-row tiles of them leave the projection."""
+    need_gpu()
+    hg = lib()
+    sp = hgsynth.spec("tiny-10k", n_user=400, n_risk=100, num_edges=6_000, n_overlap=10, dtype="bf16", d=d)
+    w = hgsynth.make_workload(sp, random_affine=True, with_ids=False, bias_margin=BF16_RELU_MARGIN)
+    g, p = w.graph, w.params[0]
+    keep = np.flatnonzero(g["rel"] == 0) if idle < 400 else np.zeros(0, np.int64)  # relation 0: user -> user
+    for k in ("src", "dst", "rel"):
+        g[k] = np.ascontiguousarray(g[k][keep])
+    targets = np.random.default_rng(0).permutation(400)[: 400 - idle]
+    if keep.size:
+        g["dst"] = targets[np.arange(keep.size) % targets.size].astype(g["dst"].dtype)
+    out, dH_in, grads = run_gpu_layer(hg, w, p, "relu", ln, w.dH_top)
+    csr = oracle.build_csr(g["src"], g["dst"], g["rel"], g["type_offsets"], g["rels"])
+    ref, _ = oracle.layer_forward(csr, g["type_offsets"], g["rels"], p, w.X, "relu", ln)
+    dref, gref = oracle.layer_backward(csr, g["type_offsets"], g["rels"], p, w.X, w.dH_top, "relu", ln)
+    assert relerr(host(out), ref) <= TOL["bf16"] and relerr(host(dH_in), dref) <= TOL["bf16"]
+    for k in ("W_rel", "W_agg", "b_agg") + (("ln_gamma", "ln_beta") if ln else ()):
+        assert np.abs(host(grads[k]) - gref[k]).max() <= TOL["bf16"] * np.abs(gref[k]).max(), k
+    assert hg.hg_device_status() == 0
