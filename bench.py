@@ -298,6 +298,10 @@ def graph_stats(w) -> dict:
     for r, (_, tt) in enumerate(g["rels"]):
         st["types"][tt]["nnz"] += st["rels"][r]["nnz"]  # stored relation rows (non-empty CSR rows)
     st["NNZ"] = sum(r["nnz"] for r in st["rels"])
+    has_in = torch.zeros(N, dtype=torch.bool, device=dst.device)
+    has_in[dst] = True
+    for t, ty in enumerate(st["types"]):
+        ty["live"] = nz(has_in[offs[t]:offs[t + 1]])  # nodes with an in-edge
     # backward: one node-major row per node; its runs are the distinct (relation, destination) dMs
     # rows it reads
     read = rel * N + dst
@@ -372,6 +376,15 @@ def kernel_models(st: dict, sp) -> dict:
     # (by source id, then CSR row: (row, source, edge id); that order by CSC row)
     passes = lambda rows: max(1, -(-int(rows).bit_length() // 8))  # noqa: E731
     m["radix_scatter"] = (2 * 12 * st["E"] * (passes(N) + passes(RR) + passes(CC)), 0)
+    # what the kernels as built move where that differs from the terms above (used for rates): the sorts
+    # take digits of up to 9 bits and the third one takes the runs; nodes without in-edges are taken from
+    # the projection by proj_fwd_idle (whole tiles of them: here all)
+    digits = lambda rows: max(1, -(-int(rows).bit_length() // 9))  # noqa: E731
+    runs = f["R_h"] + f["R_nh"]
+    idle = sum(t["n"] - t.get("live", t["n"]) for t in st["types"])
+    m["moved"] = {"radix_scatter": 2 * 12 * (st["E"] * (digits(N) + digits(RR)) + runs * digits(CC)),
+                  "proj_fwd_tc": L * (tf - idle * (3 * row + 8)), "proj_fwd_gather_tc": L * (tf - row * NNZ + fuse_in - idle * (3 * row + 8))}
+    m["proj_fwd_idle"] = (L * idle * (3 * row + 8), 0)
     nl = st.get("n_lab", 0)
     if nl:
         # per labelled row: its H row (and a replica row for overlap rows, not counted), the saved Hm
@@ -482,6 +495,7 @@ def roofline(report: dict, models: dict, steps: int, peaks: dict, src: str, dom=
     dom = dom or max(report, key=lambda k: report[k][1])
     n, ms = report[dom]
     by, fl = models.get(dom, (0, 0))
+    by = models.get("moved", {}).get(dom, by)
     secs = ms / 1e3
     alu_peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12  # fp32 FMA, TFLOP/s
     if dom.endswith("_simt") or dom == "wgrad_partial":  # CUDA-core kernels: fp32 FMA bound

@@ -172,154 +172,198 @@ hg_status exclusive_scan(const int32_t* in, int32_t* out, int64_t n, void* scrat
 }
 
 // ---------------------------------------------------------------------------------------------
-// stable LSD radix sort of (uint32 key, uint32 value) pairs, 8-bit digits
+// stable LSD radix sort of (uint32 key, uint32 value, uint32 second value), digits of up to 9 bits
 // ---------------------------------------------------------------------------------------------
+// A pass is bound by shared memory, not by HBM (random digits meet about 3.4 to a bank, and every item
+// is ranked and placed there), so a pass less is worth more than narrower digits: 24-bit keys take three
+// 8-bit passes and 26-bit keys three of 9, 9 and 8 bits (four before).  Measured on the 10M-node, 200M-edge
+// build (zipf 1.2 / 0.65), against the former tiles of 4096 with a read and a write of the counts per
+// round and 8-bit digits: 23.05 / 31.40 -> 20.65 / 29.12 ms; 1M edges 558 -> 545 us, 20k 343 -> 328 us.
+// Tiles of 4096 (three CTAs on an SM) and 8192 items spill and were slower (19.9, 19.4 ms against 17.8 ms
+// with the runs below), and so were CTAs of 256 threads (19.0 - 21.1 ms).  Graphs whose tiles of 6144
+// do not fill the SMs once take tiles of 2048.
 constexpr int kSortThreads = 512;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 8;                           // per thread
-constexpr int kSortTile = kSortThreads * kSortItems;    // 4096 per block
-constexpr int kWarpSlice = kSortTile / kSortWarps;      // 256 consecutive items per warp
-constexpr int kRadix = 256;
+constexpr int kMaxBits = 9;
+constexpr int kMaxRadix = 1 << kMaxBits;
+static_assert(kMaxRadix <= kSortThreads, "a thread per digit");
+constexpr int kItemsLarge = 12, kItemsSmall = 4;  // per thread
+constexpr int64_t kSortLarge = (int64_t)2 * 152 * kSortThreads * kItemsLarge;
 
-// Per-tile digit counts hist[digit * tiles + tile]; each warp counts into its own shared
-// histogram (atomics only contend within a warp), and the warp histograms are added at the end.
+// Per-tile digit counts hist[digit * tiles + tile]; four warps count into one shared histogram, and
+// the histograms are added at the end.
+// n_dev, if given, holds the item count on the device, at most n; tiles past it count nothing.
+template <int kItems>
 __global__ void __launch_bounds__(kSortThreads) radix_hist(const uint32_t* __restrict__ keys, int64_t n,
-                                                           int shift, int32_t* __restrict__ hist,
-                                                           int64_t tiles) {
-  __shared__ int h[kSortWarps][kRadix];
-  for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kSortThreads) (&h[0][0])[i] = 0;
-  __syncthreads();
-  const int warp = threadIdx.x >> 5;
-  // this thread's 8 consecutive keys, loaded before any of them is counted
-  const int64_t first = (int64_t)blockIdx.x * kSortTile + (int64_t)threadIdx.x * kSortItems;
-  uint32_t k[kSortItems];
-  if (first + kSortItems <= n) {
-    const uint4 a = *reinterpret_cast<const uint4*>(keys + first);
-    const uint4 b = *reinterpret_cast<const uint4*>(keys + first + 4);
-    k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
-    k[4] = b.x; k[5] = b.y; k[6] = b.z; k[7] = b.w;
-  } else {
-#pragma unroll
-    for (int i = 0; i < kSortItems; ++i) k[i] = first + i < n ? keys[first + i] : 0u;
+                                                           const int32_t* __restrict__ n_dev, int shift, int bits,
+                                                           int32_t* __restrict__ hist, int64_t tiles) {
+  constexpr int kTile = kSortThreads * kItems;
+  constexpr int kCopies = 4;  // four warps share a histogram
+  __shared__ int h[kCopies][kMaxRadix];
+  const int radix = 1 << bits;
+  const int64_t t0 = (int64_t)blockIdx.x * kTile;
+  if (n_dev) {
+    n = *n_dev;
+    if (t0 >= n) {
+      for (int d = threadIdx.x; d < radix; d += kSortThreads) hist[(int64_t)d * tiles + blockIdx.x] = 0;
+      return;
+    }
   }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < radix)
 #pragma unroll
-  for (int i = 0; i < kSortItems; ++i)
-    if (first + i < n) atomicAdd(&h[warp][(k[i] >> shift) & (kRadix - 1)], 1);
+    for (int w = 0; w < kCopies; ++w) h[w][threadIdx.x] = 0;
+  // the warp's slice, 128 keys per round (16-byte loads), all loaded before any is counted
+  const int64_t first = t0 + (int64_t)warp * 32 * kItems + lane * 4;
+  uint4 k[kItems / 4];
+#pragma unroll
+  for (int i = 0; i < kItems / 4; ++i) {
+    const int64_t p = first + i * 128;
+    if (p + 4 <= n) {
+      k[i] = *reinterpret_cast<const uint4*>(keys + p);
+    } else {
+      k[i].x = p < n ? keys[p] : 0u;
+      k[i].y = p + 1 < n ? keys[p + 1] : 0u;
+      k[i].z = p + 2 < n ? keys[p + 2] : 0u;
+      k[i].w = 0u;
+    }
+  }
   __syncthreads();
-  if (threadIdx.x < kRadix) {
+#pragma unroll
+  for (int i = 0; i < kItems / 4; ++i) {
+    const int64_t p = first + i * 128;
+    const uint32_t v[4] = {k[i].x, k[i].y, k[i].z, k[i].w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (p + e < n) atomicAdd(&h[warp % kCopies][(v[e] >> shift) & (radix - 1)], 1);
+  }
+  __syncthreads();
+  for (int d = threadIdx.x; d < radix; d += kSortThreads) {
     int t = 0;
 #pragma unroll
-    for (int w = 0; w < kSortWarps; ++w) t += h[w][threadIdx.x];
-    hist[(int64_t)threadIdx.x * tiles + blockIdx.x] = t;
+    for (int w = 0; w < kCopies; ++w) t += h[w][d];
+    hist[(int64_t)d * tiles + blockIdx.x] = t;
   }
 }
 
-// Stable scatter of one 4096-item tile.  (1) Warp w reads its 256 consecutive items, 32 at a time
-// (coalesced), into registers.  (2) It ranks them round by round with __match_any_sync, keeping
-// per-digit running counts, so the item order inside the tile is (warp, round, lane).  (3) Per-digit
-// prefixes over warps and over digits give every item its position in the tile sorted by digit
-// (equal digits keep their order), where it is written in shared memory.  (4) Consecutive threads
-// write consecutive sorted items to base[digit] + (position - tile start of the digit): runs of
-// equal digits go out coalesced.
-template <bool kTwo>
-__global__ void __launch_bounds__(kSortThreads) radix_scatter(
+// Stable scatter of one tile.  (1) Warp w reads the keys of its 32 kItems consecutive items, 32 at a
+// time (coalesced).  (2) It ranks them round by round with __match_any_sync and per-digit running
+// counts, so the item order inside the tile is (warp, round, lane).  (3) Per-digit prefixes over warps
+// and over digits, added into the warps' counts, give every item its position in the tile sorted by
+// digit (equal digits keep their order).  (4) Keys and values, then the second values, are put there in
+// shared memory and consecutive threads write consecutive sorted items to the digit's base + position:
+// runs of equal digits go out coalesced.  Only one array of values is staged at a time, which leaves
+// room for two CTAs on an SM at 12 items a thread.
+template <int kItems>
+__global__ void __launch_bounds__(kSortThreads, 2) radix_scatter(
     const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
     const uint32_t* __restrict__ vals2_in, uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
-    uint32_t* __restrict__ vals2_out, int64_t n, int shift, const int32_t* __restrict__ offs, int64_t tiles) {
-  constexpr int R = kWarpSlice / 32;  // rounds (items per thread)
+    uint32_t* __restrict__ vals2_out, int64_t n, const int32_t* __restrict__ n_dev, int shift, int bits,
+    const int32_t* __restrict__ offs, int64_t tiles) {
+  constexpr int kTile = kSortThreads * kItems;
   extern __shared__ uint32_t sort_smem[];
-  uint32_t* skey = sort_smem;           // sorted tile
-  uint32_t* sval = skey + kSortTile;
-  uint32_t* sval2 = sval + kSortTile;   // (kTwo)
-  int (*whist)[kRadix] = reinterpret_cast<int (*)[kRadix]>(sval2 + (kTwo ? kSortTile : 0));
-  __shared__ int dstart[kRadix];  // tile position where each digit's run starts
-  __shared__ int gbase[kRadix];   // global position of the digit's run of this tile
+  uint32_t* skey = sort_smem;      // sorted tile
+  uint32_t* sval = skey + kTile;   // its values, then its second values
+  int* whist = reinterpret_cast<int*>(sval + kTile);  // [warp][radix]
+  int* base = reinterpret_cast<int*>(whist + kSortWarps * kMaxRadix);  // global position of sorted position 0, per digit
+  __shared__ int wsum[kSortWarps];
+  const int radix = 1 << bits, mask = radix - 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t t0 = (int64_t)blockIdx.x * kSortTile;
-  const int cnt = (int)min((int64_t)kSortTile, n - t0);
-  for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kSortThreads) (&whist[0][0])[i] = 0;
-  if (threadIdx.x < kRadix) gbase[threadIdx.x] = offs[(int64_t)threadIdx.x * tiles + blockIdx.x];
-  uint32_t k[R], v[R], v2[R];
-  int rank[R];
+  const int64_t t0 = (int64_t)blockIdx.x * kTile;
+  if (n_dev) n = *n_dev;
+  if (t0 >= n) return;
+  const int cnt = (int)min((int64_t)kTile, n - t0);
+  int* wh = whist + warp * radix;
+  for (int i = lane; i < radix; i += 32) wh[i] = 0;
+  int goff = 0;
+  if (threadIdx.x < radix) goff = offs[(int64_t)threadIdx.x * tiles + blockIdx.x];
+  const int j0 = warp * 32 * kItems + lane;  // this thread's first item, the next ones 32 apart
+  uint32_t k[kItems], v[kItems];
+  uint32_t rank[kItems / 2];  // two 16-bit ranks, then positions, per word
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int j = warp * kWarpSlice + r * 32 + lane;
-    if (j < cnt) {
-      k[r] = keys_in[t0 + j];
-      v[r] = vals_in ? vals_in[t0 + j] : (uint32_t)(t0 + j);  // first pass: the input position
-      if (kTwo) v2[r] = vals2_in[t0 + j];
-    }
-  }
-  __syncthreads();
-  const unsigned lt_mask = (1u << lane) - 1u;
+  for (int r = 0; r < kItems; ++r) k[r] = j0 + 32 * r < cnt ? keys_in[t0 + j0 + 32 * r] : 0u;
+  __syncwarp();
+  // The first lane of each group of equal digits adds the group's size to the warp's count, and the
+  // old count is the rank of the group's first item: the adds of all rounds are in flight together (a
+  // read and a write per round, each waited for, made shared memory's latency the kernel's).
+  unsigned peers[kItems];
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int j = warp * kWarpSlice + r * 32 + lane;
-    const int d = j < cnt ? (int)((k[r] >> shift) & (kRadix - 1)) : kRadix;
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
-    const int c = d < kRadix ? whist[warp][d] : 0;
-    __syncwarp();
-    if (d < kRadix && lane == __ffs(peers) - 1) whist[warp][d] = c + __popc(peers);
-    __syncwarp();
-    rank[r] = c + __popc(peers & lt_mask);
+  for (int r = 0; r < kItems; ++r)
+    peers[r] = __match_any_sync(0xffffffffu, j0 + 32 * r < cnt ? (int)(k[r] >> shift) & mask : radix);
+  int old[kItems];
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    old[r] = 0;
+    if (j0 + 32 * r < cnt && lane == __ffs(peers[r]) - 1) old[r] = atomicAdd(&wh[(k[r] >> shift) & mask], __popc(peers[r]));
+    __syncwarp();  // the next round's adds come after
   }
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    const uint32_t rk = __shfl_sync(0xffffffffu, old[r], __ffs(peers[r]) - 1) + __popc(peers[r] & ((1u << lane) - 1u));
+    if (r & 1) rank[r / 2] |= rk << 16;
+    else rank[r / 2] = rk;
+  }
+#pragma unroll
+  for (int r = 0; r < kItems; ++r)  // in flight over the prefixes; first pass: the input position
+    v[r] = j0 + 32 * r < cnt ? (vals_in ? vals_in[t0 + j0 + 32 * r] : (uint32_t)(t0 + j0 + 32 * r)) : 0u;
   __syncthreads();
-  if (threadIdx.x < kRadix) {  // per digit: exclusive prefix over warps; tile total
-    int run = 0;
+  int tot = 0;  // this thread's digit: items of the tile
+  if (threadIdx.x < radix)
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) tot += whist[w * radix + threadIdx.x];
+  const int incl = warp_inclusive_scan(tot);
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  if (threadIdx.x < radix) {
+    int run = incl - tot;  // sorted position of the digit's first item
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) run += w < warp ? wsum[w] : 0;
+    base[threadIdx.x] = goff - run;
 #pragma unroll
     for (int w = 0; w < kSortWarps; ++w) {
-      const int c = whist[w][threadIdx.x];
-      whist[w][threadIdx.x] = run;
+      const int c = whist[w * radix + threadIdx.x];
+      whist[w * radix + threadIdx.x] = run;
       run += c;
     }
-    dstart[threadIdx.x] = run;
-  }
-  __syncthreads();
-  if (warp == 0) {  // exclusive scan of the 256 digit totals
-    int vv[kRadix / 32], sum = 0;
-#pragma unroll
-    for (int i = 0; i < kRadix / 32; ++i) {
-      vv[i] = dstart[lane * (kRadix / 32) + i];
-      sum += vv[i];
-    }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    int run = incl - sum;
-#pragma unroll
-    for (int i = 0; i < kRadix / 32; ++i) {
-      dstart[lane * (kRadix / 32) + i] = run;
-      run += vv[i];
-    }
   }
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int j = warp * kWarpSlice + r * 32 + lane;
-    if (j < cnt) {
-      const int d = (int)((k[r] >> shift) & (kRadix - 1));
-      const int p = dstart[d] + whist[warp][d] + rank[r];
+  for (int r = 0; r < kItems; ++r) {
+    if (j0 + 32 * r < cnt) {
+      const uint32_t p = wh[(k[r] >> shift) & mask] + ((rank[r / 2] >> (16 * (r & 1))) & 0xFFFFu);
       skey[p] = k[r];
       sval[p] = v[r];
-      if (kTwo) sval2[p] = v2[r];
+      rank[r / 2] = (r & 1) ? (rank[r / 2] & 0xFFFFu) | p << 16 : (rank[r / 2] & 0xFFFF0000u) | p;
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) v[r] = j0 + 32 * r < cnt ? vals2_in[t0 + j0 + 32 * r] : 0u;  // in flight meanwhile
+  __syncthreads();
+  int pos[kItems];
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    const int p = threadIdx.x + r * kSortThreads;
+    if (p < cnt) {
+      const uint32_t kk = skey[p];
+      pos[r] = base[(kk >> shift) & mask] + p;
+      keys_out[pos[r]] = kk;
+      vals_out[pos[r]] = sval[p];
     }
   }
   __syncthreads();
-  for (int p = threadIdx.x; p < cnt; p += kSortThreads) {
-    const uint32_t kk = skey[p];
-    const int d = (int)((kk >> shift) & (kRadix - 1));
-    const int64_t pos = (int64_t)gbase[d] + (p - dstart[d]);
-    keys_out[pos] = kk;
-    vals_out[pos] = sval[p];
-    if (kTwo) vals2_out[pos] = sval2[p];
+#pragma unroll
+  for (int r = 0; r < kItems; ++r)
+    if (j0 + 32 * r < cnt) sval[(rank[r / 2] >> (16 * (r & 1))) & 0xFFFFu] = v[r];
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    const int p = threadIdx.x + r * kSortThreads;
+    if (p < cnt) vals2_out[pos[r]] = sval[p];
   }
 }
 
 struct SortBuffers {
-  uint32_t* ckeys;  // CSR row keys (payload of the first sort), then the CSC keys
+  uint32_t* ckeys;  // CSR row keys (payload of the first sort), then the runs' CSC keys
   uint32_t* keys[2];
   uint32_t* vals[2];
   uint32_t* vals2[2];  // second payload (carried so the finish passes read sequentially)
@@ -327,21 +371,28 @@ struct SortBuffers {
   void* scan_scratch;
 };
 
-static int64_t sort_tiles(int64_t n) { return std::max<int64_t>(1, ceil_div(n, kSortTile)); }
-// dynamic shared memory of radix_scatter<true>: the sorted tile (key, value, payload), warp histograms
-constexpr size_t kScatterSmem = 3 * kSortTile * sizeof(uint32_t) + kSortWarps * kRadix * sizeof(int);
+static bool sort_large(int64_t n) { return n >= kSortLarge; }
+static int64_t sort_tiles(int64_t n) {
+  return std::max<int64_t>(1, ceil_div(n, kSortThreads * (sort_large(n) ? kItemsLarge : kItemsSmall)));
+}
+// dynamic shared memory of radix_scatter: the sorted tile (key, value), warp counts, digit bases
+template <int kItems>
+constexpr size_t kScatterSmem = 2 * kSortThreads * kItems * sizeof(uint32_t) +
+                                (kSortWarps + 1) * kMaxRadix * sizeof(int);
 
 // Sorts (key, value, second payload) triples by the low `bits` key bits (at least one pass), stable.
 // The first pass reads keys_src, vals_src (null: the input positions) and vals2_src, which may lie
-// in buffer `start` (it writes buffer start ^ 1 first); returns the buffer index holding the sorted
-// keys.  The last pass writes the payloads to vals_final / vals2_final when those are given (the
-// caller's final arrays), else to the sort buffers beside the keys.
-static hg_status radix_sort(SortBuffers& b, int64_t n, int bits, const uint32_t* keys_src, const uint32_t* vals_src,
-                            const uint32_t* vals2_src, int start, cudaStream_t s, int* result,
-                            uint32_t* vals_final = nullptr, uint32_t* vals2_final = nullptr) {
+// in buffer `start` (it writes buffer start ^ 1 first); n_dev as in radix_hist; returns the buffer
+// index holding the sorted keys.  The last pass writes the payloads to vals_final / vals2_final when
+// those are given (the caller's final arrays), else to the sort buffers beside the keys.
+template <int kItems>
+static hg_status radix_sort_t(SortBuffers& b, int64_t n, const int32_t* n_dev, int bits, const uint32_t* keys_src,
+                              const uint32_t* vals_src, const uint32_t* vals2_src, int start, cudaStream_t s,
+                              int* result, uint32_t* vals_final, uint32_t* vals2_final) {
   static bool attr = false;
   if (!attr) {
-    HG_CUDA(cudaFuncSetAttribute(radix_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem));
+    HG_CUDA(cudaFuncSetAttribute(radix_scatter<kItems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kScatterSmem<kItems>));
     attr = true;
   }
   int cur = start;
@@ -349,23 +400,37 @@ static hg_status radix_sort(SortBuffers& b, int64_t n, int bits, const uint32_t*
   const uint32_t* k = keys_src;
   const uint32_t* v = vals_src;
   const uint32_t* v2 = vals2_src;
-  const int nb = std::max(bits, 1);
-  for (int shift = 0; shift < nb; shift += 8) {
-    const bool last = shift + 8 >= nb;
+  int left = std::max(bits, 1), shift = 0;
+  for (int passes = (int)ceil_div(left, kMaxBits); passes > 0; --passes) {  // the widest digits first
+    const int w = (int)ceil_div(left, passes);
+    const bool last = passes == 1;
     uint32_t* vo = last && vals_final ? vals_final : b.vals[cur ^ 1];
     uint32_t* v2o = last && vals2_final ? vals2_final : b.vals2[cur ^ 1];
-    HG_TRY(launch("radix_hist", radix_hist, dim3((unsigned)tiles), dim3(kSortThreads), 0, s, k, n, shift, b.hist,
-                  tiles));
-    HG_TRY(exclusive_scan(b.hist, b.hist, tiles * kRadix, b.scan_scratch, s));
-    HG_TRY(launch("radix_scatter", radix_scatter<true>, dim3((unsigned)tiles), dim3(kSortThreads), kScatterSmem, s, k, v, v2,
-                  b.keys[cur ^ 1], vo, v2o, n, shift, (const int32_t*)b.hist, tiles));
+    HG_TRY(launch("radix_hist", radix_hist<kItems>, dim3((unsigned)tiles), dim3(kSortThreads), 0, s, k, n, n_dev, shift,
+                  w, b.hist, tiles));
+    HG_TRY(exclusive_scan(b.hist, b.hist, tiles << w, b.scan_scratch, s));
+    HG_TRY(launch("radix_scatter", radix_scatter<kItems>, dim3((unsigned)tiles), dim3(kSortThreads),
+                  kScatterSmem<kItems>, s, k, v, v2, b.keys[cur ^ 1], vo, v2o, n, n_dev, shift, w,
+                  (const int32_t*)b.hist, tiles));
     k = b.keys[cur ^ 1];
     v = vo;
     v2 = v2o;
     cur ^= 1;
+    shift += w;
+    left -= w;
   }
   *result = cur;
   return HG_OK;
+}
+
+static hg_status radix_sort(SortBuffers& b, int64_t n, const int32_t* n_dev, int bits, const uint32_t* keys_src,
+                            const uint32_t* vals_src, const uint32_t* vals2_src, int start, cudaStream_t s,
+                            int* result, uint32_t* vals_final = nullptr, uint32_t* vals2_final = nullptr) {
+  if (sort_large(n))
+    return radix_sort_t<kItemsLarge>(b, n, n_dev, bits, keys_src, vals_src, vals2_src, start, s, result, vals_final,
+                                     vals2_final);
+  return radix_sort_t<kItemsSmall>(b, n, n_dev, bits, keys_src, vals_src, vals2_src, start, s, result, vals_final,
+                                   vals2_final);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -776,7 +841,7 @@ static size_t carve_graph(void* ws, int64_t E, int64_t rows, int64_t crows, int6
     L->sort.vals[i] = c.take<uint32_t>(Ea + 1);
     L->sort.vals2[i] = c.take<uint32_t>(Ea + 1);
   }
-  const int64_t hist_n = sort_tiles(E) * kRadix;
+  const int64_t hist_n = sort_tiles(E) * kMaxRadix;
   L->sort.hist = c.take<int32_t>(hist_n + 1);
   L->sort.scan_scratch =
       c.take<char>(scan_scratch_bytes(std::max(std::max(std::max(hist_n, rows), std::max(crows, N)),
@@ -922,10 +987,10 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     HG_TRY(launch("edge_keys", edge_keys, dim3(g), dim3(256), 0, s, src, dst, rel, E, m, rows, L.sort.keys[0],
                   L.sort.ckeys));
     int r1 = 0;
-    HG_TRY(radix_sort(L.sort, E, bit_width((uint64_t)N), (const uint32_t*)L.sort.keys[0], (const uint32_t*)nullptr,
+    HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)N), (const uint32_t*)L.sort.keys[0], (const uint32_t*)nullptr,
                       (const uint32_t*)L.sort.ckeys, 0, s, &r1));
     // the last pass writes the edge ids and source ids straight into csr_eid and csr_col
-    HG_TRY(radix_sort(L.sort, E, bit_width((uint64_t)rows), (const uint32_t*)L.sort.vals2[r1],
+    HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)rows), (const uint32_t*)L.sort.vals2[r1],
                       (const uint32_t*)L.sort.vals[r1], (const uint32_t*)L.sort.keys[r1], r1, s, &res,
                       (uint32_t*)L.csr_eid, (uint32_t*)L.csr_col));
     HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(g), dim3(256), 0, s, (const uint32_t*)L.sort.keys[res],
@@ -936,7 +1001,7 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     HG_TRY(launch("csc_keys_from_csr", csc_keys_from_csr, dim3(g), dim3(256), 0, s, (const uint32_t*)L.sort.keys[r2],
                   (const uint32_t*)L.csr_col, E, (const int32_t*)L.csr_ptr, rows, crows, m, L.sort.ckeys,
                   L.sort.keys[r2]));
-    HG_TRY(radix_sort(L.sort, E, bit_width((uint64_t)crows), (const uint32_t*)L.sort.ckeys,
+    HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)crows), (const uint32_t*)L.sort.ckeys,
                       (const uint32_t*)L.csr_eid, (const uint32_t*)L.sort.keys[r2], r2, s, &res,
                       (uint32_t*)L.csc_eid, (uint32_t*)L.csc_col));
     HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(g), dim3(256), 0, s, (const uint32_t*)L.sort.keys[res],
