@@ -131,8 +131,6 @@ struct hg_graph {
   int32_t* csc_col;
   int32_t* csc_eid;
   float* csc_coef;
-  int32_t* node_ptr;        // [N + 1] node-major out-edges over all relations (backward aggregation)
-  int32_t* node_col;        // [num_edges] dMs row of each out-edge's destination
   // Parallel edges coalesced (the aggregation lists of the mean and attention layers): the CSR rows
   // as runs of equal source ids (agg_col = source, agg_cnt = multiplicity; deg = sum of the counts =
   // CSR row length) and the node-major rows as runs of equal dMs rows (bagg_col = the compact index

@@ -167,3 +167,31 @@ def test_25_bit_row_keys():
     ref = oracle.build_csr(src, dst, rel, offs, rels)
     compare_layout(hg, G, ref, rels)
     compare_node_order(hg, G, ref, offs, rels)
+
+
+@pytest.mark.parametrize("E", [1, 31, 32, 33, 1023, 1024, 1025, 2048, 2049, 12289])
+@pytest.mark.parametrize("kind", ["one pair", "pairs twice", "distinct", "mixed"])
+def test_runs_of_parallel_edges(E, kind):
+    """The CSC arrays are written run by run: one run of every edge, runs of two, runs of one edge (whose id rides with
+    its key) and a mix, at the edges of a warp's 32 runs, its 1024 positions and a sort tile."""
+    need_gpu()
+    hg = lib()
+    offs = np.array([0, 4000, 4100], np.int64)
+    rels = ((0, 0), (0, 1), (1, 0))
+    rng = np.random.default_rng(E)
+    k = np.arange(E)
+    if kind == "one pair":
+        src, dst, rel = np.full(E, 7), np.full(E, 11), np.zeros(E, np.int64)
+    elif kind == "pairs twice":
+        src, dst, rel = (k // 2) % 4000, (k // 2 * 7) // 4000 % 4000, np.zeros(E, np.int64)
+    elif kind == "distinct":
+        src, dst, rel = k % 4000, k // 4000, np.zeros(E, np.int64)
+    else:
+        rel = rng.integers(0, 3, E)
+        pick = lambda t: np.where(t == 0, np.minimum(rng.pareto(0.5, E) * 3, 3999), 4000 + rng.integers(0, 3, E)).astype(np.int64)  # noqa: E731
+        src, dst = pick(np.array([a for a, _ in rels])[rel]), pick(np.array([b for _, b in rels])[rel])
+    p = rng.permutation(E)
+    src, dst, rel = src[p], dst[p], rel[p]
+    G, bad = gpu_csr(hg, src, dst, rel, offs, rels)
+    assert bad == 0
+    compare_layout(hg, G, oracle.build_csr(src, dst, rel, offs, rels), rels)
