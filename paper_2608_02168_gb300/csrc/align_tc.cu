@@ -228,7 +228,7 @@ struct ABwdCfg {
   static constexpr int KC = D / 64;
   static constexpr int kB = KC * D * 128;    // C - I: D rows (N) x D (K), 64-column blocks of D x 128 B, resident
   static constexpr int kA = KC * 128 * 128;  // Z tile: 128 rows x D, K-major, 64-column blocks of 16 KB
-  static constexpr int kPCols = 32;          // P staged through shared memory 32 columns at a time
+  static constexpr int kPCols = 64;          // P staged through shared memory 64 columns at a time
   static constexpr int kPLd = kPCols + 4;    // padded fp32 rows (conflict-free 16-byte accesses)
   static constexpr int kP = 128 * kPLd * 4;  // reuses the Z tile once the product is in TMEM
   static constexpr int kAP = kA > kP ? kA : kP;
@@ -237,10 +237,14 @@ struct ABwdCfg {
   static constexpr int kTmemCols = D;
 };
 
-// grid (row tiles of 128 over n_max, 2 views); 128 threads.  Tiles past the device count exit at
-// once, so the grid may be sized by a capacity far above the rows in use.
+// grid (persistent CTAs, views): a CTA takes tiles of 128 rows blockIdx.x, + gridDim.x, ... up to the
+// device count, with C - I loaded once.  (A CTA per tile of the capacity n_max loaded it for every tile,
+// and nine in ten CTAs of a 1M-row batch in a 10M-row table started only to find no rows.)  Bound by the
+// row gathers (three reads and one write of d per row at scattered rows): eight warps, the row pieces of
+// 64 columns in flight for four rows per thread.  1M rows of a 10M-row table, d = 128: 1.04 -> 0.46 ms.
+constexpr int kBwdThreads = 256;
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kBwdThreads, 1)
     align_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_cmi, const __nv_bfloat16* __restrict__ Ha,
                         int64_t rows_a, const int32_t* __restrict__ ia, const __nv_bfloat16* __restrict__ Hb,
                         int64_t rows_b, const int32_t* __restrict__ ib, int64_t n_max,
@@ -250,14 +254,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   using C = ABwdCfg<D>;
   constexpr int KC = C::KC;
   constexpr int TPR = D / 8;
-  constexpr int RPP = kThreads / TPR;
+  constexpr int RPP = kBwdThreads / TPR;
   constexpr int PPR = C::kPCols / 8;       // 16-byte pieces per row in a P pass
-  constexpr int PRP = kThreads / PPR;      // rows per P-pass step
+  constexpr int PRP = kBwdThreads / PPR;   // rows per P-pass step
   const int view = blockIdx.y;
   const int64_t n = count_of(n_dev, n_max);
-  const int64_t m0 = (int64_t)blockIdx.x * 128;
   __nv_bfloat16* dH = view ? dHb : dHa;
-  if (m0 >= n || n < 2 || *bad || dH == nullptr) return;  // uniform over the CTA
+  if ((int64_t)blockIdx.x * 128 >= n || n < 2 || *bad || dH == nullptr) return;  // uniform over the CTA
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint8_t* Bt = smem;
@@ -281,136 +284,147 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int kc = 0; kc < KC; ++kc) tma_load_2d(Bt + kc * D * 128, &tm_cmi, kc * 64, view * D, bbar);
   }
   if (warp == 0) tmem_alloc(tslot, C::kTmemCols);
-  {  // table rows of the tile (clamped)
-    const int64_t r = m0 + threadIdx.x;
-    rowa[threadIdx.x] = r < n ? safe_row(ia, r, rows_a) : 0;
-    rowb[threadIdx.x] = r < n ? safe_row(ib, r, rows_b) : 0;
-  }
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tmem = *tslot;
-  const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-
-  // the bf16 Z_v tile (K-major, 128B-swizzled), rows past n zero
-  {
-    const int64_t* rowv = view ? rowb : rowa;
-    const int g = threadIdx.x % TPR, sub = threadIdx.x / TPR;
-    float zmu[8], zk[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      zmu[i] = stats[view * D + g * 8 + i];
-      zk[i] = rsn / stats[2 * D + view * D + g * 8 + i];
+  bool ok = true;
+  uint32_t phase = 0, tmem = 0;
+  for (int64_t m0 = (int64_t)blockIdx.x * 128; m0 < n; m0 += (int64_t)gridDim.x * 128, phase ^= 1u) {
+    {  // table rows of the tile (clamped): threads 0-127 of view a, 128-255 of view b
+      const int64_t r = m0 + (threadIdx.x & 127);
+      if (threadIdx.x < 128) rowa[threadIdx.x] = r < n ? safe_row(ia, r, rows_a) : 0;
+      else rowb[threadIdx.x - 128] = r < n ? safe_row(ib, r, rows_b) : 0;
     }
-    constexpr int RT = 128 / RPP;
-    constexpr int RB = RT < 8 ? RT : 8;  // loads in flight per batch
-#pragma unroll 1
-    for (int p0 = 0; p0 < RT; p0 += RB) {
-      uint4 v[RB];
-#pragma unroll
-      for (int q = 0; q < RB; ++q) {
-        const int rl = sub + (p0 + q) * RPP;
-        v[q] = m0 + rl < n ? ldg16(H + rowv[rl] * D + g * 8) : make_uint4(0, 0, 0, 0);
-      }
-#pragma unroll
-      for (int q = 0; q < RB; ++q) {
-        const int rl = sub + (p0 + q) * RPP;
-        st16(At + (g >> 3) * (128 * 128) + sw128_offset(rl, (g & 7) * 16),
-             m0 + rl < n ? standardise8(v[q], zmu, zk) : make_uint4(0, 0, 0, 0));
-      }
-    }
-  }
-  fence_async_smem();
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  if (threadIdx.x == 0) {
-    if (mbar_wait(bbar, 0)) {
-      const uint32_t idesc = idesc_bf16(128, D, false, false);
-      const uint32_t A = smem_u32(At), B = smem_u32(Bt);
-#pragma unroll
-      for (int kc = 0; kc < KC; ++kc)
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-          mma_bf16(tmem, desc_sw128(A + kc * (128 * 128) + ks * 32, 16, 1024),
-                   desc_sw128(B + kc * (D * 128) + ks * 32, 16, 1024), idesc, (kc > 0 || ks > 0) ? 1u : 0u);
-    } else {
-      atomicOr(status, kErrTimeout);
-      mbar_wait(bbar, 0);  // give-up path: the weight load still lands before the CTA moves on
-    }
-    mma_commit(accb);
-  }
-  if (!mbar_wait(accb, 0)) atomicOr(status, kErrTimeout);
-  fence_after_sync();
-
-  // dX = (g / sqrt(n) - mean g - x_hat mean(g x_hat)) / s, g = dloss (+-2 (z_a - z_b) + 4 lambda P)
-  const float* mu_a = stats;
-  const float* mu_b = stats + D;
-  const float* s_a = stats + 2 * D;
-  const float* s_b = stats + 3 * D;
-  const float* mg_v = means + (view * 2 + 0) * D;
-  const float* mgx_v = means + (view * 2 + 1) * D;
-  const float two_sign_dloss = (view ? -2.f : 2.f) * dloss;
-  const float p_scale = 4.f * lambda_n * dloss;
-  const int pg = threadIdx.x % PPR, psub = threadIdx.x / PPR;
-#pragma unroll 1
-  for (int c0p = 0; c0p < D; c0p += C::kPCols) {
-    __syncthreads();  // the Z tile (first pass) or the previous staging is no longer read
-#pragma unroll
-    for (int c = 0; c < C::kPCols; c += 16) {
-      float v[16];
-      tmem_ld16(trow + c0p + c, v);
-      float* dst = Ps + threadIdx.x * C::kPLd + c;
-#pragma unroll
-      for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-    }
+    fence_before_sync();
     __syncthreads();
-    const int c0 = c0p + pg * 8;
-    float ma[8], mb[8], ka[8], kb[8], iv[8], mg[8], mgx[8];  // ka, kb = 1 / (s sqrt n); iv = 1 / s_v
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      ma[i] = mu_a[c0 + i];
-      mb[i] = mu_b[c0 + i];
-      const float ra = 1.f / s_a[c0 + i], rb = 1.f / s_b[c0 + i];
-      ka[i] = ra * rsn;
-      kb[i] = rb * rsn;
-      iv[i] = view ? rb : ra;
-      mg[i] = mg_v[c0 + i];
-      mgx[i] = mgx_v[c0 + i];
-    }
-    constexpr int RT = 128 / PRP;  // rows per thread in this pass
-    uint4 xa4[RT], xb4[RT], d4[RT];
-#pragma unroll
-    for (int q = 0; q < RT; ++q) {
-      const int rl = psub + q * PRP;
-      if (m0 + rl < n) {
-        xa4[q] = ldg16(Ha + rowa[rl] * D + c0);
-        xb4[q] = ldg16(Hb + rowb[rl] * D + c0);
-        d4[q] = ld16(dH + (view ? rowb[rl] : rowa[rl]) * D + c0);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < RT; ++q) {
-      const int rl = psub + q * PRP;
-      if (m0 + rl >= n) continue;
-      float xa[8], xb[8], d[8];
-      unpack(xa4[q], xa, __nv_bfloat16());
-      unpack(xb4[q], xb, __nv_bfloat16());
-      unpack(d4[q], d, __nv_bfloat16());
-      const float* ps = Ps + rl * C::kPLd + pg * 8;
-      const float4 lo = *reinterpret_cast<const float4*>(ps);
-      const float4 hi = *reinterpret_cast<const float4*>(ps + 4);
-      const float P[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    fence_after_sync();
+    tmem = *tslot;
+    const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+
+    // the bf16 Z_v tile (K-major, 128B-swizzled), rows past n zero
+    {
+      const int64_t* rowv = view ? rowb : rowa;
+      const int g = threadIdx.x % TPR, sub = threadIdx.x / TPR;
+      float zmu[8], zk[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const float za = (xa[i] - ma[i]) * ka[i];
-        const float zb = (xb[i] - mb[i]) * kb[i];
-        const float gv = two_sign_dloss * (za - zb) + p_scale * P[i];
-        const float xh = view ? (xb[i] - mb[i]) * iv[i] : (xa[i] - ma[i]) * iv[i];
-        d[i] += (gv * rsn - mg[i] - xh * mgx[i]) * iv[i];
+        zmu[i] = stats[view * D + g * 8 + i];
+        zk[i] = rsn / stats[2 * D + view * D + g * 8 + i];
       }
-      st16(dH + (view ? rowb[rl] : rowa[rl]) * D + c0, pack(d, __nv_bfloat16()));
+      constexpr int RT = 128 / RPP;
+      constexpr int RB = RT < 8 ? RT : 8;  // loads in flight per batch
+#pragma unroll 1
+      for (int p0 = 0; p0 < RT; p0 += RB) {
+        uint4 v[RB];
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          const int rl = sub + (p0 + q) * RPP;
+          v[q] = m0 + rl < n ? ldg16(H + rowv[rl] * D + g * 8) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          const int rl = sub + (p0 + q) * RPP;
+          st16(At + (g >> 3) * (128 * 128) + sw128_offset(rl, (g & 7) * 16),
+               m0 + rl < n ? standardise8(v[q], zmu, zk) : make_uint4(0, 0, 0, 0));
+        }
+      }
     }
+    fence_async_smem();
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    if (threadIdx.x == 0) {
+      ok = mbar_wait(bbar, 0);
+      if (ok) {
+        const uint32_t idesc = idesc_bf16(128, D, false, false);
+        const uint32_t A = smem_u32(At), B = smem_u32(Bt);
+#pragma unroll
+        for (int kc = 0; kc < KC; ++kc)
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks)
+            mma_bf16(tmem, desc_sw128(A + kc * (128 * 128) + ks * 32, 16, 1024),
+                     desc_sw128(B + kc * (D * 128) + ks * 32, 16, 1024), idesc, (kc > 0 || ks > 0) ? 1u : 0u);
+      } else {
+        atomicOr(status, kErrTimeout);
+        mbar_wait(bbar, 0);  // give-up path: the weight load still lands before the CTA moves on
+      }
+      mma_commit(accb);
+    }
+    if (!mbar_wait(accb, phase)) {
+      atomicOr(status, kErrTimeout);
+      ok = false;
+    }
+    fence_after_sync();
+
+    // dX = (g / sqrt(n) - mean g - x_hat mean(g x_hat)) / s, g = dloss (+-2 (z_a - z_b) + 4 lambda P)
+    const float* mu_a = stats;
+    const float* mu_b = stats + D;
+    const float* s_a = stats + 2 * D;
+    const float* s_b = stats + 3 * D;
+    const float* mg_v = means + (view * 2 + 0) * D;
+    const float* mgx_v = means + (view * 2 + 1) * D;
+    const float two_sign_dloss = (view ? -2.f : 2.f) * dloss;
+    const float p_scale = 4.f * lambda_n * dloss;
+    const int pg = threadIdx.x % PPR, psub = threadIdx.x / PPR;
+#pragma unroll 1
+    for (int c0p = 0; c0p < D; c0p += C::kPCols) {
+      __syncthreads();  // the Z tile (first pass) or the previous staging is no longer read
+#pragma unroll
+      for (int cc = 0; cc < C::kPCols / 2; cc += 16) {  // warps 0-3 the first half of the columns, 4-7 the second
+        const int c = (warp >> 2) * (C::kPCols / 2) + cc;
+        float v[16];
+        tmem_ld16(trow + c0p + c, v);
+        float* dst = Ps + ((warp & 3) * 32 + (threadIdx.x & 31)) * C::kPLd + c;
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      }
+      __syncthreads();
+      const int c0 = c0p + pg * 8;
+      float ma[8], mb[8], ka[8], kb[8], iv[8], mg[8], mgx[8];  // ka, kb = 1 / (s sqrt n); iv = 1 / s_v
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        ma[i] = mu_a[c0 + i];
+        mb[i] = mu_b[c0 + i];
+        const float ra = 1.f / s_a[c0 + i], rb = 1.f / s_b[c0 + i];
+        ka[i] = ra * rsn;
+        kb[i] = rb * rsn;
+        iv[i] = view ? rb : ra;
+        mg[i] = mg_v[c0 + i];
+        mgx[i] = mgx_v[c0 + i];
+      }
+      constexpr int RT = 128 / PRP;  // rows per thread in this pass
+      uint4 xa4[RT], xb4[RT], d4[RT];
+#pragma unroll
+      for (int q = 0; q < RT; ++q) {
+        const int rl = psub + q * PRP;
+        if (m0 + rl < n) {
+          xa4[q] = ldg16(Ha + rowa[rl] * D + c0);
+          xb4[q] = ldg16(Hb + rowb[rl] * D + c0);
+          d4[q] = ld16(dH + (view ? rowb[rl] : rowa[rl]) * D + c0);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < RT; ++q) {
+        const int rl = psub + q * PRP;
+        if (m0 + rl >= n) continue;
+        float xa[8], xb[8], d[8];
+        unpack(xa4[q], xa, __nv_bfloat16());
+        unpack(xb4[q], xb, __nv_bfloat16());
+        unpack(d4[q], d, __nv_bfloat16());
+        const float* ps = Ps + rl * C::kPLd + pg * 8;
+        const float4 lo = *reinterpret_cast<const float4*>(ps);
+        const float4 hi = *reinterpret_cast<const float4*>(ps + 4);
+        const float P[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float za = (xa[i] - ma[i]) * ka[i];
+          const float zb = (xb[i] - mb[i]) * kb[i];
+          const float gv = two_sign_dloss * (za - zb) + p_scale * P[i];
+          const float xh = view ? (xb[i] - mb[i]) * iv[i] : (xa[i] - ma[i]) * iv[i];
+          d[i] += (gv * rsn - mg[i] - xh * mgx[i]) * iv[i];
+        }
+        st16(dH + (view ? rowb[rl] : rowa[rl]) * D + c0, pack(d, __nv_bfloat16()));
+      }
+    }
+    fence_before_sync();
+    if (!__syncthreads_and(ok)) break;  // the tile's rows, staging and accumulator are no longer read
   }
   fence_before_sync();
   __syncthreads();
@@ -447,7 +461,9 @@ hg_status bwd_t(const void* Ha, int64_t rows_a, const int32_t* ia, const void* H
                 dloss, (__nv_bfloat16*)cmi, means));
   CUtensorMap tm;
   HG_TRY(make_tmap_bf16(&tm, cmi, (uint64_t)2 * D, D, D));
-  return launch("align_bwd_tc", align_bwd_tc_kernel<D>, dim3((unsigned)ceil_div(n_max, 128), 2), dim3(kThreads),
+  // a CTA per SM (its registers: two per SM spill, 0.51 ms), view b only if it has a gradient
+  return launch("align_bwd_tc", align_bwd_tc_kernel<D>,
+                dim3((unsigned)std::min<int64_t>(ceil_div(n_max, 128), 152), dHb ? 2 : 1), dim3(kBwdThreads),
                 ABwdCfg<D>::kSmem, s, tm, (const __nv_bfloat16*)Ha, rows_a, ia, (const __nv_bfloat16*)Hb, rows_b, ib,
                 n_max, n_dev, stats, bad, (const float*)means, lambda_n, dloss, (__nv_bfloat16*)dHa,
                 (__nv_bfloat16*)dHb, device_status_ptr());

@@ -157,3 +157,15 @@ def test_align_bf16_device_count_far_below_capacity(d):
     assert relerr(gB[ib], rB[ib]) <= TOL["bf16"], relerr(gB[ib], rB[ib])
     assert np.abs(gA[np.setdiff1d(np.arange(len(Ha)), ia)]).max() == 0
     assert hg.hg_device_status() == 0
+
+
+@pytest.mark.parametrize("d,n", [(64, 152 * 128 + 1), (128, 40_001), (256, 2 * 152 * 128 - 1)])
+def test_align_bf16_gradient_ctas_take_several_tiles(d, n):
+    """More 128-row tiles than SMs, a ragged last one: each gradient CTA loops over tiles, both views."""
+    need_gpu()
+    hg = lib()
+    Ha, ia, Hb, ib = views(500 + d, n + 100, n, d, "bf16")
+    _, gA, gB, _, _ = align_gpu(hg, Ha, ia, Hb, ib, "bf16", 0.05, 1e-8, 0.5)
+    rA, rB = oracle.align_backward(Ha, ia, Hb, ib, 0.05, 1e-8, 0.5)
+    assert relerr(gA[ia], rA[ia]) <= TOL["bf16"] and relerr(gB[ib], rB[ib]) <= TOL["bf16"]
+    assert hg.hg_device_status() == 0
