@@ -66,7 +66,7 @@ constexpr int kAlignBlocks = 304;  // row blocks of the column reductions (2 per
 //   MODE 0: x_a, x_b                               part[block][2][d]
 //   MODE 1: (x_a - mu_a)^2, (x_b - mu_b)^2          part[block][2][d]
 //   MODE 2: the kNumCross sums of z (CrossSum)      part[block][6][d]
-// A thread owns one 16-byte piece (VEC columns) of a row and keeps four rows in flight.
+// A thread owns one 16-byte piece (VEC columns) of a row and keeps eight rows (mode 2: four) in flight.
 template <typename T, int D, int MODE>
 __global__ void __launch_bounds__(256, 2) align_colstats(const T* __restrict__ Ha, int64_t rows_a,
                                                       const int32_t* __restrict__ ia, const T* __restrict__ Hb,
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256, 2) align_colstats(const T* __restrict__ H
   constexpr int TPR = D / VEC;                // threads per row
   constexpr int RPP = 256 / TPR;              // rows per block pass
   constexpr int Q = MODE == 2 ? kNumCross : 2;
-  constexpr int U = MODE == 2 ? 2 : 4;        // rows in flight per thread
+  constexpr int U = MODE == 2 ? 4 : 8;        // rows in flight per thread
   constexpr int SLOTS = TPR < 32 ? 8 : RPP;   // partial rows left after the warp-level sums
   __shared__ float red[SLOTS][D];
   const int64_t n = count_of(n_dev, n_max);
@@ -98,36 +98,51 @@ __global__ void __launch_bounds__(256, 2) align_colstats(const T* __restrict__ H
   for (int q = 0; q < Q; ++q)
 #pragma unroll
     for (int i = 0; i < VEC; ++i) acc[q][i] = 0.f;
+  // The rows' table indexes are read an iteration ahead, and the row pieces are kept as loaded until they
+  // are added: eight (four) rows of both views in flight per thread instead of waiting on an index and
+  // then a row.  1M rows of a 10M-row table, d = 128, the three modes: 220 / 211 / 235 -> 96 / 137 / 158 us.
   const int64_t step = (int64_t)gridDim.x * RPP;
-  for (int64_t r0 = (int64_t)blockIdx.x * RPP + sub; r0 < n; r0 += U * step) {
-    float xa[U][VEC], xb[U][VEC];
+  int64_t na[U], nb[U];
+  auto rows_of = [&](int64_t r0) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t r = r0 + u * step;
-      if (r < n) {
-        if (MODE == 0 && g == 0) {
-          const int64_t va = ia[r], vb = ib[r];
-          if (va < 0 || va >= rows_a || vb < 0 || vb >= rows_b) atomicOr(bad, 1);
-        }
-        unpack(ldg16(Ha + safe_row(ia, r, rows_a) * D + c0), xa[u], T());
-        unpack(ldg16(Hb + safe_row(ib, r, rows_b) * D + c0), xb[u], T());
+      const int64_t r = min(r0 + u * step, n - 1);
+      na[u] = safe_row(ia, r, rows_a);
+      nb[u] = safe_row(ib, r, rows_b);
+      if (MODE == 0 && g == 0) {
+        const int64_t va = ia[r], vb = ib[r];
+        if (va < 0 || va >= rows_a || vb < 0 || vb >= rows_b) atomicOr(bad, 1);
       }
     }
+  };
+  int64_t r0 = (int64_t)blockIdx.x * RPP + sub;
+  if (r0 < n) rows_of(r0);
+  for (; r0 < n; r0 += U * step) {
+    uint4 va[U], vb[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      va[u] = ldg16(Ha + na[u] * D + c0);
+      vb[u] = ldg16(Hb + nb[u] * D + c0);
+    }
+    rows_of(r0 + U * step);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (r0 + u * step >= n) break;
+      float xa[VEC], xb[VEC];
+      unpack(va[u], xa, T());
+      unpack(vb[u], xb, T());
 #pragma unroll
       for (int i = 0; i < VEC; ++i) {
         if (MODE == 0) {
-          acc[0][i] += xa[u][i];
-          acc[1][i] += xb[u][i];
+          acc[0][i] += xa[i];
+          acc[1][i] += xb[i];
         } else if (MODE == 1) {
-          const float da = xa[u][i] - ma[i], db = xb[u][i] - mb[i];
+          const float da = xa[i] - ma[i], db = xb[i] - mb[i];
           acc[0][i] += da * da;
           acc[1][i] += db * db;
         } else {
-          const float za = (xa[u][i] - ma[i]) * ka[i];
-          const float zb = (xb[u][i] - mb[i]) * kb[i];
+          const float za = (xa[i] - ma[i]) * ka[i];
+          const float zb = (xb[i] - mb[i]) * kb[i];
           acc[kSumZa][i] += za;
           acc[kSumZb][i] += zb;
           acc[kSumZaZb][i] += za * zb;
