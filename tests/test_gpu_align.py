@@ -169,3 +169,23 @@ def test_align_bf16_gradient_ctas_take_several_tiles(d, n):
     rA, rB = oracle.align_backward(Ha, ia, Hb, ib, 0.05, 1e-8, 0.5)
     assert relerr(gA[ia], rA[ia]) <= TOL["bf16"] and relerr(gB[ib], rB[ib]) <= TOL["bf16"]
     assert hg.hg_device_status() == 0
+
+
+@pytest.mark.parametrize("na,nb", [(1023, 1023), (1024, 1024), (1025, 4096), (4096, 300_000), (300_000, 70), (2049, 2)])
+@pytest.mark.parametrize("kind", ["same", "apart", "mixed"])
+def test_intersect_stretches(na, nb, kind):
+    """A CTA's 1024 entries of a and the stretch of b they span: at its edges, one that fits shared memory and one
+    that does not, lists that are equal where they overlap or share nothing."""
+    need_gpu()
+    hg = lib()
+    rng = np.random.default_rng(na * 7 + nb)
+    if kind == "same":
+        a, b = np.arange(na, dtype=np.int64) * 3, np.arange(nb, dtype=np.int64) * 3
+    elif kind == "apart":
+        a, b = np.arange(na, dtype=np.int64) * 2, np.arange(nb, dtype=np.int64) * 2 + 1
+    else:
+        space = 2 * max(na, nb)
+        a, b = (np.sort(rng.choice(space, n, replace=False)).astype(np.int64) for n in (na, nb))
+    k, ia, ib = intersect_gpu(hg, a, b)
+    ra, rb = oracle.overlap_intersect(a, b)
+    assert k == len(ra) and np.array_equal(ia, ra) and np.array_equal(ib, rb)
