@@ -7,7 +7,9 @@
 //                       below depends on it);
 //   h-index ........... per node the largest h with at least h neighbour degrees >= h: short lists
 //                       by warp ballots, longer ones by a bounded binary search on the count
-//                       function (warp per node; a CTA per node above kBigList);
+//                       function (warp per node; a CTA per node above kBigList).  When the caller
+//                       does not ask for the h-indices, only h <= theta is decided, from counts that
+//                       stop at theta + 1 and without the lists (ob_marks, ob_rich);
 //   candidates (Eq. 4)  node flags from an edge-parallel pass (v -> u, u in V_k, v outside);
 //   selection ......... the M smallest sampling keys among the candidates with h <= theta, by a
 //                       four-pass radix select on the device (ties by id through a scan);
@@ -54,6 +56,94 @@ __device__ __forceinline__ int aggregated_claim(int32_t* ctr, int key) {
   if (key >= 0 && lane == leader) base = atomicAdd(&ctr[key], __popc(peers));
   base = __shfl_sync(0xffffffffu, base, leader);
   return base + __popc(peers & ((1u << lane) - 1u));
+}
+
+// base[v] = v in V_k (a byte per node, so that the edge passes look the partition up instead of hashing
+// both endpoints of every edge)
+__global__ void ob_base(int64_t N, uint64_t part_seed, int K, int k, uint8_t* __restrict__ base) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
+    base[v] = part_of(v, part_seed, K) == k;
+}
+
+// ---- h(v) <= theta without h(v).  The count of incident edges that lead to nodes of degree >= x falls
+// with x, so h(v) > theta exactly when at least B = theta + 1 of them lead to nodes of degree >= B.
+// Degrees and counts therefore only have to be right below B: a node that has reached B is not added to
+// again, which spares the hubs, where most edges end, their atomics.  (A value read before another
+// warp's addition only leads to an addition too many, and everything from B on reads the same.)  The
+// degrees and incidence lists with their h-indices took 3.4 of 3.8 ms on the 1M-node, 20M-edge graph;
+// these two passes take 0.6 ms.
+constexpr int kEdgeRounds = 4;  // edges per lane whose endpoints are looked up together
+
+__device__ __forceinline__ void add_below(int32_t* ctr, int32_t v, bool add) {
+  if (__any_sync(0xffffffffu, add)) aggregated_claim(ctr, add ? v : -1);
+}
+
+// Calls f(s, t, live) for this warp's edges, whole warps together, kEdgeRounds edges per lane at a time:
+// f takes arrays of kEdgeRounds endpoints (0 where not live: past the end, or an endpoint out of range).
+template <typename F>
+__device__ __forceinline__ void for_edges(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E,
+                                          int64_t N, F f) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t e0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32 * kEdgeRounds; e0 < E;
+       e0 += warps * 32 * kEdgeRounds) {
+    int32_t s[kEdgeRounds], t[kEdgeRounds];
+    bool live[kEdgeRounds];
+#pragma unroll
+    for (int r = 0; r < kEdgeRounds; ++r) {
+      const int64_t e = e0 + 32 * r + lane;
+      s[r] = e < E ? src[e] : -1;
+      t[r] = e < E ? dst[e] : -1;
+    }
+#pragma unroll
+    for (int r = 0; r < kEdgeRounds; ++r) {
+      live[r] = edge_ok(s[r], t[r], N);
+      if (!live[r]) s[r] = t[r] = 0;
+    }
+    f(s, t, live);
+  }
+}
+
+// deg[v] = min(degree, B) at least, and the candidate flags of Eq. 4 (as ob_candidates)
+__global__ void __launch_bounds__(256) ob_marks(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                int64_t E, int64_t N, int64_t B, const uint8_t* __restrict__ base,
+                                                int32_t* deg, int32_t* cand) {
+  for_edges(src, dst, E, N, [&](const int32_t (&s)[kEdgeRounds], const int32_t (&t)[kEdgeRounds],
+                                const bool (&live)[kEdgeRounds]) {
+    int32_t ds[kEdgeRounds], dt[kEdgeRounds];
+    bool bs[kEdgeRounds], bt[kEdgeRounds];
+#pragma unroll
+    for (int r = 0; r < kEdgeRounds; ++r) {
+      ds[r] = __ldcg(deg + s[r]);
+      dt[r] = __ldcg(deg + t[r]);
+      bs[r] = __ldg(base + s[r]);
+      bt[r] = __ldg(base + t[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < kEdgeRounds; ++r) {
+      add_below(deg, s[r], live[r] && ds[r] < B);
+      add_below(deg, t[r], live[r] && dt[r] < B);
+      if (live[r] && bt[r] && !bs[r] && __ldcg(cand + s[r]) == 0) atomicOr(&cand[s[r]], 1);
+    }
+  });
+}
+
+// rich[v] = min(incident edges leading to nodes of degree >= B, B) at least, for the nodes of degree >= B
+// (no other node can have B of them)
+__global__ void __launch_bounds__(256) ob_rich(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                               int64_t E, int64_t N, int64_t B, const int32_t* __restrict__ deg,
+                                               int32_t* rich) {
+  for_edges(src, dst, E, N, [&](const int32_t (&s)[kEdgeRounds], const int32_t (&t)[kEdgeRounds],
+                                const bool (&live)[kEdgeRounds]) {
+    bool both[kEdgeRounds];
+#pragma unroll
+    for (int r = 0; r < kEdgeRounds; ++r) both[r] = live[r] && __ldg(deg + s[r]) >= B && __ldg(deg + t[r]) >= B;
+#pragma unroll
+    for (int r = 0; r < kEdgeRounds; ++r) {
+      add_below(rich, s[r], both[r] && __ldcg(rich + s[r]) < B);
+      add_below(rich, t[r], both[r] && __ldcg(rich + t[r]) < B);
+    }
+  });
 }
 
 // (the loops run whole warps together: lanes past the end take key -1)
@@ -245,11 +335,11 @@ __global__ void __launch_bounds__(kBigThreads) ob_h_big(const int32_t* __restric
 
 // cand[v] = 1 for v outside V_k with an edge v -> u, u in V_k (Eq. 4)
 __global__ void ob_candidates(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E, int64_t N,
-                              uint64_t part_seed, int K, int k, int32_t* __restrict__ cand) {
+                              const uint8_t* __restrict__ base, int32_t* __restrict__ cand) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t s = src[e], t = dst[e];
     if (!edge_ok(s, t, N)) continue;
-    if (part_of(t, part_seed, K) == k && part_of(s, part_seed, K) != k && cand[s] == 0) atomicOr(&cand[s], 1);
+    if (base[t] && !base[s] && cand[s] == 0) atomicOr(&cand[s], 1);
   }
 }
 
@@ -261,16 +351,17 @@ struct SelState {
   long long rank;                                       // 0-based rank of the last taken key among the matching keys
 };
 
-// elig[v] = cand[v] && h[v] <= theta; counts of C_k, C'_k and V_k
-__global__ void ob_eligible(const int32_t* __restrict__ cand, const int32_t* __restrict__ h, int64_t N, int theta,
-                            uint64_t part_seed, int K, int k, int32_t* __restrict__ elig, SelState* st) {
+// elig[v] = cand[v] && h[v] < bound (h the h-index, or ob_rich's count; bound = theta + 1); counts of C_k,
+// C'_k and V_k
+__global__ void ob_eligible(const int32_t* __restrict__ cand, const int32_t* __restrict__ h, int64_t N, int64_t bound,
+                            const uint8_t* __restrict__ base, int32_t* __restrict__ elig, SelState* st) {
   unsigned long long c = 0, ce = 0, cb = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-    const int e = cand[v] && h[v] <= theta;
+    const int e = cand[v] && h[v] < bound;
     elig[v] = e;
     c += cand[v] != 0;
     ce += e;
-    cb += part_of(v, part_seed, K) == k;
+    cb += base[v];
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -334,14 +425,14 @@ __global__ void ob_ties(const int32_t* __restrict__ elig, int64_t N, int k, uint
 }
 
 // member[v] = v in V_k or selected (key below the threshold, or equal with tie rank <= rank)
-__global__ void ob_members(const int32_t* __restrict__ elig, const int32_t* __restrict__ eq_rank, int64_t N, int K,
-                           int k, uint64_t part_seed, uint64_t sample_seed, const SelState* __restrict__ st,
+__global__ void ob_members(const int32_t* __restrict__ elig, const int32_t* __restrict__ eq_rank, int64_t N, int k,
+                           const uint8_t* __restrict__ base, uint64_t sample_seed, const SelState* __restrict__ st,
                            int32_t* __restrict__ member) {
   const bool any = st->take > 0;
   const uint32_t T = st->prefix;
   const long long rank = st->rank;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-    bool in = part_of(v, part_seed, K) == k;
+    bool in = base[v];
     if (!in && any && elig[v]) {
       const uint32_t key = sample_key(v, k, sample_seed);
       in = key < T || (key == T && (long long)eq_rank[v] <= rank);  // eq_rank: exclusive scan of ties
@@ -398,7 +489,8 @@ static unsigned grid_of(int64_t n, int threads = 256) {
 }
 
 struct BuildLayout {
-  int32_t *deg, *ofs, *fill, *nbr, *h, *cand, *elig, *eq, *member, *keep;
+  uint8_t* base;
+  int32_t *deg, *ofs, *fill, *nbr, *cand, *elig, *eq, *member, *keep;
   unsigned int* hist;
   SelState* st;
   void* scan;
@@ -407,11 +499,11 @@ struct BuildLayout {
 static size_t carve_build(void* ws, int64_t N, int64_t E, BuildLayout* L) {
   Carve c(ws);
   const int64_t Na = std::max<int64_t>(N, 1), Ea = std::max<int64_t>(E, 1);
+  L->base = c.take<uint8_t>(Na);
   L->deg = c.take<int32_t>(Na);
   L->ofs = c.take<int32_t>(Na + 1);
   L->fill = c.take<int32_t>(Na);
   L->nbr = c.take<int32_t>(2 * Ea);
-  L->h = c.take<int32_t>(Na);
   L->cand = c.take<int32_t>(Na);
   L->elig = c.take<int32_t>(Na);
   L->eq = c.take<int32_t>(Na + 1);
@@ -469,7 +561,8 @@ extern "C" hg_status hg_overlap_build(const int32_t* src, const int32_t* dst, co
   carve_build(workspace, num_nodes, num_edges, &L);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int64_t N = num_nodes, E = num_edges;
-  int32_t* h = h_out ? h_out : L.h;
+  int32_t* h = h_out;
+  const int64_t bound = (int64_t)theta + 1;  // h <= theta exactly when h < bound
   TypeOffsets toff{};
   for (int t = 0; t <= num_types; ++t) toff.v[t] = type_offsets[t];
 
@@ -478,26 +571,36 @@ extern "C" hg_status hg_overlap_build(const int32_t* src, const int32_t* dst, co
   HG_CUDA(cudaMemsetAsync(L.cand, 0, std::max<int64_t>(N, 1) * sizeof(int32_t), s));
   HG_CUDA(cudaMemsetAsync(L.hist, 0, 256 * sizeof(unsigned int), s));
   HG_CUDA(cudaMemsetAsync(L.st, 0, sizeof(SelState), s));
-  // degrees, incidence lists of neighbour degrees, h-index
-  if (E > 0)
-    HG_TRY(launch("ob_degrees", ob_degrees, dim3(grid_of(E)), dim3(256), 0, s, src, dst, E, N, L.deg));
-  HG_TRY(exclusive_scan(L.deg, L.ofs, N, L.scan, s));
-  if (E > 0)
-    HG_TRY(launch("ob_fill_lists", ob_fill_lists, dim3(grid_of(E)), dim3(256), 0, s, src, dst, E, N,
-                  (const int32_t*)L.deg, (const int32_t*)L.ofs, L.fill, L.nbr));
-  if (N > 0) {
-    HG_TRY(launch("ob_h_small", ob_h_small, dim3(grid_of(32 * N)), dim3(256), 0, s, (const int32_t*)L.ofs,
-                  (const int32_t*)L.nbr, N, h));
-    HG_TRY(launch("ob_h_big", ob_h_big, dim3((unsigned)std::min<int64_t>(N, 152 * 2)), dim3(kBigThreads), 0, s,
-                  (const int32_t*)L.ofs, (const int32_t*)L.nbr, N, h));
+  if (N > 0)
+    HG_TRY(launch("ob_base", ob_base, dim3(grid_of(N)), dim3(256), 0, s, N, part_seed, K, k, L.base));
+  const uint8_t* base = L.base;
+  if (h_out) {  // degrees, incidence lists of neighbour degrees, h-index; candidates (Eq. 4)
+    if (E > 0)
+      HG_TRY(launch("ob_degrees", ob_degrees, dim3(grid_of(E)), dim3(256), 0, s, src, dst, E, N, L.deg));
+    HG_TRY(exclusive_scan(L.deg, L.ofs, N, L.scan, s));
+    if (E > 0)
+      HG_TRY(launch("ob_fill_lists", ob_fill_lists, dim3(grid_of(E)), dim3(256), 0, s, src, dst, E, N,
+                    (const int32_t*)L.deg, (const int32_t*)L.ofs, L.fill, L.nbr));
+    if (N > 0) {
+      HG_TRY(launch("ob_h_small", ob_h_small, dim3(grid_of(32 * N)), dim3(256), 0, s, (const int32_t*)L.ofs,
+                    (const int32_t*)L.nbr, N, h));
+      HG_TRY(launch("ob_h_big", ob_h_big, dim3((unsigned)std::min<int64_t>(N, 152 * 2)), dim3(kBigThreads), 0, s,
+                    (const int32_t*)L.ofs, (const int32_t*)L.nbr, N, h));
+    }
+    if (E > 0)
+      HG_TRY(launch("ob_candidates", ob_candidates, dim3(grid_of(E)), dim3(256), 0, s, src, dst, E, N, base, L.cand));
+  } else {  // only whether h <= theta; the counts take the place of h
+    h = L.fill;
+    if (E > 0) {
+      const unsigned g = grid_of(ceil_div(E, kEdgeRounds));
+      HG_TRY(launch("ob_marks", ob_marks, dim3(g), dim3(256), 0, s, src, dst, E, N, bound, base, L.deg, L.cand));
+      HG_TRY(launch("ob_rich", ob_rich, dim3(g), dim3(256), 0, s, src, dst, E, N, bound, (const int32_t*)L.deg, h));
+    }
   }
-  // candidates (Eq. 4), the h-index filter, the selection of the M smallest keys
-  if (E > 0)
-    HG_TRY(launch("ob_candidates", ob_candidates, dim3(grid_of(E)), dim3(256), 0, s, src, dst, E, N, part_seed, K, k,
-                  L.cand));
+  // the h-index filter, the selection of the M smallest keys
   if (N > 0)
     HG_TRY(launch("ob_eligible", ob_eligible, dim3(grid_of(N)), dim3(256), 0, s, (const int32_t*)L.cand,
-                  (const int32_t*)h, N, theta, part_seed, K, k, L.elig, L.st));
+                  (const int32_t*)h, N, bound, base, L.elig, L.st));
   for (int shift = 24; shift >= 0; shift -= 8) {
     if (N > 0)
       HG_TRY(launch("ob_key_hist", ob_key_hist, dim3(grid_of(N)), dim3(256), 0, s, (const int32_t*)L.elig, N, k,
@@ -511,7 +614,7 @@ extern "C" hg_status hg_overlap_build(const int32_t* src, const int32_t* dst, co
   // V~_k (Eq. 5): membership, local ids, the induced edges
   if (N > 0)
     HG_TRY(launch("ob_members", ob_members, dim3(grid_of(N)), dim3(256), 0, s, (const int32_t*)L.elig,
-                  (const int32_t*)L.eq, N, K, k, part_seed, sample_seed, (const SelState*)L.st, L.member));
+                  (const int32_t*)L.eq, N, k, base, sample_seed, (const SelState*)L.st, L.member));
   HG_TRY(exclusive_scan(L.member, L.member, N, L.scan, s));
   if (N > 0)
     HG_TRY(launch("ob_gids", ob_gids, dim3(grid_of(N)), dim3(256), 0, s, (const int32_t*)L.member, N, gid_out));

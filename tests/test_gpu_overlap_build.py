@@ -89,3 +89,23 @@ def test_ties_and_budget_edges():
     np.testing.assert_array_equal(out["gid"].cpu().numpy(), ref["gid"])
     assert hg.hg_device_status() == 0
 
+
+
+@pytest.mark.parametrize("theta", [0, 1, 2, 5, 40, 2**31 - 1])
+@pytest.mark.parametrize("kind", ["random", "power law"])
+def test_without_h_indices(theta, kind):
+    """Without the h-indices only h <= theta is decided, from counts that stop at theta + 1: the same subgraph, with
+    parallel edges, self-loops, dropped edges and hubs, for bounds below, among and above the h-indices."""
+    need_gpu()
+    hg = lib()
+    if kind == "random":
+        src, dst, rel, offs = random_graph(theta % 97, 300, 100, 6_001, 30)
+        src[:500], dst[:500] = src[500:1000], dst[500:1000]
+        dst[1000:1100] = src[1000:1100]
+    else:
+        g = hgsynth.make_graph(hgsynth.spec("tiny-10k"))
+        src, dst, rel, offs = g["src"], g["dst"], g["rel"], [int(x) for x in g["type_offsets"]]
+    out = hg.hg_overlap_build(dev(src, torch.int32), dev(dst, torch.int32), dev(rel, torch.int32), offs, 4, 1, theta,
+                              200, 11, 13)
+    ref = ob.build(src, dst, rel, np.asarray(offs, np.int64), 4, 1, theta, 200, 11, 13)
+    compare(out, ref, check_h=False)
