@@ -1256,8 +1256,7 @@ hg_status hgt_bwd_t(const hg_graph* g, const hg_hgt_params* p, const void* H_in,
       HG_TRY(tc_weight_grad_rows(D, H.dQp, g->csr_rows, g->mlist, g->mbase, r, m.row_base[r], H.Qbuf, off, n,
                                  H.L.wpart, out, H.L.rtmp, s));
     } else if (n > 0) {
-      HG_TRY(weight_grad(kDt, D, H.dQp, m.row_base[r], H.Qbuf, off, n, H.L.wpart, out, H.L.rtmp, s, g->mrow,
-                         g->csr_rows));
+      HG_TRY(weight_grad(kDt, D, H.dQp, 0, H.Qbuf, off, n, H.L.wpart, out, H.L.rtmp, s, rel_rows(g, r, false)));
     } else {
       HG_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * dd, s));
     }

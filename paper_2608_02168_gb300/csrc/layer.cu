@@ -473,8 +473,8 @@ hg_status project_backward(const hg_graph* graph, const hg_layer_params* p, cons
     for (int r = 0; r < m.num_rels; ++r) {
       const int t = m.rel_dst[r];
       const int64_t n = m.type_off[t + 1] - m.type_off[t];
-      HG_TRY(weight_grad(p->dtype, d, L.M, m.row_base[r], L.dZ, m.type_off[t], n, L.wpart,
-                         grads->dW_rel + (size_t)r * d * d, L.rtmp, s, graph->mrow, graph->csr_rows));
+      HG_TRY(weight_grad(p->dtype, d, L.M, 0, L.dZ, m.type_off[t], n, L.wpart, grads->dW_rel + (size_t)r * d * d,
+                         L.rtmp, s, RowMap{graph->mlist, graph->mbase, r, m.row_base[r]}));
     }
   }
   if (tc)  // dW_r = G_r W_agg^T, dW_agg[t] = sum_{r -> t} W_r^T G_r

@@ -151,10 +151,19 @@ hg_status aggregate_backward(const hg_graph* g, hg_dtype dt, int d, const void* 
                              float* partials, int32_t* work, cudaStream_t s);
 hg_status proj_forward(hg_dtype dt, int d, const FwdArgs& a, cudaStream_t s);
 hg_status proj_backward(hg_dtype dt, int d, const BwdArgs& a, cudaStream_t s);
-// out = X^T Y over rows [x0, x0 + n) of X and [y0, y0 + n) of Y; with xmap, X row x0 + k is
-// X[xmap[x0 + k]] and a mapped row >= xsent is zero (X stored for non-empty rows only).
+// The stored (non-empty) rows of relation `rel`: compact rows k = base[rel] .. base[rel + 1] (device),
+// each at node list[k] - row0 of its destination type.  list null: no map.
+struct RowMap {
+  const int32_t* list = nullptr;
+  const int32_t* base = nullptr;
+  int rel = 0;
+  int64_t row0 = 0;
+  int scatter = 0;  // 0: A indexed by node, out by compact row; 1: A by compact row, out by node
+};
+// out = X^T Y over rows [x0, x0 + n) of X and [y0, y0 + n) of Y; with a map, over the relation's stored
+// rows: compact rows of X with their nodes' rows (y0 + node) of Y, at most n of them.
 hg_status weight_grad(hg_dtype dt, int d, const void* X, int64_t x0, const void* Y, int64_t y0, int64_t n, float* part,
-                      float* out, float* tmp, cudaStream_t s, const int32_t* xmap = nullptr, int64_t xsent = 0);
+                      float* out, float* tmp, cudaStream_t s, const RowMap& map = RowMap{});
 hg_status transpose_weights(hg_dtype dt, int d, const void* W, void* Wt, int count, cudaStream_t s);
 // fixed-order sum of `splits` partial arrays (tmp: reduce_tmp_floats(splits, count) floats)
 hg_status reduce_partials(const float* part, int64_t stride, int splits, int64_t count, float* out, float* tmp,
@@ -165,15 +174,6 @@ size_t reduce_tmp_floats(int splits, int64_t count);
 hg_status reduce_partials3(const float* part, int64_t stride, int splits, int64_t seg, float* out0, float* out1,
                            float* out2, cudaStream_t s);
 int wgrad_splits(int64_t n);
-// The stored (non-empty) rows of relation `rel`: compact rows k = base[rel] .. base[rel + 1] (device),
-// each at node list[k] - row0 of its destination type.  list null: no map.
-struct RowMap {
-  const int32_t* list = nullptr;
-  const int32_t* base = nullptr;
-  int rel = 0;
-  int64_t row0 = 0;
-  int scatter = 0;  // 0: A indexed by node, out by compact row; 1: A by compact row, out by node
-};
 // Tensor-core row product (bf16): out[r][ocol0 + c] (=, or += when accumulate) scale A[r] B + bias,
 // A: n x d rows (row stride d), B: d x d row-major, bias: d or null; out row stride ldo; scale =
 // scale_mul * (*scale_ptr), scale_ptr a device fp32 scalar or null (1).  With a map, over the stored
