@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(256) proj_bwd_simt(BwdArgs a) {
 // weight gradients: out = X^T Y over rows, split over row ranges, fixed-order reduction
 // ---------------------------------------------------------------------------------------------
 // With a map, over a relation's stored rows: X rows are compact rows, Y rows the rows' nodes (their count
-// is a device value, split over the grid on the device).  The next step's rows are loaded while a step
-// is multiplied.  Bound by fp32 FMA on large graphs and by the steps' latency on small ones, so a split is
+// is a device value, split over the grid on the device).  At d = 64 the next step's rows are loaded
+// while a step is multiplied (at 128 and 256 that left one CTA on an SM and lost 1 %).  Bound by fp32 FMA on large graphs and by the steps' latency on small ones, so a split is
 // 64 rows (256 before) until there are two CTAs per SM.  Per launch on 8000 nodes, d = 64: 18.1 -> 4.1 us (a
 // scan of all rows before, empty ones as zeros); 100k nodes, six launches: 183 -> 67 us.
 constexpr int kWT = 128;  // output tile edge (D >= 128) or D
@@ -289,8 +289,10 @@ __global__ void __launch_bounds__(256) wgrad_partial(const T* __restrict__ X, in
       }
     }
   };
-  if (r0 < r1) fetch(r0);
+  constexpr bool kAhead = TW < 128;  // the wide tile's sums leave no registers for it
+  if (kAhead && r0 < r1) fetch(r0);
   for (int64_t rb = r0; rb < r1; rb += kWR) {
+    if (!kAhead) fetch(rb);
 #pragma unroll
     for (int q = 0; q < kLoads; ++q) {
       const int idx = threadIdx.x + q * 256, k = idx / (TW / VEC), cv = idx % (TW / VEC);
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(256) wgrad_partial(const T* __restrict__ X, in
         Ys[k][cv * VEC + e] = fy[e];
       }
     }
-    if (rb + kWR < r1) fetch(rb + kWR);
+    if (kAhead && rb + kWR < r1) fetch(rb + kWR);
     __syncthreads();
 #pragma unroll 4
     for (int k = 0; k < kWR; ++k) {
