@@ -229,15 +229,41 @@ __global__ void __launch_bounds__(256) hgt_gemm_simt(const T* __restrict__ A, in
   }
 }
 
-// part[block][c] = sum over the block's rows (in order) of X[row][c], rows [0, n), row stride ldx.
-template <typename T>
-__global__ void hgt_colsum(const T* __restrict__ X, int64_t ldx, int d, int64_t n, int64_t rows_per_block,
-                           float* __restrict__ part) {
+// part[block][c] = sum over the block's rows of X[row][c], rows [0, n), row stride ldx.  A thread owns one
+// 16-byte piece of a row and every kRows-th row of the block, eight in flight; the threads' sums are added
+// in row order.  Bound by HBM; three sums of 1M rows, d = 128
+// bf16: 512 -> 145 us (a column per thread and a row at a time before).
+template <typename T, int D>
+__global__ void __launch_bounds__(256) hgt_colsum(const T* __restrict__ X, int64_t ldx, int64_t n,
+                                                  int64_t rows_per_block, float* __restrict__ part) {
+  constexpr int VEC = VecTraits<T>::kElems, TPR = D / VEC, kRows = 256 / TPR, U = 8;
+  __shared__ float red[kRows][D];
+  const int g = threadIdx.x % TPR, sub = threadIdx.x / TPR;
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    float s = 0.f;
-    for (int64_t r = r0; r < r1; ++r) s += to_f32(X[r * ldx + c]);
-    part[(int64_t)blockIdx.x * d + c] = s;
+  float s[VEC];
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) s[i] = 0.f;
+  for (int64_t r = r0 + sub; r < r1; r += U * kRows) {
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      v[u] = r + u * kRows < r1 ? ldg16(X + (r + u * kRows) * ldx + g * VEC) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      float f[VEC];
+      unpack(v[u], f, T());
+#pragma unroll
+      for (int i = 0; i < VEC; ++i) s[i] += f[i];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) red[sub][g * VEC + i] = s[i];
+  __syncthreads();
+  for (int c = threadIdx.x; c < D; c += 256) {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) t += red[k][c];
+    part[(int64_t)blockIdx.x * D + c] = t;
   }
 }
 
@@ -969,7 +995,9 @@ struct HgtLayout {
   float* Gq;      // R x d x d
 };
 
-constexpr int64_t kColRows = 128;  // rows per block of the bias sums (many blocks in flight)
+// rows per block of the bias sums: 128, or more so that there are at most eight blocks per SM
+constexpr int64_t kColRows = 128;
+int64_t col_rows(int64_t n) { return std::max(kColRows, ceil_div(n, 152 * 8)); }
 
 int64_t max_type_rows(const GraphMeta& m) {
   int64_t r = 1;
@@ -1006,7 +1034,7 @@ void carve_hgt(const hg_graph* g, const hg_hgt_params* p, void* saved, void* scr
   H->dQ = k.take<char>((size_t)std::max<int64_t>(N, 1) * d * b);
   const int64_t pc = std::max<int64_t>(g->chunk_cap_csr * (2 * S + d), g->chunk_cap_node * 2 * d);
   H->part = k.take<float>((size_t)std::max<int64_t>(pc, 1));
-  H->cs = k.take<float>((size_t)ceil_div(max_type_rows(m), kColRows) * d);
+  H->cs = k.take<float>((size_t)152 * 8 * d);
   H->Gw = k.take<float>(m.num_rels * dd);
   H->Gq = k.take<float>(m.num_rels * dd);
   if (saved_bytes) *saved_bytes = s.used;
@@ -1106,16 +1134,16 @@ RowMap rel_rows(const hg_graph* g, int r, bool scatter) {
   return RowMap{g->mlist, g->mbase, r, g->meta.row_base[r], scatter ? 1 : 0};
 }
 
-template <typename T>
-hg_status colsum(const void* X, int64_t ldx, int d, int64_t n, float* cs, float* out, float* tmp, cudaStream_t s) {
+template <typename T, int D>
+hg_status colsum(const void* X, int64_t n, float* cs, float* out, float* tmp, cudaStream_t s) {
   if (n <= 0) {
-    HG_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * d, s));
+    HG_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * D, s));
     return HG_OK;
   }
-  const int blocks = (int)ceil_div(n, kColRows);
-  HG_TRY(launch("hgt_colsum", hgt_colsum<T>, dim3(blocks), dim3(std::min(d, 256)), 0, s, (const T*)X, ldx, d, n,
-                kColRows, cs));
-  return reduce_partials(cs, d, blocks, d, out, tmp, s);
+  const int blocks = (int)ceil_div(n, col_rows(n));
+  HG_TRY(launch("hgt_colsum", (hgt_colsum<T, D>), dim3(blocks), dim3(256), 0, s, (const T*)X, (int64_t)D, n,
+                col_rows(n), cs));
+  return reduce_partials(cs, D, blocks, D, out, tmp, s);
 }
 
 hg_status wgrad(hg_dtype dt, int d, const void* X, int64_t x0, const void* Y, int64_t y0, int64_t n, float* out,
@@ -1241,10 +1269,10 @@ hg_status hgt_bwd_t(const hg_graph* g, const hg_hgt_params* p, const void* H_in,
     const int64_t off = m.type_off[t], n = m.type_off[t + 1] - off;
     HG_TRY(wgrad(kDt, D, H_in, off, H.dK, off, n, gr->dW_K + t * dd, H.L, s));
     HG_TRY(wgrad(kDt, D, H_in, off, H.dV, off, n, gr->dW_V + t * dd, H.L, s));
-    HG_TRY(colsum<T>((const T*)H.dK + off * D, D, D, n, H.cs, gr->db_K + (size_t)t * D, H.L.rtmp, s));
-    HG_TRY(colsum<T>((const T*)H.dV + off * D, D, D, n, H.cs, gr->db_V + (size_t)t * D, H.L.rtmp, s));
+    HG_TRY((colsum<T, D>((const T*)H.dK + off * D, n, H.cs, gr->db_K + (size_t)t * D, H.L.rtmp, s)));
+    HG_TRY((colsum<T, D>((const T*)H.dV + off * D, n, H.cs, gr->db_V + (size_t)t * D, H.L.rtmp, s)));
     HG_TRY(wgrad(kDt, D, H_in, off, H.dQ, off, n, gr->dW_Q + t * dd, H.L, s));
-    HG_TRY(colsum<T>((const T*)H.dQ + off * D, D, D, n, H.cs, gr->db_Q + (size_t)t * D, H.L.rtmp, s));
+    HG_TRY((colsum<T, D>((const T*)H.dQ + off * D, n, H.cs, gr->db_Q + (size_t)t * D, H.L.rtmp, s)));
     HG_TRY((gemm<T, D>(Hin + off * D, D, (const T*)p->W_Q + t * dd, (const T*)p->b_Q + (size_t)t * D, D, n,
                        (T*)H.Qbuf + off * D, D, 0, 0, s)));
   }
