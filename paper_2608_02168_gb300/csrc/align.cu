@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(256) align_bwd_rows(const T* __restrict__ Ha, 
     for (int k0 = 0; k0 < D; k0 += kKC) {
       for (int e = threadIdx.x; e < kKC * D; e += blockDim.x) {
         const int k = e / D, c = e % D;
-        Bs[e] = Cv[(int64_t)(k0 + k) * D + c] - ((k0 + k) == c ? 1.f : 0.f);
+        Bs[k * D + b_pos<D>(c)] = Cv[(int64_t)(k0 + k) * D + c] - ((k0 + k) == c ? 1.f : 0.f);
       }
       __syncthreads();
       mma_chunk<D, RM, CN>(Zs, LD, k0, Bs, acc);

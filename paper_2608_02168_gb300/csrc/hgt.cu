@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(256) hgt_gemm_simt(const T* __restrict__ A, in
     }
     for (int idx = threadIdx.x; idx < kKC * D; idx += blockDim.x) {
       const int k = idx / D, c = idx % D;
-      Bs[k * D + c] = to_f32(B[(int64_t)(k0 + k) * D + c]);
+      Bs[k * D + b_pos<D>(c)] = to_f32(B[(int64_t)(k0 + k) * D + c]);
     }
     __syncthreads();
     mma_chunk<D, RM, CN>(&As[0][0], kAPad, 0, Bs, acc);

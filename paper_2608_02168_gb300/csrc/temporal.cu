@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256) tgemm_simt(const TA* __restrict__ A, int6
     }
     for (int idx = threadIdx.x; idx < kKC * D; idx += blockDim.x) {
       const int k = idx / D, c = idx % D;
-      Bs[k * D + c] = to_f32(B[(int64_t)(k0 + k) * ldb + bcol0 + c]);
+      Bs[k * D + b_pos<D>(c)] = to_f32(B[(int64_t)(k0 + k) * ldb + bcol0 + c]);
     }
     __syncthreads();
     mma_chunk<D, RM, CN>(&As[0][0], kAPad, 0, Bs, acc);
