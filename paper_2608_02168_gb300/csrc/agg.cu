@@ -52,6 +52,7 @@ template <int D>
 __global__ void __launch_bounds__(D) combine_chunk_partials(const int32_t* __restrict__ chunk_row,
                                                             const int32_t* __restrict__ chunk_ofs, int64_t rows,
                                                             float* __restrict__ partials) {
+  pdl_begin();
   const int nchunks = chunk_ofs[rows];
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int row = chunk_row[c];
@@ -98,6 +99,7 @@ __global__ void __launch_bounds__(256) agg_chunks(const int32_t* __restrict__ pt
                                                   const T* __restrict__ src, const int32_t* __restrict__ chunk_row,
                                                   const int32_t* __restrict__ chunk_ofs, int64_t rows,
                                                   float* __restrict__ partials) {
+  pdl_begin();
   using S = AggShape<T, D>;
   using C = ChunkCfg<T, D>;
   extern __shared__ uint4 chunk_smem[];
@@ -470,6 +472,7 @@ __global__ void __launch_bounds__(StreamCfg<T, D>::kFwdThreads) agg_fwd_rows(
     const int32_t* __restrict__ eptr, const int32_t* __restrict__ mlist, const int32_t* __restrict__ nnz_p,
     const T* __restrict__ H, T* __restrict__ M, const int32_t* __restrict__ chunk_ofs,
     const float* __restrict__ partials, int32_t* __restrict__ work) {
+  pdl_begin();
   stream_rows<T, D, false, kGapped>(ptr, col, cnt, eptr, mlist, (int64_t)*nnz_p, H, nullptr, M, chunk_ofs, partials, work,
                            nullptr);
 }
@@ -479,6 +482,7 @@ __global__ void __launch_bounds__(StreamCfg<T, D>::kBwdThreads) agg_bwd_nodes(
     int64_t N, const int32_t* __restrict__ nptr, const int32_t* __restrict__ ncol, const int32_t* __restrict__ ncnt,
     const T* __restrict__ dMs, const T* __restrict__ dY, T* __restrict__ dH, const int32_t* __restrict__ chunk_ofs,
     const float* __restrict__ partials, int32_t* __restrict__ work) {
+  pdl_begin();
   extern __shared__ uint4 ysm_raw[];
   stream_rows<T, D, true>(nptr, ncol, ncnt, nullptr, nullptr, N, dMs, dY, dH, chunk_ofs, partials, work,
                           reinterpret_cast<T*>(ysm_raw));

@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256) intersect_flags(const int64_t* __restrict
                                                        const int64_t* __restrict__ b, int64_t nb,
                                                        int32_t* __restrict__ flag, int32_t* __restrict__ pos,
                                                        int32_t* __restrict__ bad) {
+  pdl_begin();
   __shared__ int64_t stage[kIsectStage];
   __shared__ int64_t range[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(256) intersect_flags(const int64_t* __restrict
 __global__ void intersect_write(const int32_t* __restrict__ flag, const int32_t* __restrict__ pos,
                                 const int32_t* __restrict__ ofs, int64_t na, int64_t cap, const int32_t* __restrict__ bad,
                                 int32_t* __restrict__ idx_a, int32_t* __restrict__ idx_b, int64_t* __restrict__ n_out) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < na; i += (int64_t)gridDim.x * blockDim.x) {
     if (flag[i] && ofs[i] < cap) {  // cap bounds the writes even for lists that are not ascending
       idx_a[ofs[i]] = (int32_t)i;
@@ -114,6 +116,7 @@ __global__ void __launch_bounds__(256, 2) align_colstats(const T* __restrict__ H
                                                       const int64_t* __restrict__ n_dev,
                                                       const float* __restrict__ stats, float* __restrict__ part,
                                                       int32_t* __restrict__ bad) {
+  pdl_begin();
   constexpr int VEC = VecTraits<T>::kElems;
   constexpr int TPR = D / VEC;                // threads per row
   constexpr int RPP = 256 / TPR;              // rows per block pass
@@ -228,6 +231,7 @@ __global__ void __launch_bounds__(256, 2) align_colstats(const T* __restrict__ H
 // mode 0 -> mu = sum / n;  mode 1 -> s = sqrt(sum / n + eps).
 __global__ void align_colscale(float* __restrict__ v, int count, const int64_t* __restrict__ n_dev, int64_t n_max,
                                int mode, float eps) {
+  pdl_begin();
   const int64_t n = count_of(n_dev, n_max);
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
@@ -242,6 +246,7 @@ __global__ void __launch_bounds__(256) align_gram(const T* __restrict__ Ha, int6
                                                   int64_t rows_b, const int32_t* __restrict__ ib,
                                                   int64_t n_max, const int64_t* __restrict__ n_dev,
                                                   const float* __restrict__ stats, float* __restrict__ part) {
+  pdl_begin();
   constexpr int TW = D < 128 ? D : 128;
   constexpr int TPT = TW / 16;
   constexpr int KR = 32;
@@ -304,6 +309,7 @@ __global__ void __launch_bounds__(256) align_gram(const T* __restrict__ Ha, int6
 
 // C[view] = sum of Gram partials in split order (count = 2 d^2 entries).
 __global__ void align_gram_reduce(const float* __restrict__ part, int splits, int64_t count, float* __restrict__ C) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t per = count / 2;
     const int view = (int)(i / per);
@@ -321,6 +327,7 @@ __global__ void __launch_bounds__(1024) align_loss_finish(const float* __restric
                                                           const int64_t* __restrict__ n_dev, int64_t n_max,
                                                           float lambda_n, const int32_t* __restrict__ bad,
                                                           float* __restrict__ loss) {
+  pdl_begin();
   __shared__ float red[2][32];
   const int64_t n = count_of(n_dev, n_max);
   const int64_t dd = (int64_t)d * d;
@@ -371,6 +378,7 @@ __global__ void __launch_bounds__(256) align_bwd_rows(const T* __restrict__ Ha, 
                                                       const float* __restrict__ stats, const float* __restrict__ C,
                                                       float lambda_n, float dloss, float* __restrict__ G,
                                                       float* __restrict__ part) {
+  pdl_begin();
   using TL = Tile<float, D>;
   constexpr int RM = TL::RM, CN = TL::CN;
   constexpr int LD = D + 4;
@@ -456,6 +464,7 @@ __global__ void __launch_bounds__(256) align_bwd_rows(const T* __restrict__ Ha, 
 // means[view][0][c] = mean g, means[view][1][c] = mean g * x_hat (sum of block partials / n)
 __global__ void align_bwd_means(const float* __restrict__ part, int blocks, int d, const int64_t* __restrict__ n_dev,
                                 int64_t n_max, float* __restrict__ means) {
+  pdl_begin();
   const int64_t n = count_of(n_dev, n_max);
   for (int k = threadIdx.x; k < 4 * d; k += blockDim.x) {
     float s = 0.f;
@@ -471,6 +480,7 @@ __global__ void align_bwd_apply(const T* __restrict__ Ha, int64_t rows_a, const 
                                 const int64_t* __restrict__ n_dev, int d, const float* __restrict__ stats,
                                 const float* __restrict__ G, const float* __restrict__ means,
                                 const int32_t* __restrict__ bad, T* __restrict__ dHa, T* __restrict__ dHb) {
+  pdl_begin();
   const int64_t n = count_of(n_dev, n_max);
   if (n < 2 || *bad) return;
   const float rsn = rsqrtf((float)n);

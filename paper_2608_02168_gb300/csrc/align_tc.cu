@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                          const __nv_bfloat16* __restrict__ Hb, int64_t rows_b, const int32_t* __restrict__ ib,
                          int64_t n_max, const int64_t* __restrict__ n_dev, const float* __restrict__ stats,
                          float* __restrict__ part, int* __restrict__ status) {
+  pdl_begin();
   using C = GramCfg<D>;
   constexpr int S = C::kStages;
   constexpr int TPR = D / 8;             // 16-byte pieces per row
@@ -183,6 +184,7 @@ __global__ void __launch_bounds__(256) align_bwd_coef(const float* __restrict__ 
                                                       const int64_t* __restrict__ n_dev, int64_t n_max,
                                                       float lambda_n, float dloss, __nv_bfloat16* __restrict__ cmi,
                                                       float* __restrict__ means) {
+  pdl_begin();
   __shared__ float red[2][8][33];
   const int view = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.y * 32 + lane;
@@ -251,6 +253,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
                         const int64_t* __restrict__ n_dev, const float* __restrict__ stats,
                         const int32_t* __restrict__ bad, const float* __restrict__ means, float lambda_n, float dloss,
                         __nv_bfloat16* __restrict__ dHa, __nv_bfloat16* __restrict__ dHb, int* __restrict__ status) {
+  pdl_begin();
   using C = ABwdCfg<D>;
   constexpr int KC = C::KC;
   constexpr int TPR = D / 8;

@@ -77,6 +77,7 @@ __device__ __forceinline__ void scan_store4(int32_t* out, int64_t i, int64_t n, 
 // sums[tile] = sum of the tile's kScanTile items (warp w: items tile * kScanTile + w * 512 ..)
 __global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __restrict__ in, int64_t n,
                                                                 int32_t* __restrict__ sums) {
+  pdl_begin();
   __shared__ int wt[kScanThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool vec = (reinterpret_cast<uintptr_t>(in) & 15) == 0;
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __
 // tile also writes out[n] = the grand total.  out may equal in.
 __global__ void __launch_bounds__(kScanThreads) scan_tiles(const int32_t* in, int32_t* out, int64_t n,
                                                             const int32_t* __restrict__ tile_off) {
+  pdl_begin();
   __shared__ int wt[kScanThreads / 32 + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
@@ -201,6 +203,7 @@ template <int kItems>
 __global__ void __launch_bounds__(kSortThreads) radix_hist(const uint32_t* __restrict__ keys, int64_t n,
                                                            const int32_t* __restrict__ n_dev, int shift, int bits,
                                                            int32_t* __restrict__ hist, int64_t tiles) {
+  pdl_begin();
   constexpr int kTile = kSortThreads * kItems;
   constexpr int kCopies = 4;  // four warps share a histogram
   __shared__ int h[kCopies][kMaxRadix];
@@ -264,6 +267,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter(
     const uint32_t* __restrict__ vals2_in, uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
     uint32_t* __restrict__ vals2_out, int64_t n, const int32_t* __restrict__ n_dev, int shift, int bits,
     const int32_t* __restrict__ offs, int64_t tiles) {
+  pdl_begin();
   constexpr int kTile = kSortThreads * kItems;
   extern __shared__ uint32_t sort_smem[];
   uint32_t* skey = sort_smem;      // sorted tile
@@ -448,6 +452,7 @@ __global__ void __launch_bounds__(256) edge_keys(const int32_t* __restrict__ src
                                                  const int32_t* __restrict__ rel, int64_t E, GraphMeta m,
                                                  int64_t rows, uint32_t* __restrict__ skeys,
                                                  uint32_t* __restrict__ rkeys) {
+  pdl_begin();
   __shared__ int64_t row0[kMaxRels];  // first row of relation r minus its destination type's offset
   __shared__ int32_t rsrc[kMaxRels], rdst[kMaxRels];
   if (threadIdx.x < kMaxRels) {
@@ -477,12 +482,14 @@ __global__ void __launch_bounds__(256) edge_keys(const int32_t* __restrict__ src
 // and is never stored, read or gathered)
 // ---------------------------------------------------------------------------------------------
 __global__ void nonempty_flags(const int32_t* __restrict__ ptr, int64_t rows, int32_t* __restrict__ flag) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x)
     flag[r] = ptr[r + 1] > ptr[r] ? 1 : 0;
 }
 
 // long rows of the fused layer: flag[r] = 1 when CSR row r has more than kFuseRuns runs
 __global__ void long_flags(const int32_t* __restrict__ aptr, int64_t rows, int32_t* __restrict__ flag) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x)
     flag[r] = aptr[r + 1] - aptr[r] > kFuseRuns ? 1 : 0;
 }
@@ -490,6 +497,7 @@ __global__ void long_flags(const int32_t* __restrict__ aptr, int64_t rows, int32
 // list[ofs[r]] = r for every flagged row r (ofs = the exclusive scan of the flags)
 __global__ void compact_list(const int32_t* __restrict__ flag, const int32_t* __restrict__ ofs, int64_t rows,
                              int32_t* __restrict__ list) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x)
     if (flag[r]) list[ofs[r]] = (int32_t)r;
 }
@@ -497,6 +505,7 @@ __global__ void compact_list(const int32_t* __restrict__ flag, const int32_t* __
 // mbase[r] = compact index of relation r's first non-empty row (pos = the scan of the flags, whose
 // entry `rows` is the number of non-empty rows).
 __global__ void compact_bases(const int32_t* __restrict__ pos, GraphMeta m, int32_t* __restrict__ mbase) {
+  pdl_begin();
   const int r = threadIdx.x;
   if (r <= m.num_rels) mbase[r] = pos[m.row_base[r]];
 }
@@ -505,6 +514,7 @@ __global__ void compact_bases(const int32_t* __restrict__ pos, GraphMeta m, int3
 // = the CSR row of compact row k.
 __global__ void compact_rows(const int32_t* __restrict__ flag, int64_t rows, int32_t* __restrict__ mrow,
                              int32_t* __restrict__ mlist) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
     const int32_t k = mrow[r];
     if (flag[r]) {
@@ -523,6 +533,7 @@ __global__ void compact_rows(const int32_t* __restrict__ flag, int64_t rows, int
 // capacity the scan runs over).
 __global__ void run_flags(const uint32_t* __restrict__ rkey, const int32_t* __restrict__ col,
                           const int32_t* __restrict__ ptr, int64_t rows, int64_t cap, int32_t* __restrict__ flag) {
+  pdl_begin();
   const int64_t n = ptr[rows];
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < cap; p += (int64_t)gridDim.x * blockDim.x)
     flag[p] = (p < n && (p == 0 || col[p] != col[p - 1] || rkey[p] != rkey[p - 1])) ? 1 : 0;
@@ -542,6 +553,7 @@ __global__ void __launch_bounds__(256) run_write(const int32_t* __restrict__ u, 
                                                  int32_t* __restrict__ ucol, int32_t* __restrict__ upos,
                                                  uint32_t* __restrict__ ckey, uint32_t* __restrict__ udst,
                                                  uint32_t* __restrict__ uval) {
+  pdl_begin();
   constexpr int kRounds = 4;  // positions per thread, a block apart, their loads in flight together
   const int64_t n = ptr[rows];
   for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x * kRounds + threadIdx.x; p0 <= n;
@@ -582,6 +594,7 @@ __global__ void __launch_bounds__(256) run_write(const int32_t* __restrict__ u, 
 __global__ void run_finish(const int32_t* __restrict__ u, const int32_t* __restrict__ upos,
                            const int32_t* __restrict__ ptr, int64_t rows, int32_t* __restrict__ ucnt,
                            int32_t* __restrict__ uptr) {
+  pdl_begin();
   const int64_t U = u[ptr[rows]];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < U; k += stride) ucnt[k] = upos[k + 1] - upos[k];
@@ -595,6 +608,7 @@ __global__ void run_finish(const int32_t* __restrict__ u, const int32_t* __restr
 // *invalid when that is given.  n_dev, if given, holds n on the device.
 __global__ void row_ptr_from_keys(const uint32_t* __restrict__ keys, int64_t n, const int32_t* __restrict__ n_dev,
                                   int64_t rows, int32_t* __restrict__ ptr, int32_t* __restrict__ invalid) {
+  pdl_begin();
   if (n_dev) n = *n_dev;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= n;
        p += (int64_t)gridDim.x * blockDim.x) {
@@ -608,6 +622,7 @@ __global__ void row_ptr_from_keys(const uint32_t* __restrict__ keys, int64_t n, 
 // Out-runs of every node over all relations leaving its type (the length of its node-major row), from
 // the CSC row pointers over runs.
 __global__ void node_out_counts(const int32_t* __restrict__ cptr, GraphMeta m, int32_t* __restrict__ cnt) {
+  pdl_begin();
   __shared__ int64_t cbase[kMaxRels];  // CSC row of the type's node 0 in relation r, minus the type offset
   __shared__ int32_t rsrc[kMaxRels];
   if (threadIdx.x < kMaxRels) {
@@ -638,6 +653,7 @@ struct PackBits {
 __global__ void __launch_bounds__(256) row_pack(const int32_t* __restrict__ mrow, const int32_t* __restrict__ mbase,
                                                 const int32_t* __restrict__ csr_ptr, int64_t rows, GraphMeta m,
                                                 PackBits pb, uint32_t* __restrict__ pack) {
+  pdl_begin();
   for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < rows;
        row += (int64_t)gridDim.x * blockDim.x) {
     int r = 0;
@@ -663,6 +679,7 @@ __global__ void __launch_bounds__(256) csc_runs(
     const int32_t* __restrict__ mbase, const int32_t* __restrict__ upos, const int32_t* __restrict__ bptr,
     int32_t* __restrict__ bcol, int32_t* __restrict__ bcnt, int32_t* __restrict__ qlen, int32_t* __restrict__ qstart,
     float* __restrict__ qcoef) {
+  pdl_begin();
   const int64_t U = *n_dev;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < cap; q += (int64_t)gridDim.x * blockDim.x) {
     if (q >= U) {
@@ -711,6 +728,7 @@ __global__ void __launch_bounds__(256) csc_expand(const int32_t* __restrict__ qp
                                                   const int32_t* __restrict__ n_dev,
                                                   const int32_t* __restrict__ csr_eid, int32_t* __restrict__ ccol,
                                                   int32_t* __restrict__ ceid, float* __restrict__ ccoef) {
+  pdl_begin();
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int64_t U = *n_dev, nv = qpos[U];
@@ -775,11 +793,13 @@ __global__ void __launch_bounds__(256) csc_expand(const int32_t* __restrict__ qp
 
 // ptr[r] = pos[ptr[r]]: row pointers over runs become row pointers over edges
 __global__ void run_to_edge_ptr(const int32_t* __restrict__ pos, int64_t rows, int32_t* __restrict__ ptr) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= rows; r += (int64_t)gridDim.x * blockDim.x)
     ptr[r] = pos[ptr[r]];
 }
 
 __global__ void chunk_counts(const int32_t* __restrict__ ptr, int64_t rows, int32_t* __restrict__ cnt) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
        r += (int64_t)gridDim.x * blockDim.x) {
     const int deg = ptr[r + 1] - ptr[r];
@@ -788,6 +808,7 @@ __global__ void chunk_counts(const int32_t* __restrict__ ptr, int64_t rows, int3
 }
 
 __global__ void chunk_fill(const int32_t* __restrict__ ofs, int64_t rows, int32_t* __restrict__ chunk_row) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
        r += (int64_t)gridDim.x * blockDim.x) {
     for (int c = ofs[r]; c < ofs[r + 1]; ++c) chunk_row[c] = (int32_t)r;
@@ -816,6 +837,7 @@ __device__ __forceinline__ uint32_t node_mask(const int32_t* __restrict__ csr_pt
 // hist[v * nblk + block] = nodes of the block with mask v
 __global__ void __launch_bounds__(256) order_hist(const int32_t* __restrict__ csr_ptr, TypeRels tr, int64_t n,
                                                   int nblk, int32_t* __restrict__ hist) {
+  pdl_begin();
   __shared__ int32_t h[kMaskValues];
   const int V = 1 << tr.n;
   for (int v = threadIdx.x; v < V; v += blockDim.x) h[v] = 0;
@@ -834,6 +856,7 @@ __global__ void __launch_bounds__(256) order_hist(const int32_t* __restrict__ cs
 __global__ void __launch_bounds__(256) order_scatter(const int32_t* __restrict__ csr_ptr, TypeRels tr, int64_t n,
                                                      int nblk, const int32_t* __restrict__ ofs,
                                                      int32_t* __restrict__ perm) {
+  pdl_begin();
   __shared__ int32_t next[kMaskValues];
   __shared__ int32_t wcnt[8][kMaskValues];
   const int V = 1 << tr.n;
@@ -871,6 +894,7 @@ __global__ void __launch_bounds__(256) order_tiles(const int32_t* __restrict__ c
                                                    const int32_t* __restrict__ perm, int64_t tiles,
                                                    int32_t* __restrict__ tmask, const int32_t* __restrict__ nz_src,
                                                    int32_t* __restrict__ nzero) {
+  pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) *nzero = *nz_src;
   const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;

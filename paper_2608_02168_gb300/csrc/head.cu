@@ -40,6 +40,7 @@ __device__ __forceinline__ float sigmoid_f(float z) {
 // map[idx_a[k]] = idx_b[k] for the k < n overlap pairs whose rows are in range.
 __global__ void head_rep_map(const int32_t* __restrict__ ia, const int32_t* __restrict__ ib, int64_t n_max,
                              const int64_t* __restrict__ n_dev, int64_t rows, int64_t rows_rep, int32_t* __restrict__ map) {
+  pdl_begin();
   int64_t n = n_max;
   if (n_dev) n = max((int64_t)0, min(n_max, *n_dev));
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
@@ -59,6 +60,7 @@ struct HeadSmem {
 // unit gradients, block partials of the row sums.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) head_fwd_simt(HeadFwdArgs a) {
+  pdl_begin();
   using Tl = Tile<T, D>;
   constexpr int CN = Tl::CN, RM = Tl::RM, VEC = Tl::kVec;
   constexpr int LDA = HeadSmem<T, D>::kLda;
@@ -203,6 +205,7 @@ __global__ void __launch_bounds__(256) head_fwd_simt(HeadFwdArgs a) {
 // loss_out[1] = L_BCE = sums[0] / n; loss_out[0] = L_BCE + lambda_CCA * cca[0] (Eq. 20).
 __global__ void head_loss_finish(const float* __restrict__ sums, int64_t n, const float* __restrict__ cca, float lam,
                                  float* __restrict__ loss_out) {
+  pdl_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     const float bce = n > 0 ? sums[0] / (float)n : 0.f;
     loss_out[1] = bce;
@@ -215,6 +218,7 @@ __global__ void head_loss_finish(const float* __restrict__ sums, int64_t n, cons
 // every destination row has one writer.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) head_bwd_dx_simt(HeadBwdArgs a) {
+  pdl_begin();
   using Tl = Tile<T, D>;
   constexpr int CN = Tl::CN, RM = Tl::RM;
   extern __shared__ __align__(16) float smem[];
@@ -266,6 +270,7 @@ __global__ void __launch_bounds__(256) head_bwd_dx_simt(HeadBwdArgs a) {
 // dW1 *= dloss (it holds sum_r h_r^T dA_r); db1, dw2, db2 = dloss * the saved unit sums.
 __global__ void head_grad_finish(float* __restrict__ dW1, const float* __restrict__ sums, float dloss, int d,
                                  float* __restrict__ db1, float* __restrict__ dw2, float* __restrict__ db2) {
+  pdl_begin();
   const int64_t dd = (int64_t)d * d;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dd; i += (int64_t)gridDim.x * blockDim.x) {
     dW1[i] *= dloss;

@@ -81,6 +81,7 @@ __device__ __forceinline__ float warp_sum(float x) {
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     head_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_W, HeadFwdArgs a) {
+  pdl_begin();
   using C = HeadTcCfg<D>;
   constexpr int TPR = D / 8;           // 16-byte pieces per row
   constexpr int RPP = kThreads / TPR;  // rows per gather pass
@@ -293,6 +294,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     head_dx_tc_kernel(const __grid_constant__ CUtensorMap tm_W, const __grid_constant__ CUtensorMap tm_dA,
                       HeadBwdArgs a) {
+  pdl_begin();
   using C = HeadTcCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);

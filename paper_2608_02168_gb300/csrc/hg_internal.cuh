@@ -70,15 +70,35 @@ hg_status device_guard();
 int timing_begin(const char* name, cudaStream_t s);  // -1 when timing is off
 void timing_end(int slot, cudaStream_t s);
 
+// First statement of every kernel.  launch() lets a kernel be set up while the one before it in the stream
+// drains; this returns when that one has completed and its writes are visible.  No thread may touch
+// memory, or leave, before it.
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A launch that may overlap the end of the kernel before it in the stream, up to pdl_begin(): the chains of
+// short kernels gain the set-up time between two of them (step on 10k nodes 1451 -> 1016 us, on 1M nodes
+// 4.83 -> 4.43 ms; fp32 layer on 112k nodes 509 -> 449 us).  No kernel asks for its successor early
+// (griddepcontrol.launch_dependents): the successor's waiting CTAs then take the SMs' shared memory, and with it
+// the L1 of the gather kernels, for their whole run (10M-node layer 10.4 -> 11.3 ms).
 template <typename... KArgs, typename... Args>
 hg_status launch(const char* name, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                  cudaStream_t s, Args&&... args) {
   if (grid.x == 0 || grid.y == 0 || grid.z == 0) return HG_OK;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   int slot = timing_begin(name, s);
-  kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
   timing_end(slot, s);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     set_error("launch of %s failed: %s", name, cudaGetErrorString(e));
     return HG_ERR_CUDA;
   }

@@ -139,6 +139,7 @@ __device__ __forceinline__ float head_sum(float x, int lph) {
 // out[r] = blockdiag(W[r]) (d x d, S blocks of d_h x d_h), or its transpose when transpose != 0.
 template <typename T>
 __global__ void hgt_blockdiag(const T* __restrict__ W, int R, int d, int S, int transpose, T* __restrict__ out) {
+  pdl_begin();
   const int dh = d / S;
   const int64_t total = (int64_t)R * d * d;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
@@ -157,6 +158,7 @@ __global__ void hgt_blockdiag(const T* __restrict__ W, int R, int d, int S, int 
 // out[i][j] = W[j][i] for one d x d matrix per block row.
 template <typename T>
 __global__ void hgt_transpose(const T* __restrict__ W, int count, int d, T* __restrict__ out) {
+  pdl_begin();
   const int64_t total = (int64_t)count * d * d;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t m = q / ((int64_t)d * d);
@@ -177,6 +179,7 @@ __global__ void __launch_bounds__(256) hgt_gemm_simt(const T* __restrict__ A, in
                                                      int64_t ldo, int ocol0, int accumulate,
                                                      const float* __restrict__ scale_ptr, float scale_mul,
                                                      RowMap map) {
+  pdl_begin();
   using Tl = Tile<float, D>;
   constexpr int CN = Tl::CN, RM = Tl::RM;
   __shared__ __align__(16) float As[kBM][kAPad];
@@ -236,6 +239,7 @@ __global__ void __launch_bounds__(256) hgt_gemm_simt(const T* __restrict__ A, in
 template <typename T, int D>
 __global__ void __launch_bounds__(256) hgt_colsum(const T* __restrict__ X, int64_t ldx, int64_t n,
                                                   int64_t rows_per_block, float* __restrict__ part) {
+  pdl_begin();
   constexpr int VEC = VecTraits<T>::kElems, TPR = D / VEC, kRows = 256 / TPR, U = 8;
   __shared__ float red[kRows][D];
   const int g = threadIdx.x % TPR, sub = threadIdx.x / TPR;
@@ -444,6 +448,7 @@ __device__ __forceinline__ void merge_part(float pm, float pl, const float (&pv)
 // runs [64 w, 64 w + 64) of the chunk; warp 0 merges the warps' parts in order.
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kChunkWarps) hgt_fwd_chunks(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   __shared__ float part[kChunkWarps][32][E + 2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S;
@@ -515,6 +520,7 @@ __device__ __forceinline__ void live_node(const HgtArgs& a, int64_t x, int& t, i
 // Lane n KS + k holds the bounds of the claim's node n, relation slot k.
 template <typename T, int D, int KS>
 __global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1) hgt_fwd_nodes(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32, NC = 32 / KS;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
   const int64_t total = live_nodes(a);
@@ -603,6 +609,7 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1
 // on every row of j (the target and source passes read them by row).  One warp per node with in-edges.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) hgt_bwd_dstats(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
   const int64_t total = live_nodes(a), nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -699,6 +706,7 @@ __device__ __forceinline__ void add_warps(float (&v)[N], float (*part)[32][N], i
 
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_dst_chunks(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   __shared__ float part[kChunkWarps][32][E];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S, h = lane / lph;
@@ -751,6 +759,7 @@ __device__ __forceinline__ void add_parts(const float* __restrict__ p, int64_t s
 constexpr int kRowClaim = 8;
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_dst_rows(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S, h = lane / lph;
   const int64_t total = *a.mcount;
@@ -855,6 +864,7 @@ __device__ __forceinline__ void src_edges(const HgtArgs& a, int64_t beg, int64_t
 // Partials of the source pass: lane-major, 2 E floats per lane (dK then dV).
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_src_chunks(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   __shared__ float part[kChunkWarps][32][2 * E];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S;
@@ -884,6 +894,7 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_src_chunks(HgtArgs a
 // dK(i), dV(i) of every node (zeros without out-edges); claims and prefetch as in hgt_bwd_dst_rows.
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_src_nodes(HgtArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
   const T* KV = (const T*)a.KV;
@@ -943,6 +954,7 @@ __global__ void __launch_bounds__(256) hgt_finish(const float* __restrict__ G, c
                                                   const T* __restrict__ W_att, const float* __restrict__ mu, int d,
                                                   int S, float* __restrict__ dW_msg, float* __restrict__ dW_att,
                                                   float* __restrict__ dmu) {
+  pdl_begin();
   __shared__ float red[256];
   const int r = blockIdx.x, dh = d / S;
   const float rs = rsqrtf((float)dh);

@@ -61,6 +61,7 @@ __device__ __forceinline__ int aggregated_claim(int32_t* ctr, int key) {
 // base[v] = v in V_k (a byte per node, so that the edge passes look the partition up instead of hashing
 // both endpoints of every edge)
 __global__ void ob_base(int64_t N, uint64_t part_seed, int K, int k, uint8_t* __restrict__ base) {
+  pdl_begin();
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
     base[v] = part_of(v, part_seed, K) == k;
 }
@@ -108,6 +109,7 @@ __device__ __forceinline__ void for_edges(const int32_t* __restrict__ src, const
 __global__ void __launch_bounds__(256) ob_marks(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                 int64_t E, int64_t N, int64_t B, const uint8_t* __restrict__ base,
                                                 int32_t* deg, int32_t* cand) {
+  pdl_begin();
   for_edges(src, dst, E, N, [&](const int32_t (&s)[kEdgeRounds], const int32_t (&t)[kEdgeRounds],
                                 const bool (&live)[kEdgeRounds]) {
     int32_t ds[kEdgeRounds], dt[kEdgeRounds];
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(256) ob_marks(const int32_t* __restrict__ src,
 __global__ void __launch_bounds__(256) ob_rich(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                int64_t E, int64_t N, int64_t B, const int32_t* __restrict__ deg,
                                                int32_t* rich) {
+  pdl_begin();
   for_edges(src, dst, E, N, [&](const int32_t (&s)[kEdgeRounds], const int32_t (&t)[kEdgeRounds],
                                 const bool (&live)[kEdgeRounds]) {
     bool both[kEdgeRounds];
@@ -149,6 +152,7 @@ __global__ void __launch_bounds__(256) ob_rich(const int32_t* __restrict__ src, 
 // (the loops run whole warps together: lanes past the end take key -1)
 __global__ void ob_degrees(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E, int64_t N,
                            int32_t* __restrict__ deg) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); e0 < E; e0 += stride) {
     const int64_t e = e0 + (threadIdx.x & 31);
@@ -167,6 +171,7 @@ __global__ void ob_degrees(const int32_t* __restrict__ src, const int32_t* __res
 __global__ void ob_fill_lists(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E, int64_t N,
                               const int32_t* __restrict__ deg, const int32_t* __restrict__ ofs,
                               int32_t* __restrict__ fill, int32_t* __restrict__ nbr) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); e0 < E; e0 += stride) {
     const int64_t e = e0 + (threadIdx.x & 31);
@@ -212,6 +217,7 @@ __device__ int warp_h_index(const int32_t* __restrict__ nb, int n) {
 // one warp per node (grid-stride); lists longer than kBigList are left to ob_h_big
 __global__ void ob_h_small(const int32_t* __restrict__ ofs, const int32_t* __restrict__ nbr, int64_t N,
                            int32_t* __restrict__ h) {
+  pdl_begin();
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t v = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < N; v += warps) {
     const int n = ofs[v + 1] - ofs[v];
@@ -234,6 +240,7 @@ constexpr int kRegBins = 8;
 constexpr int kBigThreads = 1024;
 __global__ void __launch_bounds__(kBigThreads) ob_h_big(const int32_t* __restrict__ ofs, const int32_t* __restrict__ nbr,
                                                         int64_t N, int32_t* __restrict__ h) {
+  pdl_begin();
   __shared__ int hist[kCap];
   __shared__ int part[kBigThreads / 32];
   __shared__ int best_s;
@@ -336,6 +343,7 @@ __global__ void __launch_bounds__(kBigThreads) ob_h_big(const int32_t* __restric
 // cand[v] = 1 for v outside V_k with an edge v -> u, u in V_k (Eq. 4)
 __global__ void ob_candidates(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E, int64_t N,
                               const uint8_t* __restrict__ base, int32_t* __restrict__ cand) {
+  pdl_begin();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t s = src[e], t = dst[e];
     if (!edge_ok(s, t, N)) continue;
@@ -355,6 +363,7 @@ struct SelState {
 // C'_k and V_k
 __global__ void ob_eligible(const int32_t* __restrict__ cand, const int32_t* __restrict__ h, int64_t N, int64_t bound,
                             const uint8_t* __restrict__ base, int32_t* __restrict__ elig, SelState* st) {
+  pdl_begin();
   unsigned long long c = 0, ce = 0, cb = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
     const int e = cand[v] && h[v] < bound;
@@ -379,6 +388,7 @@ __global__ void ob_eligible(const int32_t* __restrict__ cand, const int32_t* __r
 // histogram of key digit (key >> shift) & 255 over the eligible nodes whose fixed key bits match
 __global__ void ob_key_hist(const int32_t* __restrict__ elig, int64_t N, int k, uint64_t sample_seed, int shift,
                             const SelState* __restrict__ st, unsigned int* __restrict__ hist) {
+  pdl_begin();
   __shared__ unsigned int hs[256];
   hs[threadIdx.x] = 0;
   __syncthreads();
@@ -394,6 +404,7 @@ __global__ void ob_key_hist(const int32_t* __restrict__ elig, int64_t N, int k, 
 
 // one thread: fixes the next 8 key bits from the histogram (first pass: also M' and the rank)
 __global__ void ob_key_select(unsigned int* __restrict__ hist, int shift, long long M, SelState* st) {
+  pdl_begin();
   if (shift == 24) {
     st->take = (unsigned long long)min((long long)st->count_elig, M);
     st->rank = (long long)st->take - 1;  // the last key taken, 0-based
@@ -418,6 +429,7 @@ __global__ void ob_key_select(unsigned int* __restrict__ hist, int shift, long l
 // eq[v] = eligible with key == the selected threshold key (for the tie ranks)
 __global__ void ob_ties(const int32_t* __restrict__ elig, int64_t N, int k, uint64_t sample_seed,
                         const SelState* __restrict__ st, int32_t* __restrict__ eq) {
+  pdl_begin();
   const bool any = st->take > 0;
   const uint32_t T = st->prefix;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
@@ -428,6 +440,7 @@ __global__ void ob_ties(const int32_t* __restrict__ elig, int64_t N, int k, uint
 __global__ void ob_members(const int32_t* __restrict__ elig, const int32_t* __restrict__ eq_rank, int64_t N, int k,
                            const uint8_t* __restrict__ base, uint64_t sample_seed, const SelState* __restrict__ st,
                            int32_t* __restrict__ member) {
+  pdl_begin();
   const bool any = st->take > 0;
   const uint32_t T = st->prefix;
   const long long rank = st->rank;
@@ -442,6 +455,7 @@ __global__ void ob_members(const int32_t* __restrict__ elig, const int32_t* __re
 }
 
 __global__ void ob_gids(const int32_t* __restrict__ mscan, int64_t N, int64_t* __restrict__ gid_out) {
+  pdl_begin();
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
     if (mscan[v + 1] > mscan[v]) gid_out[mscan[v]] = v;
 }
@@ -449,6 +463,7 @@ __global__ void ob_gids(const int32_t* __restrict__ mscan, int64_t N, int64_t* _
 // keep[e] = both endpoints in V~_k
 __global__ void ob_keep(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E, int64_t N,
                         const int32_t* __restrict__ mscan, int32_t* __restrict__ keep) {
+  pdl_begin();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t s = src[e], t = dst[e];
     keep[e] = edge_ok(s, t, N) && mscan[s + 1] > mscan[s] && mscan[t + 1] > mscan[t];
@@ -459,6 +474,7 @@ __global__ void ob_compact(const int32_t* __restrict__ src, const int32_t* __res
                            const int32_t* __restrict__ rel, int64_t E, const int32_t* __restrict__ mscan,
                            const int32_t* __restrict__ kscan, int32_t* __restrict__ src_out,
                            int32_t* __restrict__ dst_out, int32_t* __restrict__ rel_out, int32_t* __restrict__ eid_out) {
+  pdl_begin();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
     if (kscan[e + 1] == kscan[e]) continue;
     const int32_t p = kscan[e];
@@ -473,6 +489,7 @@ __global__ void ob_compact(const int32_t* __restrict__ src, const int32_t* __res
 __global__ void ob_finish(const int32_t* __restrict__ mscan, const int32_t* __restrict__ kscan, int64_t N, int64_t E,
                           TypeOffsets toff, int num_types, const SelState* __restrict__ st,
                           int64_t* __restrict__ type_offsets_out, int64_t* __restrict__ counts_out) {
+  pdl_begin();
   if (threadIdx.x == 0) {
     counts_out[0] = mscan[N];
     counts_out[1] = (int64_t)st->count_base;

@@ -24,6 +24,7 @@ namespace hg {
 
 template <typename T, int D>
 __global__ void __launch_bounds__(256) proj_fwd_simt(FwdArgs a) {
+  pdl_begin();
   using TL = Tile<T, D>;
   constexpr int RM = TL::RM, CN = TL::CN;
   extern __shared__ __align__(16) float smem[];
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(256) proj_fwd_simt(FwdArgs a) {
 
 template <typename T, int D>
 __global__ void __launch_bounds__(256) proj_bwd_simt(BwdArgs a) {
+  pdl_begin();
   using TL = Tile<T, D>;
   constexpr int RM = TL::RM, CN = TL::CN;
   constexpr int LD = D + 4;
@@ -253,6 +255,7 @@ constexpr int kWR = 32;   // rows per step
 template <typename T, int D>
 __global__ void __launch_bounds__(256) wgrad_partial(const T* __restrict__ X, int64_t x0, const T* __restrict__ Y,
                                                      int64_t y0, int64_t n, float* __restrict__ part, RowMap map) {
+  pdl_begin();
   constexpr int TW = D < kWT ? D : kWT;
   constexpr int TPT = TW / 16;  // outputs per thread per dim
   constexpr int VEC = VecTraits<T>::kElems;
@@ -345,6 +348,7 @@ struct RedOuts {
 };
 __global__ void __launch_bounds__(32 * kRedLanes) reduce_lanes(const float* __restrict__ part, int64_t stride,
                                                              int splits, int64_t count, int64_t seg, RedOuts outs) {
+  pdl_begin();
   __shared__ float red[kRedLanes][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * 32 + lane;
@@ -374,6 +378,7 @@ __global__ void __launch_bounds__(32 * kRedLanes) reduce_lanes(const float* __re
 
 template <typename T>
 __global__ void transpose_square(const T* __restrict__ W, T* __restrict__ Wt, int d, int count) {
+  pdl_begin();
   const int64_t total = (int64_t)count * d * d;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t m = i / ((int64_t)d * d), rc = i % ((int64_t)d * d);

@@ -160,6 +160,7 @@ __device__ __forceinline__ void store_raw(__nv_bfloat16* p, const float* v) {
 constexpr int kIdleRows = 4;
 template <int D>
 __global__ void __launch_bounds__(256) proj_fwd_idle(TcFwdArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, c0 = lane * E;
   const int64_t n = idle_rows(a.nzero);
@@ -892,12 +893,14 @@ __device__ __forceinline__ void proj_fwd_body(const CUtensorMap& tm_Vt, const Tc
 template <int D>
 __global__ void __launch_bounds__(FwdCfg<D>::kThreads, 1)
     proj_fwd_tc(const __grid_constant__ CUtensorMap tm_Vt, TcFwdArgs a) {
+  pdl_begin();
   proj_fwd_body<D, false>(tm_Vt, a);
 }
 
 template <int D>
 __global__ void __launch_bounds__(FwdCfg<D, true>::kThreads, 1)
     proj_fwd_gather_tc(const __grid_constant__ CUtensorMap tm_Vt, TcFwdArgs a) {
+  pdl_begin();
   if constexpr (D == 128) proj_fwd_body<D, true>(tm_Vt, a);
 }
 
@@ -911,6 +914,7 @@ __global__ void __launch_bounds__(256) fuse_weights(const __nv_bfloat16* __restr
                                                     const __nv_bfloat16* __restrict__ W_agg, RelDst rel_dst,
                                                     int num_rels, __nv_bfloat16* __restrict__ V,
                                                     __nv_bfloat16* __restrict__ Vt) {
+  pdl_begin();
   __shared__ double As[32][33];
   __shared__ double Bs[32][33];
   const int r = blockIdx.z, i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
@@ -955,6 +959,7 @@ __global__ void __launch_bounds__(256) wgrad_finish(const float* __restrict__ G,
                                                     const __nv_bfloat16* __restrict__ W_agg, RelDst rel_dst,
                                                     int num_rels, int num_types, float* __restrict__ dW_rel,
                                                     float* __restrict__ dW_agg) {
+  pdl_begin();
   __shared__ float As[32][33];
   __shared__ float Bs[32][33];
   const int z = blockIdx.z, i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
@@ -1021,6 +1026,7 @@ struct LnCfg {
 // column partials part[block] = {sum dU, sum dH_out Xh, sum dH_out} over the block's rows.
 template <int D>
 __global__ void __launch_bounds__(256, LnCfg<D>::kBlocks) ln_act_bwd(TcBwdArgs a) {
+  pdl_begin();
   constexpr int E = D / 32;
   constexpr int kLnRows = LnCfg<D>::kRows;
   __shared__ float red[8][3][D];
@@ -1169,6 +1175,7 @@ struct BwdJobs {
 template <int D>
 __global__ void __launch_bounds__(BwdCfg<D>::kThreads, 1)
     proj_bwd_tc(const __grid_constant__ CUtensorMap tm_dU, const __grid_constant__ CUtensorMap tm_V, TcBwdArgs a) {
+  pdl_begin();
   using C = BwdCfg<D>;
   constexpr int S = C::kStages;
   constexpr int NB = C::kNumAcc;
@@ -1362,6 +1369,7 @@ template <int D>
 __global__ void __launch_bounds__(WgCfg<D>::kThreads, 1)
     wgrad_tc(const __grid_constant__ RelMaps tm_X, const __grid_constant__ CUtensorMap tm_Y, int R, int S,
              int64_t n, int chunks_per_split, float* __restrict__ part, int* __restrict__ status) {
+  pdl_begin();
   using C = WgCfg<D>;
   constexpr int NB = D / 64;  // 64-wide column blocks of Y
   extern __shared__ uint8_t smem_raw[];
@@ -1490,6 +1498,7 @@ __global__ void __launch_bounds__(WgRowsCfg<D>::kThreads, 1)
     wgrad_rows_tc(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __restrict__ Y,
                   const int32_t* __restrict__ mlist, const int32_t* __restrict__ mbase, int rel, int64_t row0,
                   int64_t ny, float* __restrict__ part, int* __restrict__ status) {
+  pdl_begin();
   using C = WgRowsCfg<D>;
   constexpr int S = C::kStages;
   constexpr uint32_t kLag = S - 1;
@@ -1653,6 +1662,7 @@ __global__ void __launch_bounds__(WgGatherCfg::kThreads, 1)
                     const int32_t* __restrict__ long_ofs, const __nv_bfloat16* __restrict__ Y,
                     const int32_t* __restrict__ mlist, const int32_t* __restrict__ mbase, int rel, int64_t row0,
                     int64_t ny, float* __restrict__ part, int* __restrict__ status) {
+  pdl_begin();
   constexpr int D = 128;
   using C = WgGatherCfg;
   constexpr int S = C::kStages;

@@ -63,6 +63,7 @@ enum : int { kDense = 0, kGather = 1, kScatter = 2 };
 template <int D, int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
     rows_gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_A, const __grid_constant__ CUtensorMap tm_B, GArgs p) {
+  pdl_begin();
   using C = GCfg<D>;
   constexpr int CW = D / kGroups;
   extern __shared__ uint8_t smem_raw[];

@@ -66,6 +66,7 @@ hg_status make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint
 // nothing arrives at (no copy, store or MMA is in flight) and records the give-up in the status
 // word, as every tensor-core kernel does when one of its waits runs out.
 __global__ void selftest_bounded_wait(uint32_t polls, int* status) {
+  pdl_begin();
   __shared__ uint64_t bar;
   if (threadIdx.x == 0) {
     tc::mbar_init(&bar, 1);

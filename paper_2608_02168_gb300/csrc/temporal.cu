@@ -34,6 +34,7 @@ template <typename TA, typename TB, int D>
 __global__ void __launch_bounds__(256) tgemm_simt(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B,
                                                   int64_t ldb, int bcol0, int K, int64_t n, float* __restrict__ out,
                                                   int64_t ldo, int ocol0, int accumulate) {
+  pdl_begin();
   bcol0 += blockIdx.y * D;
   ocol0 += blockIdx.y * D;
   using Tl = Tile<float, D>;
@@ -79,6 +80,7 @@ __device__ __forceinline__ float sigm(float x) {
 template <typename T, int D>
 __global__ void temporal_attn_simt(const float* __restrict__ U, const T* __restrict__ C, const T* __restrict__ rvec,
                                    int64_t n, int w, T* __restrict__ Ht, float* __restrict__ a_out) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (v >= n) return;
@@ -115,6 +117,7 @@ __global__ void temporal_attn_simt(const float* __restrict__ U, const T* __restr
 template <typename T, int D>
 __global__ void temporal_gru_simt(const float* __restrict__ Gi, const float* __restrict__ Gh, const T* __restrict__ Ht,
                                   const T* __restrict__ b_i, const T* __restrict__ b_h, int64_t n, T* __restrict__ out) {
+  pdl_begin();
   const int64_t total = n * D;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = q / D;
@@ -137,6 +140,7 @@ __global__ void temporal_gru_bwd_simt(const float* __restrict__ Gi, const float*
                                       const T* __restrict__ Ht, const T* __restrict__ b_i, const T* __restrict__ b_h,
                                       const T* __restrict__ dOut, int64_t n, T* __restrict__ dgi,
                                       T* __restrict__ dgh_n, float* __restrict__ dh) {
+  pdl_begin();
   const int64_t total = n * D;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = q / D;
@@ -171,6 +175,7 @@ __global__ void __launch_bounds__(256) temporal_attn_bwd_simt(const float* __res
                                                               const float* __restrict__ dHt, int64_t n, int w,
                                                               int64_t nodes_per_block, T* __restrict__ dpre,
                                                               float* __restrict__ dr_part) {
+  pdl_begin();
   constexpr int PL = D / 32;
   __shared__ float red[8][D];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -220,6 +225,7 @@ __global__ void __launch_bounds__(256) temporal_attn_bwd_simt(const float* __res
 template <typename T, int D>
 __global__ void temporal_colsum(const T* __restrict__ X0, const T* __restrict__ X1, const T* __restrict__ X2,
                                 int64_t n, int64_t rows_per_block, float* __restrict__ part) {
+  pdl_begin();
   const T* Xs[3] = {X0, X1, X2};
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
   for (int q = threadIdx.x; q < 3 * D; q += blockDim.x) {
@@ -234,6 +240,7 @@ __global__ void temporal_colsum(const T* __restrict__ X0, const T* __restrict__ 
 // out[i][j] = W[j][i] for a rows x cols matrix W (storage type).
 template <typename T>
 __global__ void temporal_transpose(const T* __restrict__ W, int rows, int cols, T* __restrict__ out) {
+  pdl_begin();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < rows * cols; q += gridDim.x * blockDim.x) {
     const int i = q / rows, j = q % rows;
     out[q] = W[(int64_t)j * cols + i];
@@ -242,6 +249,7 @@ __global__ void temporal_transpose(const T* __restrict__ W, int rows, int cols, 
 
 // dst[row][g D + c] = scale * G[row][c] (a d x d block into a d x 3d gradient).
 __global__ void temporal_place(const float* __restrict__ G, int d, int g, float* __restrict__ dst) {
+  pdl_begin();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < d * d; q += gridDim.x * blockDim.x) {
     const int row = q / d, c = q % d;
     dst[(int64_t)row * 3 * d + g * d + c] = G[q];
@@ -250,6 +258,7 @@ __global__ void temporal_place(const float* __restrict__ G, int d, int g, float*
 
 template <typename T>
 __global__ void temporal_to_storage(const float* __restrict__ x, int64_t count, T* __restrict__ out) {
+  pdl_begin();
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < count; q += (int64_t)gridDim.x * blockDim.x)
     out[q] = from_f32<T>(x[q]);
 }

@@ -139,6 +139,7 @@ struct TAttnArgs {
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     temporal_attn_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ CUtensorMap tm_Wa, TAttnArgs p) {
+  pdl_begin();
   using C = TCfg<D>;
   constexpr int CW = D / kGroups;  // columns of a warp's group
   extern __shared__ uint8_t smem_raw[];
@@ -272,6 +273,7 @@ template <int D, bool kBwd>
 __global__ void __launch_bounds__(kThreads, 1)
     temporal_gru_tc(const __grid_constant__ CUtensorMap tm_X, const __grid_constant__ CUtensorMap tm_Ht,
                     const __grid_constant__ CUtensorMap tm_Wi, const __grid_constant__ CUtensorMap tm_Wh, TGruArgs p) {
+  pdl_begin();
   using C = TCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -442,6 +444,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     temporal_dx_tc(const __grid_constant__ CUtensorMap tm_dG, const __grid_constant__ CUtensorMap tm_Wi,
                    const __grid_constant__ CUtensorMap tm_Wh, TDxArgs p) {
+  pdl_begin();
   using C = TCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -547,6 +550,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     temporal_attn_bwd_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ CUtensorMap tm_Wa,
                          TAttnBwdArgs p) {
+  pdl_begin();
   using C = TCfg<D>;
   constexpr int CW = D / kGroups;
   extern __shared__ uint8_t smem_raw[];
@@ -734,6 +738,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // dst[row][g D + c] = G[c][row]: the transposed block of a gate (d x d into d x 3d).
 __global__ void temporal_place_t(const float* __restrict__ G, int d, int g, float* __restrict__ dst) {
+  pdl_begin();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < d * d; q += gridDim.x * blockDim.x) {
     const int row = q / d, c = q % d;
     dst[(int64_t)row * 3 * d + g * d + c] = G[(int64_t)c * d + row];
@@ -743,6 +748,7 @@ __global__ void temporal_place_t(const float* __restrict__ G, int d, int g, floa
 // db_i = [s_r, s_z, s_n], db_h = [s_r, s_z, s_hn] from the four column sums s (4 d).
 __global__ void temporal_bias_finish(const float* __restrict__ s, int d, float* __restrict__ db_i,
                                      float* __restrict__ db_h) {
+  pdl_begin();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < 3 * d; q += gridDim.x * blockDim.x) {
     db_i[q] = s[q];
     db_h[q] = q < 2 * d ? s[q] : s[q + d];

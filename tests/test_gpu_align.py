@@ -159,7 +159,7 @@ def test_align_bf16_device_count_far_below_capacity(d):
     assert hg.hg_device_status() == 0
 
 
-@pytest.mark.parametrize("d,n", [(64, 152 * 128 + 1), (128, 40_001), (256, 2 * 152 * 128 - 1)])
+@pytest.mark.parametrize("d,n", [(64, 152 * 128 + 1), (128, 2 * 152 * 128 - 1), (256, 152 * 128 + 1)])
 def test_align_bf16_gradient_ctas_take_several_tiles(d, n):
     """More 128-row tiles than SMs, a ragged last one: each gradient CTA loops over tiles, both views."""
     need_gpu()

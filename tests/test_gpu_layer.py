@@ -138,8 +138,8 @@ def test_relu_near_zero_pre_activations_bf16():
         assert np.linalg.norm(x - y) / np.linalg.norm(y) <= 2e-2, k
 
 
-@pytest.mark.parametrize("d,ln", [(64, True), (128, False), (128, True), (256, True)])
-@pytest.mark.parametrize("idle", [0, 127, 128, 129, 400])
+@pytest.mark.parametrize("d,ln,idle", [(128, True, 0), (128, True, 127), (128, False, 128), (128, True, 129),
+                                       (128, True, 400), (64, True, 128), (64, False, 400), (256, True, 129)])
 def test_nodes_without_in_edges_bf16(d, ln, idle):
     """`idle` of 400 users and every risk node without in-edges: whole 128-row tiles of them leave the projection."""
     need_gpu()
