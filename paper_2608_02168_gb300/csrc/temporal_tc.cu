@@ -336,16 +336,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (!ok) record_device_error(p.status, kErrTimeout);
   }
+  constexpr int CW = D / kGroups;
+  const int q = warp & 3, cg = warp >> 2;
+  const int row = q * 32 + lane;
+  const int64_t r = r0 + row;
+  uint4 graw[CW / 8];  // backward: the row's upstream gradient, in flight while the products are awaited
+  if (kBwd)
+#pragma unroll
+    for (int c0 = 0; c0 < CW; c0 += 8)
+      graw[c0 / 8] = r < p.n ? ld16(p.dOut + r * D + cg * CW + c0) : make_uint4(0u, 0u, 0u, 0u);
   ok = __syncthreads_and(ok);
   if (ok && !mbar_wait(&bars[2], 0)) {
     record_device_error(p.status, kErrTimeout);
     ok = false;
   }
   fence_after_sync();
-  constexpr int CW = D / kGroups;
-  const int q = warp & 3, cg = warp >> 2;
-  const int row = q * 32 + lane;
-  const int64_t r = r0 + row;
   const bool live = ok && r < p.n;
   const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
 #pragma unroll
@@ -357,14 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_ld8(trow + 2 * D + c, anx);
     tmem_ld8(trow + 3 * D + c, anh);
     tile_row8(Himg, row, c, h);
-    if (kBwd) {
-      if (live) {
-        unpack(ld16(p.dOut + r * D + c), g, __nv_bfloat16());
-      } else {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) g[t] = 0.f;
-      }
-    }
+    if (kBwd) unpack(graw[c0 / 8], g, __nv_bfloat16());
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
       const int col = c + t;
@@ -499,15 +497,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (!ok) record_device_error(p.status, kErrTimeout);
   }
+  constexpr int CW = D / kGroups;
+  const int q = warp & 3, cg = warp >> 2, lane = tid & 31;
+  const int64_t r = r0 + q * 32 + lane;
+  uint4 draw[CW / 8];  // the row's z dH^t, in flight while the products are awaited
+#pragma unroll
+  for (int c0 = 0; c0 < CW; c0 += 8)
+    draw[c0 / 8] = r < p.n ? ld16(p.dh + r * D + cg * CW + c0) : make_uint4(0u, 0u, 0u, 0u);
   ok = __syncthreads_and(ok);
   if (ok && !mbar_wait(&bars[2], 0)) {
     record_device_error(p.status, kErrTimeout);
     ok = false;
   }
   fence_after_sync();
-  constexpr int CW = D / kGroups;
-  const int q = warp & 3, cg = warp >> 2, lane = tid & 31;
-  const int64_t r = r0 + q * 32 + lane;
   const bool live = ok && r < p.n;
   const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
 #pragma unroll
@@ -518,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_ld8(trow + D + c, h);
     if (live) {
       float d0[8];
-      unpack(ld16(p.dh + r * D + c), d0, __nv_bfloat16());
+      unpack(draw[c0 / 8], d0, __nv_bfloat16());
 #pragma unroll
       for (int t = 0; t < 8; ++t) h[t] += d0[t];
       st16(p.dX + r * D + c, pack(x, __nv_bfloat16()));
