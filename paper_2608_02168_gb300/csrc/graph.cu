@@ -74,10 +74,17 @@ __device__ __forceinline__ void scan_store4(int32_t* out, int64_t i, int64_t n, 
   if (i + 3 < n) out[i + 3] = v.w;
 }
 
-// sums[tile] = sum of the tile's kScanTile items (warp w: items tile * kScanTile + w * 512 ..)
+// sums[tile] = sum of the tile's kScanTile items (warp w: items tile * kScanTile + w * 512 ..).  n_dev, if
+// given, holds the item count on the device (at most n; tiles past it sum to 0 and are not read).
 __global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __restrict__ in, int64_t n,
+                                                                const int32_t* __restrict__ n_dev,
                                                                 int32_t* __restrict__ sums) {
   pdl_begin();
+  if (n_dev) n = *n_dev;
+  if ((int64_t)blockIdx.x * kScanTile >= n) {
+    if (threadIdx.x == 0) sums[blockIdx.x] = 0;
+    return;
+  }
   __shared__ int wt[kScanThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool vec = (reinterpret_cast<uintptr_t>(in) & 15) == 0;
@@ -100,10 +107,19 @@ __global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __
 }
 
 // Exclusive scan of one tile plus tile_off[tile] (nullptr: a single tile starting at 0); the last
-// tile also writes out[n] = the grand total.  out may equal in.
+// tile also writes out[n] = the grand total.  out may equal in.  With n_dev (n the capacity), the scan ends
+// at the device count: out[*n_dev] = the grand total, and nothing past it is read or written.
 __global__ void __launch_bounds__(kScanThreads) scan_tiles(const int32_t* in, int32_t* out, int64_t n,
+                                                            const int32_t* __restrict__ n_dev,
                                                             const int32_t* __restrict__ tile_off) {
   pdl_begin();
+  bool last = blockIdx.x == gridDim.x - 1;  // the tile that writes the grand total
+  if (n_dev) {
+    n = *n_dev;
+    const int64_t t0 = (int64_t)blockIdx.x * kScanTile;
+    if (t0 > n || (t0 == n && n > 0)) return;
+    last = n <= t0 + kScanTile;
+  }
   __shared__ int wt[kScanThreads / 32 + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
@@ -147,7 +163,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles(const int32_t* in, in
     scan_store4(out, seg + 128 * j + 4 * lane, n, o, vec);
     carry += __shfl_sync(0xffffffffu, incl, 31);
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = wt[kScanThreads / 32];
+  if (last && threadIdx.x == 0) out[n] = wt[kScanThreads / 32];
 }
 
 size_t scan_scratch_bytes(int64_t n) {
@@ -159,22 +175,23 @@ size_t scan_scratch_bytes(int64_t n) {
   return b + 256;
 }
 
-hg_status exclusive_scan(const int32_t* in, int32_t* out, int64_t n, void* scratch, cudaStream_t s) {
+hg_status exclusive_scan(const int32_t* in, int32_t* out, int64_t n, void* scratch, cudaStream_t s,
+                         const int32_t* n_dev) {
   if (n <= 0) {
     if (n == 0) HG_CUDA(cudaMemsetAsync(out, 0, sizeof(int32_t), s));
     return HG_OK;
   }
   if (n <= kScanTile)
-    return launch("scan_tiles", scan_tiles, dim3(1), dim3(kScanThreads), 0, s, in, out, n,
+    return launch("scan_tiles", scan_tiles, dim3(1), dim3(kScanThreads), 0, s, in, out, n, n_dev,
                   (const int32_t*)nullptr);
   const int64_t tiles = ceil_div(n, kScanTile);
   int32_t* sums = static_cast<int32_t*>(scratch);
   char* rest = static_cast<char*>(scratch) + align_up((size_t)(tiles + 1) * sizeof(int32_t));
   HG_TRY(launch("scan_tile_sums", scan_tile_sums, dim3((unsigned)tiles), dim3(kScanThreads), 0, s,
-                in, n, sums));
+                in, n, n_dev, sums));
   HG_TRY(exclusive_scan(sums, sums, tiles, rest, s));
   return launch("scan_tiles", scan_tiles, dim3((unsigned)tiles), dim3(kScanThreads), 0, s, in, out,
-                n, (const int32_t*)sums);
+                n, n_dev, (const int32_t*)sums);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -531,12 +548,25 @@ __global__ void compact_rows(const int32_t* __restrict__ flag, int64_t rows, int
 // ---------------------------------------------------------------------------------------------
 // flag[p] = 1 where a run starts (a new row or a new source) for p < ptr[rows]; 0 up to cap (the
 // capacity the scan runs over).
-__global__ void run_flags(const uint32_t* __restrict__ rkey, const int32_t* __restrict__ col,
-                          const int32_t* __restrict__ ptr, int64_t rows, int64_t cap, int32_t* __restrict__ flag) {
+// Four positions per thread, as 16-byte vectors (the arrays are 256-byte aligned).
+__global__ void __launch_bounds__(256) run_flags(const uint32_t* __restrict__ rkey, const int32_t* __restrict__ col,
+                                                 const int32_t* __restrict__ ptr, int64_t rows, int64_t cap,
+                                                 int32_t* __restrict__ flag) {
   pdl_begin();
   const int64_t n = ptr[rows];
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < cap; p += (int64_t)gridDim.x * blockDim.x)
-    flag[p] = (p < n && (p == 0 || col[p] != col[p - 1] || rkey[p] != rkey[p - 1])) ? 1 : 0;
+  for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; p < cap;
+       p += (int64_t)gridDim.x * blockDim.x * 4) {
+    if (p + 4 <= n) {
+      const uint4 k = *reinterpret_cast<const uint4*>(rkey + p);
+      const int4 c = *reinterpret_cast<const int4*>(col + p);
+      const bool first = p == 0 || c.x != col[p - 1] || k.x != rkey[p - 1];
+      *reinterpret_cast<int4*>(flag + p) = make_int4(first, c.y != c.x || k.y != k.x, c.z != c.y || k.z != k.y,
+                                                     c.w != c.z || k.w != k.z);
+    } else {
+      for (int64_t q = p; q < min(p + 4, cap); ++q)
+        flag[q] = (q < n && (q == 0 || col[q] != col[q - 1] || rkey[q] != rkey[q - 1])) ? 1 : 0;
+    }
+  }
 }
 
 constexpr uint32_t kOneEdge = 0x80000000u;
@@ -605,17 +635,34 @@ __global__ void run_finish(const int32_t* __restrict__ u, const int32_t* __restr
 // Position p owns the rows k with key[p-1] < k <= key[p] (key[-1] = -1, key[n] = rows), so every
 // entry is written exactly once and empty rows get the position of the next non-empty one.  The
 // owner of k = rows also writes n - ptr[rows] (the positions with keys past the last row) to
-// *invalid when that is given.  n_dev, if given, holds n on the device.
+// *invalid when that is given.  n_dev, if given, holds n on the device.  Four keys per thread.
 __global__ void row_ptr_from_keys(const uint32_t* __restrict__ keys, int64_t n, const int32_t* __restrict__ n_dev,
                                   int64_t rows, int32_t* __restrict__ ptr, int32_t* __restrict__ invalid) {
   pdl_begin();
   if (n_dev) n = *n_dev;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= n;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t lo = p == 0 ? 0 : (int64_t)keys[p - 1] + 1;
-    const int64_t hi = p == n ? rows : min((int64_t)keys[p], rows);
-    for (int64_t k = lo; k <= hi; ++k) ptr[k] = (int32_t)p;
-    if (invalid && lo <= rows && rows <= hi) *invalid = (int32_t)(n - p);
+  for (int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; p0 <= n;
+       p0 += (int64_t)gridDim.x * blockDim.x * 4) {
+    uint32_t k[4];
+    if (p0 + 4 <= n) {
+      const uint4 v = *reinterpret_cast<const uint4*>(keys + p0);
+      k[0] = v.x;
+      k[1] = v.y;
+      k[2] = v.z;
+      k[3] = v.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) k[i] = p0 + i < n ? keys[p0 + i] : 0u;
+    }
+    int64_t lo = p0 == 0 ? 0 : (int64_t)keys[p0 - 1] + 1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t p = p0 + i;
+      if (p > n) break;
+      const int64_t hi = p == n ? rows : min((int64_t)k[i], rows);
+      for (int64_t r = lo; r <= hi; ++r) ptr[r] = (int32_t)p;
+      if (invalid && lo <= rows && rows <= hi) *invalid = (int32_t)(n - p);
+      lo = (int64_t)k[i] + 1;
+    }
   }
 }
 
@@ -669,23 +716,19 @@ __global__ void __launch_bounds__(256) row_pack(const int32_t* __restrict__ mrow
 // The runs in CSC order (sorted keys, uval and destination of each; cptr: CSC row pointers over
 // runs).  Writes the node-major list of out-runs used by the backward aggregation -- node i's row holds,
 // relation by relation (ascending) and in CSC order within a relation, the compact row of each run's
-// target and its multiplicity -- and, per run, its length (0 up to cap, for the scan that follows), its
+// target and its multiplicity -- and, per run, its length, its
 // first CSR position (or uval, for one edge), and
 // 1 / deg_r(destination).
 __global__ void __launch_bounds__(256) csc_runs(
     const uint32_t* __restrict__ skey, const uint32_t* __restrict__ srun, const uint32_t* __restrict__ sdst,
-    const int32_t* __restrict__ n_dev, int64_t cap, const int32_t* __restrict__ cptr, GraphMeta m,
+    const int32_t* __restrict__ n_dev, const int32_t* __restrict__ cptr, GraphMeta m,
     const int32_t* __restrict__ csr_ptr, const uint32_t* __restrict__ pack, PackBits pb,
     const int32_t* __restrict__ mbase, const int32_t* __restrict__ upos, const int32_t* __restrict__ bptr,
     int32_t* __restrict__ bcol, int32_t* __restrict__ bcnt, int32_t* __restrict__ qlen, int32_t* __restrict__ qstart,
     float* __restrict__ qcoef) {
   pdl_begin();
   const int64_t U = *n_dev;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < cap; q += (int64_t)gridDim.x * blockDim.x) {
-    if (q >= U) {
-      qlen[q] = 0;
-      continue;
-    }
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < U; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t key = skey[q];
     const int64_t j = sdst[q];
     const uint32_t run = srun[q];
@@ -1109,7 +1152,7 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)rows), (const uint32_t*)L.sort.vals2[r1],
                       (const uint32_t*)L.sort.vals[r1], (const uint32_t*)L.sort.keys[r1], r1, s, &res,
                       (uint32_t*)L.csr_eid, (uint32_t*)L.csr_col));
-    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(g), dim3(256), 0, s, (const uint32_t*)L.sort.keys[res],
+    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, (const uint32_t*)L.sort.keys[res],
                   E, (const int32_t*)nullptr, rows, L.csr_ptr, L.invalid));
   }
   // non-empty CSR rows (the rows the mean layer stores) and their compact numbering
@@ -1125,7 +1168,7 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     int32_t* flag = reinterpret_cast<int32_t*>(L.sort.keys[o]);
     int32_t* u = reinterpret_cast<int32_t*>(L.sort.vals[o]);
     const uint32_t* rkey = L.sort.keys[res];
-    HG_TRY(launch("run_flags", run_flags, dim3(grid_for(E)), dim3(256), 0, s, rkey, (const int32_t*)L.csr_col,
+    HG_TRY(launch("run_flags", run_flags, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, rkey, (const int32_t*)L.csr_col,
                   (const int32_t*)L.csr_ptr, rows, E, flag));
     HG_TRY(exclusive_scan(flag, u, E, L.sort.scan_scratch, s));
     HG_TRY(launch("run_write", run_write, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, (const int32_t*)u,
@@ -1139,7 +1182,7 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     HG_TRY(radix_sort(L.sort, E, nruns, bit_width((uint64_t)crows), (const uint32_t*)L.sort.ckeys,
                       (const uint32_t*)L.sort.vals[res], (const uint32_t*)L.sort.vals2[res], res, s, &x));
     const uint32_t *skey = L.sort.keys[x], *srun = L.sort.vals[x], *sdst = L.sort.vals2[x];
-    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(g), dim3(256), 0, s, skey, E, nruns, crows, L.csc_ptr,
+    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, skey, E, nruns, crows, L.csc_ptr,
                   (int32_t*)nullptr));
     // node-major rows: out-runs per node over its relations, their scan, then the runs
     HG_TRY(launch("node_out_counts", node_out_counts, dim3(grid_for(N)), dim3(256), 0, s, (const int32_t*)L.csc_ptr,
@@ -1153,11 +1196,11 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     for (int r = 0; r < num_rels; ++r) pb.deg[r] = 32 - bit_width((uint64_t)(m.row_base[r + 1] - m.row_base[r]));
     HG_TRY(launch("row_pack", row_pack, dim3(grid_for(rows)), dim3(256), 0, s, (const int32_t*)L.mrow,
                   (const int32_t*)L.mbase, (const int32_t*)L.csr_ptr, rows, m, pb, L.row_pack));
-    HG_TRY(launch("csc_runs", csc_runs, dim3(g), dim3(256), 0, s, skey, srun, sdst, nruns, E,
+    HG_TRY(launch("csc_runs", csc_runs, dim3(g), dim3(256), 0, s, skey, srun, sdst, nruns,
                   (const int32_t*)L.csc_ptr, m, (const int32_t*)L.csr_ptr, (const uint32_t*)L.row_pack, pb,
                   (const int32_t*)L.mbase, (const int32_t*)L.run_pos, (const int32_t*)L.bagg_ptr, L.bagg_col,
                   L.bagg_cnt, qpos, qstart, qcoef));
-    HG_TRY(exclusive_scan(qpos, qpos, E, L.sort.scan_scratch, s));
+    HG_TRY(exclusive_scan(qpos, qpos, E, L.sort.scan_scratch, s, nruns));
     HG_TRY(launch("csc_expand", csc_expand, dim3((unsigned)std::min<int64_t>(ceil_div(E, kExpand * 8), 152 * 8)),
                   dim3(256), 0, s, (const int32_t*)qpos, (const int32_t*)qstart, (const float*)qcoef,
                   sdst, nruns,

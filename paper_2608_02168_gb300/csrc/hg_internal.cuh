@@ -263,8 +263,10 @@ __device__ __forceinline__ int node_type_of(const GraphMeta& m, int64_t node) {
 // ---------------------------------------------------------------------------------------------
 // internal entry points implemented in the other translation units
 // ---------------------------------------------------------------------------------------------
-// exclusive scan of n int32 counts into out[0..n] (out[n] = total); in may equal out.
+// exclusive scan of n int32 counts into out[0..n] (out[n] = total); in may equal out.  With n_dev, of the
+// first *n_dev (device, at most n) counts: out[0..*n_dev].
 size_t scan_scratch_bytes(int64_t n);
-hg_status exclusive_scan(const int32_t* in, int32_t* out, int64_t n, void* scratch, cudaStream_t s);
+hg_status exclusive_scan(const int32_t* in, int32_t* out, int64_t n, void* scratch, cudaStream_t s,
+                         const int32_t* n_dev = nullptr);
 
 }  // namespace hg

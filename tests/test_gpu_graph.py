@@ -169,11 +169,11 @@ def test_25_bit_row_keys():
     compare_node_order(hg, G, ref, offs, rels)
 
 
-@pytest.mark.parametrize("E", [1, 31, 32, 33, 1023, 1024, 1025, 2048, 2049, 12289])
+@pytest.mark.parametrize("E", [1, 31, 32, 33, 1023, 1024, 1025, 2048, 2049, 4096, 8192, 12289])
 @pytest.mark.parametrize("kind", ["one pair", "pairs twice", "distinct", "mixed"])
 def test_runs_of_parallel_edges(E, kind):
     """The CSC arrays are written run by run: one run of every edge, runs of two, runs of one edge (whose id rides with
-    its key) and a mix, at the edges of a warp's 32 runs, its 1024 positions and a sort tile."""
+    its key) and a mix, at the edges of a warp's 32 runs, its 1024 positions, a sort tile and a scan tile."""
     need_gpu()
     hg = lib()
     offs = np.array([0, 4000, 4100], np.int64)
