@@ -955,24 +955,24 @@ __global__ void __launch_bounds__(256) hgt_finish(const float* __restrict__ G, c
                                                   int S, float* __restrict__ dW_msg, float* __restrict__ dW_att,
                                                   float* __restrict__ dmu) {
   pdl_begin();
-  __shared__ float red[256];
+  __shared__ double red[256];  // the sum's terms cancel: in fp32 its rounding was most of dmu's error
   const int r = blockIdx.x, dh = d / S;
   const float rs = rsqrtf((float)dh);
   const float c = mu[r] * rs;
-  float acc = 0.f;
+  double acc = 0.0;
   for (int q = threadIdx.x; q < S * dh * dh; q += blockDim.x) {
     const int s = q / (dh * dh), a = (q / dh) % dh, b = q % dh;
     const int64_t gi = (int64_t)r * d * d + (int64_t)(s * dh + a) * d + s * dh + b;
     dW_msg[(int64_t)r * S * dh * dh + q] = G[gi];
     dW_att[(int64_t)r * S * dh * dh + q] = c * Gq[gi];
-    acc = fmaf(to_f32(W_att[(int64_t)r * S * dh * dh + q]), Gq[gi], acc);
+    acc = fma((double)to_f32(W_att[(int64_t)r * S * dh * dh + q]), (double)Gq[gi], acc);
   }
   red[threadIdx.x] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
-    float t = 0.f;
+    double t = 0.0;
     for (int k = 0; k < (int)blockDim.x; ++k) t += red[k];
-    dmu[r] = t * rs;
+    dmu[r] = (float)(t * (double)rs);
   }
 }
 
