@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(256) csc_expand(const int32_t* __restrict__ qp
 #pragma unroll
         for (int k = 0; k < kRounds; ++k) {
           if (p + 32 * k >= wend) break;
-          const int x = (int)p + 32 * k + lane;
+          const int64_t x = p + 32 * k + lane;  // past wend it may exceed 31 bits
           int i = 0;  // lanes whose run ends at or before x: the index of x's run
 #pragma unroll
           for (int b = 16; b > 0; b >>= 1)
@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(256) csc_expand(const int32_t* __restrict__ qp
         }
 #pragma unroll
         for (int k = 0; k < kRounds; ++k) {
-          const int x = (int)p + 32 * k + lane;
+          const int64_t x = p + 32 * k + lane;
           if (x < wend) {
             ceid[x] = id[k];
             ccol[x] = t[k];
