@@ -49,10 +49,12 @@ struct TCfg {
   static constexpr int kA = NB * kABlk;  // 128 x D bf16
 };
 
-// Logistic function.  exp(-x) = inf gives 0, as it should; the divide without its branches (2 ulp), for the
-// gate epilogues are bound by their instructions (about 90 per element forward, half of all issue slots of
-// the kernel): 1M rows, d = 128, forward 648 -> 522 us, backward 1304 -> 1181 us.
-__device__ __forceinline__ float sigm(float x) { return __fdividef(1.f, 1.f + expf(-x)); }
+// Logistic function, to the last bit for either sign (e^x / (1 + e^x) below zero, which stays above 0 until e^x
+// itself underflows); one divide, by a value in [1, 2].
+__device__ __forceinline__ float sigm(float x) {
+  const float e = expf(-fabsf(x));
+  return (x >= 0.f ? 1.f : e) / (1.f + e);
+}
 
 // Sum over the warp of v[L], returned to lane L (fixed butterfly order).
 __device__ __forceinline__ float tsum32(float (&v)[32]) {

@@ -76,6 +76,29 @@ def test_temporal_matches_oracle(dt, d, n, w):
     check(X, C, p, dOut, dt, out, dX, g)
 
 
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+@pytest.mark.parametrize("pre", [-20.0, -86.0, -87.5, -90.0])
+def test_nearly_closed_update_gate(dt, pre):
+    """z = sigmoid(pre) is tiny, not 0: with zero weights and candidate n = 0 the output is z h alone, h = 2^100."""
+    need_gpu()
+    hg = lib()
+    n, d, w = 130, 64, 1
+    X, C, p = problem(1, n, d, w, dt)
+    for k in ("W_i", "W_h", "b_i", "b_h"):
+        p[k][:] = 0
+    p["b_i"][d:2 * d] = p["b_h"][d:2 * d] = pre / 2  # exact in bf16
+    C[:] = np.float32(2.0**100)
+    p["Wa"][:] = 0
+    dOut = np.ones((n, d), np.float32)
+    out, dX, g = temporal_gpu(hg, X, C, p, dOut, dt, w)
+    # exp(pre) in fp32 is subnormal below pre = -87.3: two of its last bits, 2^-148, are allowed beside TOL
+    z, h = 1 / (1 + np.exp(-np.float64(pre))), 2.0**100
+    assert np.abs(out - z * h).max() <= TOL[dt] * z * h + 2.0**-148 * h
+    db = n * h * z * (1 - z)  # dL/dz sums (h - n) z (1 - z) over the rows
+    for k in ("b_i", "b_h"):
+        assert np.abs(g[k][d:2 * d] - db).max() <= TOL[dt] * db + n * h * 2.0**-148, k
+
+
 def test_temporal_empty_and_deterministic():
     need_gpu()
     hg = lib()
