@@ -347,6 +347,10 @@ __device__ __forceinline__ int64_t claim(int32_t* counter, int n) {
   return __shfl_sync(kAll, c, 0);
 }
 
+// What the exponents of a part with maximum m are taken from: a part whose scores are all -inf has sum and
+// values 0 (exp(-inf - -inf) would make it, and every row merged from it, NaN).
+__device__ __forceinline__ float exp_base(float m) { return m == -INFINITY ? 0.f : m; }
+
 // Online softmax over a batch of nb runs of one row (per lane: its head's running maximum m and sum l;
 // the value accumulators are rescaled when the maximum grows).
 template <typename T, int E, int NACC>
@@ -366,10 +370,11 @@ __device__ __forceinline__ void online_batch(const float (&sc)[kBatch], const fl
       for (int e = 0; e < E; ++e) acc[k][e] *= so;
     m = mn;
   }
+  const float mb = exp_base(m);
 #pragma unroll
   for (int u = 0; u < kBatch; ++u) {
     if (u >= nb) break;
-    const float p = w[u] * expf(sc[u] - m);  // w runs with this score
+    const float p = w[u] * expf(sc[u] - mb);  // w runs with this score
     l += p;
     float f[E];
     v[u].get(f);
@@ -435,7 +440,7 @@ __device__ __forceinline__ void merge_part(float pm, float pl, const float (&pv)
       for (int e = 0; e < E; ++e) acc[k][e] *= so;
     m = mn;
   }
-  const float sp = expf(pm - m);
+  const float sp = expf(pm - exp_base(m));
   l = fmaf(pl, sp, l);
 #pragma unroll
   for (int k = 0; k < NACC; ++k)
@@ -590,7 +595,7 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1
           fwd_edges<T, D, KS>(a, b, e, win[k], qf, lph, m, l, acc, k);
         }
       }
-      const float inv = l > 0.f ? 1.f / l : 0.f;
+      const float inv = l > 0.f ? 1.f / l : NAN;  // (every node here has a run: 0 only if all its scores are -inf)
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
         if (row[k] < 0) continue;

@@ -1,6 +1,8 @@
 """Attention layer (Heterogeneous Graph Transformer, Eq. 6-11) forward and backward through the C
 ABI against the oracle, on seeded power-law graphs whose in- and out-degree hubs exceed the hub
 degree (so the chunked paths of all three edge passes run), ragged type sizes and isolated nodes."""
+from types import SimpleNamespace
+
 import numpy as np
 import pytest
 import torch
@@ -110,4 +112,44 @@ def test_hgt_few_stored_rows(dtype, rows):
         if k == "mu":
             scale = np.linalg.norm(p["W_att"][0]) * np.linalg.norm(gref["W_att"][0]) / abs(p["mu"][0])
         assert np.abs(gr[k] - gref[k]).max() <= TOL[dtype] * scale, k
+    assert hg.hg_device_status() == 0
+
+
+def test_scores_of_minus_infinity():
+    """Parts of a row whose scores all overflow to -inf: the first four runs of a short row, a warp's 64 runs and a
+    whole chunk of hub rows.  They weigh 0 beside the row's finite scores, forward and backward."""
+    need_gpu()
+    hg = lib()
+    sp = hgsynth.spec("tiny-10k", n_user=2000, n_risk=10, num_rels=2, d=64)
+    rng = np.random.default_rng(5)
+    rels, offs, d = ((0, 1), (0, 0)), np.array([0, 2000, 2010], np.int64), 64
+    # the rows' sources in run order, masked ones marked
+    rows = [(range(96, 104), range(96, 100)), (range(0, 100), range(64, 100)), (range(200, 900), range(200, 712)),
+            (range(1000, 1700), range(1512, 1700))]
+    src = np.concatenate([np.array(s) for s, _ in rows]).astype(np.int32)
+    dst = np.concatenate([np.full(len(s), 2000 + k) for k, (s, _) in enumerate(rows)]).astype(np.int32)
+    w = SimpleNamespace(spec=sp, graph={"src": src, "dst": dst, "rel": np.zeros(src.size, np.int32),
+                                        "type_offsets": offs, "rels": rels},
+                        X=rng.standard_normal((2010, d)).astype(np.float32),
+                        dH_top=rng.standard_normal((2010, d)).astype(np.float32))
+    p = hgsynth.make_hgt_params(sp, 1)
+    w.X[:, 0] = 0
+    for _, masked in rows:
+        w.X[list(masked), 0] = -1e30
+    for k in ("W_K", "W_Q", "W_V", "W_att"):  # feature 0 reaches the keys alone, where it meets a query of 1e30
+        p[k][..., 0, :] = 0
+        p[k][..., :, 0] = 0
+    p["W_K"][:, 0, 0] = p["W_att"][..., 0, 0] = 1
+    p["b_K"][:, 0], p["b_Q"][:, 0] = 0, 1e30
+    g = w.graph
+    args = (g["src"], g["dst"], g["rel"], offs, rels, p, w.X)
+    with np.errstate(under="ignore"):
+        ref, _ = OH.hgt_forward(*args, 1, layernorm=False)
+        dref, gref = OH.hgt_backward(*args, w.dH_top, 1, layernorm=False)
+    out, dH, gr = run_gpu(hg, w, p, 1, False, w.dH_top)
+    assert np.isfinite(out).all() and np.isfinite(dH).all()
+    assert relerr(out[2000:], ref[2000:]) <= TOL["f32"]
+    assert relerr(dH[:, 1:], dref[:, 1:]) <= TOL["f32"]
+    for k in ("W_V", "W_msg", "W_agg", "b_V", "b_agg"):
+        assert relerr(gr[k], gref[k]) <= TOL["f32"], k
     assert hg.hg_device_status() == 0
