@@ -802,27 +802,28 @@ __global__ void __launch_bounds__(256) csc_expand(const int32_t* __restrict__ qp
       const float ccf = coef;
       window(q0 + 32);  // the next runs, in flight meanwhile
       const int64_t wend = min(p1, (int64_t)__shfl_sync(kAll, cend, 31));
+      const uint32_t xend = (uint32_t)wend;
       for (; p < wend; p += 32 * kRounds) {
         int id[kRounds], t[kRounds];
         float c[kRounds];
 #pragma unroll
         for (int k = 0; k < kRounds; ++k) {
           if (p + 32 * k >= wend) break;
-          const int64_t x = p + 32 * k + lane;  // past wend it may exceed 31 bits
+          const uint32_t x = (uint32_t)p + 32 * k + lane;  // past the end, up to 127 above 31 bits
           int i = 0;  // lanes whose run ends at or before x: the index of x's run
 #pragma unroll
           for (int b = 16; b > 0; b >>= 1)
-            if (__shfl_sync(kAll, cend, i + b - 1) <= x) i += b;
+            if ((uint32_t)__shfl_sync(kAll, cend, i + b - 1) <= x) i += b;
           const int s0 = __shfl_sync(kAll, cstart, i), f0 = __shfl_sync(kAll, cfirst, i);
           t[k] = __shfl_sync(kAll, cdst, i);
           c[k] = __shfl_sync(kAll, ccf, i);
           id[k] = s0 & ~(int)kOneEdge;
-          if (s0 >= 0 && x < wend) id[k] = __ldg(csr_eid + s0 + (x - f0));
+          if (s0 >= 0 && x < xend) id[k] = __ldg(csr_eid + s0 + (x - (uint32_t)f0));
         }
 #pragma unroll
         for (int k = 0; k < kRounds; ++k) {
-          const int64_t x = p + 32 * k + lane;
-          if (x < wend) {
+          const uint32_t x = (uint32_t)p + 32 * k + lane;
+          if (x < xend) {
             ceid[x] = id[k];
             ccol[x] = t[k];
             ccoef[x] = c[k];
