@@ -959,7 +959,10 @@ static int64_t order_tiles_cap(int64_t N) { return N / kProjTileRows + kMaxTypes
 
 // Rows above kHubDegree hold sum ceil(deg / kChunkEdges) <= E / kChunkEdges + E / (kHubDegree + 1)
 // chunks (each such row adds at most one partial chunk); +2 covers the integer floors.
-static int64_t chunk_cap(int64_t E) { return E / kChunkEdges + E / (kHubDegree + 1) + 2; }
+// Chunks of `rows` rows with E runs in all: the whole ones, and one more per row above the hub degree.
+static int64_t chunk_cap(int64_t E, int64_t rows) {
+  return E / kChunkEdges + std::min(E / (kHubDegree + 1), rows) + 2;
+}
 // a long row has more than kFuseRuns runs, each of at least one edge
 static int64_t long_cap(int64_t E) { return E / (kFuseRuns + 1) + 1; }
 
@@ -994,12 +997,12 @@ static size_t carve_graph(void* ws, int64_t E, int64_t rows, int64_t crows, int6
   L->agg_col = c.take<int32_t>(Ea);
   L->agg_cnt = c.take<int32_t>(Ea);
   L->agg_chunk_ofs = c.take<int32_t>(rows + 1);
-  L->agg_chunk_row = c.take<int32_t>(chunk_cap(E));
+  L->agg_chunk_row = c.take<int32_t>(chunk_cap(E, rows));
   L->bagg_ptr = c.take<int32_t>(N + 1);
   L->bagg_col = c.take<int32_t>(Ea);
   L->bagg_cnt = c.take<int32_t>(Ea);
   L->bagg_chunk_ofs = c.take<int32_t>(N + 1);
-  L->bagg_chunk_row = c.take<int32_t>(chunk_cap(E));
+  L->bagg_chunk_row = c.take<int32_t>(chunk_cap(E, N));
   L->mrow = c.take<int32_t>(rows + 1);
   L->mlist = c.take<int32_t>(rows + 1);
   L->mbase = c.take<int32_t>(kMaxRels + 1);
@@ -1246,8 +1249,8 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
   gh->num_edges = E;
   gh->csr_rows = rows;
   gh->csc_rows = crows;
-  gh->chunk_cap_csr = chunk_cap(E);
-  gh->chunk_cap_node = chunk_cap(E);
+  gh->chunk_cap_csr = chunk_cap(E, rows);
+  gh->chunk_cap_node = chunk_cap(E, N);
   gh->stream = s;
   gh->csr_ptr = L.csr_ptr;
   gh->csr_col = L.csr_col;

@@ -1006,7 +1006,7 @@ struct HgtLayout {
   void* dV;       // N x d
   void* Qbuf;     // N x d: Q (forward), recomputed in the backward
   void* dQ;       // N x d
-  float* part;    // chunk partials
+  float* part;    // chunk partials (L.agg_part)
   float* cs;      // column-sum partials
   float* Gw;      // R x d x d
   float* Gq;      // R x d x d
@@ -1030,7 +1030,10 @@ void carve_hgt(const hg_graph* g, const hg_hgt_params* p, void* saved, void* scr
   const int64_t N = m.type_off[m.num_types];
   const size_t dd = (size_t)d * d;
   size_t ls = 0, lk = 0;
-  carve_layer(g, d, p->dtype, saved, scratch, &H->L, &ls, &lk);
+  // the chunk partials are the layer's: the projection has none of its own
+  const int64_t pc = std::max<int64_t>(g->chunk_cap_csr * (2 * S + d), g->chunk_cap_node * 2 * d);
+  carve_layer(g, d, p->dtype, saved, scratch, &H->L, &ls, &lk, false, pc);
+  H->part = H->L.agg_part;
   Carve s(saved), k(scratch);
   s.used = align_up(ls);
   k.used = align_up(lk);
@@ -1049,8 +1052,6 @@ void carve_hgt(const hg_graph* g, const hg_hgt_params* p, void* saved, void* scr
   H->dV = k.take<char>((size_t)std::max<int64_t>(N, 1) * d * b);
   H->Qbuf = k.take<char>((size_t)std::max<int64_t>(N, 1) * d * b);
   H->dQ = k.take<char>((size_t)std::max<int64_t>(N, 1) * d * b);
-  const int64_t pc = std::max<int64_t>(g->chunk_cap_csr * (2 * S + d), g->chunk_cap_node * 2 * d);
-  H->part = k.take<float>((size_t)std::max<int64_t>(pc, 1));
   H->cs = k.take<float>((size_t)152 * 8 * d);
   H->Gw = k.take<float>(m.num_rels * dd);
   H->Gq = k.take<float>(m.num_rels * dd);

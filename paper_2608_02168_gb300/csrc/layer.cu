@@ -69,7 +69,7 @@ void timing_end(int slot, cudaStream_t s) {
 static size_t elem_size(hg_dtype dt) { return dt == HG_F32 ? 4 : 2; }
 
 void carve_layer(const hg_graph* g, int d, hg_dtype dt, void* saved, void* scratch, LayerLayout* L,
-                 size_t* saved_bytes, size_t* scratch_bytes, bool fused) {
+                 size_t* saved_bytes, size_t* scratch_bytes, bool fused, int64_t part_floats) {
   const GraphMeta& m = g->meta;
   const int64_t N = m.type_off[m.num_types];
   const size_t b = elem_size(dt);
@@ -89,7 +89,7 @@ void carve_layer(const hg_graph* g, int d, hg_dtype dt, void* saved, void* scrat
     L->V = s.take<char>(2 * m.num_rels * dd * b);  // hi and lo halves of each fused weight
     L->Vt = s.take<char>(2 * m.num_rels * dd * b);
   }
-  L->agg_part = k.take<float>((size_t)std::max(g->chunk_cap_csr, g->chunk_cap_node) * d);
+  L->agg_part = k.take<float>((size_t)(part_floats ? part_floats : std::max(g->chunk_cap_csr, g->chunk_cap_node) * d));
   L->work = k.take<int32_t>(64);
   L->dY = k.take<char>((size_t)N * d * b);
   L->dU = k.take<char>((size_t)N * d * b);
@@ -100,7 +100,7 @@ void carve_layer(const hg_graph* g, int d, hg_dtype dt, void* saved, void* scrat
   const int cblocks = (int)std::max<int64_t>(ceil_div(max_rows, 64), std::min<int64_t>(ceil_div(max_rows, 8), 152 * 8));
   L->cpart = k.take<float>((size_t)cblocks * 3 * d);
   const int wsplits = std::max(wgrad_splits(max_rows), wgrad_tc_splits(max_rows, d));
-  L->wpart = k.take<float>((size_t)wsplits * dd * (tc ? wgrad_tc_max_rels(d) : 1));
+  L->wpart = k.take<float>((size_t)wsplits * dd);
   L->rtmp = k.take<float>(std::max(reduce_tmp_floats(cblocks, d), reduce_tmp_floats(wsplits, (int64_t)dd)));
   if (tc) {
     L->G = k.take<float>(m.num_rels * dd);

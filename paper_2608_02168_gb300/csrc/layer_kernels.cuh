@@ -120,8 +120,6 @@ hg_status tc_proj_forward(int d, const TcFwdArgs& a, const void* M, int64_t m_ro
 hg_status tc_proj_forward_gather(int d, const TcFwdArgs& a, const void* Vt, int num_rels, cudaStream_t s);
 hg_status tc_ln_act_backward(int d, const TcBwdArgs& a, int* blocks, cudaStream_t s);
 hg_status tc_proj_backward(int d, const TcBwdArgs& a, const void* V, int num_rels, cudaStream_t s);
-// outs[r] = X[x0[r] .. x0[r]+n)^T Y[y0 .. y0+n) for r < R (R <= wgrad_tc_max_rels(d)); the R
-// products share the loads of Y.  part: R x wgrad_tc_splits(n, d) x d x d floats.
 // out = G_r = M^T dU over relation `rel`'s stored rows: compact rows mbase[rel] .. mbase[rel + 1]
 // of M (m_rows rows in all) paired with dU rows mlist[k] - row0 (of the type's n rows at y0).
 hg_status tc_weight_grad_rows(int d, const void* M, int64_t m_rows, const int32_t* mlist, const int32_t* mbase, int rel,
@@ -132,9 +130,10 @@ hg_status tc_weight_grad_rows(int d, const void* M, int64_t m_rows, const int32_
 hg_status tc_weight_grad_gather(int d, const hg_graph* g, const void* H, const void* Mlong, int rel, int64_t row0,
                                 const void* dU, int64_t y0, int64_t n, float* part, float* out, float* tmp,
                                 cudaStream_t s);
+// outs[r] = X[x0[r] .. x0[r]+n)^T Y[y0 .. y0+n) for r < R (at most WgCfg<d>::kMaxR); the R products share
+// the loads of Y.  part: R x wgrad_tc_splits(n, d) x d x d floats.
 hg_status tc_weight_grad(int d, const void* X, const int64_t* x0, int R, const void* Y, int64_t y0, int64_t n,
                          float* part, float* const* outs, float* tmp, cudaStream_t s);
-int wgrad_tc_max_rels(int d);
 hg_status tc_wgrad_finish(int d, const float* G, const void* W_rel, const void* W_agg, RelDst rd, int num_rels,
                           int num_types, float* dW_rel, float* dW_agg, cudaStream_t s);
 int wgrad_tc_splits(int64_t n, int d);
@@ -204,9 +203,10 @@ struct LayerLayout {
   void* WrelT;    // scratch (fp32 storage only): R x d x d
   void* WaggT;    // scratch (fp32 storage only): T x d x d
 };
-// fused: the mean layer without stored relation means (L->M null; L->Mlong holds the long rows')
+// fused: the mean layer without stored relation means (L->M null; L->Mlong holds the long rows');
+// part_floats: the size of agg_part (0: what the mean aggregation needs)
 void carve_layer(const hg_graph* g, int d, hg_dtype dt, void* saved, void* scratch, LayerLayout* L,
-                 size_t* saved_bytes, size_t* scratch_bytes, bool fused = false);
+                 size_t* saved_bytes, size_t* scratch_bytes, bool fused = false, int64_t part_floats = 0);
 RelDst rel_dst_of(const GraphMeta& m);
 // Eq. 7 and Eq. 11 from the relation rows in L.M (bias, activation, residual, optional LayerNorm).
 // L.M holds the non-empty CSR rows only, in the graph's compact order.

@@ -2132,7 +2132,6 @@ hg_status tc_weight_grad_gather(int d, const hg_graph* g, const void* H, const v
                                 cudaStream_t s) {
   HG_TC_DISPATCH(d, tc_wgrad_gather_t, g, H, Mlong, rel, row0, dU, y0, n, part, out, tmp, s);
 }
-int wgrad_tc_max_rels(int d) { return d == 64 ? WgCfg<64>::kMaxR : (d == 128 ? WgCfg<128>::kMaxR : WgCfg<256>::kMaxR); }
 hg_status tc_wgrad_finish(int d, const float* G, const void* W_rel, const void* W_agg, RelDst rd, int num_rels,
                           int num_types, float* dW_rel, float* dW_agg, cudaStream_t s) {
   HG_TC_DISPATCH(d, tc_finish_t, G, W_rel, W_agg, rd, num_rels, num_types, dW_rel, dW_agg, s);

@@ -161,3 +161,27 @@ def test_nodes_without_in_edges_bf16(d, ln, idle):
     for k in ("W_rel", "W_agg", "b_agg") + (("ln_gamma", "ln_beta") if ln else ()):
         assert np.abs(host(grads[k]) - gref[k]).max() <= TOL["bf16"] * np.abs(gref[k]).max(), k
     assert hg.hg_device_status() == 0
+
+
+@pytest.mark.parametrize("kind", ["mean", "attention"])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+def test_scratch_for_hub_partials_follows_the_rows(kind, dt):
+    """400 rows and a million edges: room for a chunk per 512 runs and one more per row, once, in both layers."""
+    need_gpu()
+    hg = lib()
+    n, d, heads, E = 400, 64, 4, 1_000_000
+    offs, rels = np.array([0, n, n], np.int64), ((0, 0),)
+    sp = hgsynth.spec("tiny-10k", n_user=n, n_risk=0, num_rels=1, d=d, dtype=dt)
+    size = {}
+    for edges in (1, E):
+        e = dev(np.zeros(edges, np.int32))
+        G = hg.hg_build_csr(e, e, e, offs, rels)
+        if kind == "mean":
+            P = layer_params(hg, hgsynth.make_layer_params(sp, 0), dt)
+            size[edges] = hg.hg_layer_workspace_size(G, P)[1]
+        else:
+            p = hgsynth.make_hgt_params(sp, heads)
+            P = hg.HgtParams({k: dev(v, torch.float32 if k == "mu" else tdtype(dt)) for k, v in p.items()}, heads)
+            size[edges] = hg.hg_hgt_workspace_size(G, P)[1]
+    partial = d if kind == "mean" else max(2 * heads + d, 2 * d)
+    assert size[E] - size[1] <= (E // 512 + n) * partial * 4 + 256
