@@ -146,9 +146,9 @@ def test_node_order_with_eight_relations_into_one_type():
 
 
 def test_25_bit_row_keys():
-    # three relations into a 6M-node type: 18M CSR rows and 18M CSC rows (25-bit keys, four radix
-    # passes each, the last on a 1-bit digit), 23-bit node ids; bit-exact against the oracle on 2M
-    # random edges with parallel edges
+    # three relations into a 6M-node type: 18M CSR rows and 18M CSC rows (25-bit keys, three radix
+    # passes each, of 9, 8 and 8 bits), 23-bit node ids (8, 8 and 7 bits); bit-exact against the
+    # oracle on 2M random edges with parallel edges
     need_gpu()
     hg = lib()
     n0 = 6_000_000
@@ -194,4 +194,28 @@ def test_runs_of_parallel_edges(E, kind):
     src, dst, rel = src[p], dst[p], rel[p]
     G, bad = gpu_csr(hg, src, dst, rel, offs, rels)
     assert bad == 0
+    compare_layout(hg, G, oracle.build_csr(src, dst, rel, offs, rels), rels)
+
+
+LARGE = 2 * 152 * 512 * 12  # edges from which the sort takes tiles of 6144 items, two CTAs on each SM
+
+
+@pytest.mark.parametrize("E,nodes,pairs", [
+    # the switch of tile size, a ragged last tile; few distinct pairs: nearly all tiles of the runs' sort are empty
+    (LARGE - 1, 50_000, None), (LARGE, 50_000, None), (LARGE + 1, 50_000, None), (LARGE + 1, 50_000, 300),
+    # node and row keys of 9, 10, 18 and 19 bits, where the number of passes changes
+    (20_001, 510, None), (20_001, 511, None), (20_001, 512, None), (20_001, 262_143, None), (20_001, 262_144, None),
+    (LARGE + 5, 511, None), (LARGE + 5, 512, None), (LARGE + 5, 262_144, None)])
+def test_sort_sizes_and_key_widths(E, nodes, pairs):
+    need_gpu()
+    hg = lib()
+    offs, rels = np.array([0, nodes, nodes], np.int64), ((0, 0),)
+    rng = np.random.default_rng(E + nodes)
+    k = np.arange(E) if pairs is None else rng.integers(0, pairs, E)
+    src = np.random.default_rng(1).integers(0, nodes, E)[k]
+    dst = np.minimum((np.random.default_rng(2).pareto(1.0, E)[k] * nodes / 100).astype(np.int64), nodes - 1)
+    rel = np.zeros(E, np.int64)
+    src[:7] = -1  # dropped edges
+    G, bad = gpu_csr(hg, src, dst, rel, offs, rels)
+    assert bad == 7
     compare_layout(hg, G, oracle.build_csr(src, dst, rel, offs, rels), rels)

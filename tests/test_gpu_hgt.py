@@ -153,3 +153,50 @@ def test_scores_of_minus_infinity():
     for k in ("W_V", "W_msg", "W_agg", "b_V", "b_agg"):
         assert relerr(gr[k], gref[k]) <= TOL["f32"], k
     assert hg.hg_device_status() == 0
+
+
+@pytest.mark.parametrize("into,dtype,d,heads", [(5, "f32", 64, 4), (5, "bf16", 128, 4), (8, "f32", 128, 8),
+                                                (8, "bf16", 64, 2), (8, "bf16", 256, 4)])
+def test_more_than_four_relations_into_a_type(into, dtype, d, heads):
+    """Five to eight relations into the users (a claim holds four nodes, eight relation slots each): every subset of
+    them occurs among the nodes, rows of one run, hub rows of one and of two chunks, live nodes not a multiple of 4."""
+    need_gpu()
+    hg = lib()
+    nu, nr = 1201, 150
+    rels = tuple((k % 2, 0) for k in range(into)) + ((0, 1),) * (into < 8)
+    sp = hgsynth.spec("tiny-10k", n_user=nu, n_risk=nr, num_rels=len(rels), d=d, dtype=dtype)
+    rng = np.random.default_rng(into * d)
+    offs, sizes = np.array([0, nu, nu + nr], np.int64), (nu, nr)
+    live = rng.permutation(nu)[: 4 * 220 + 3]
+    src, dst, rel = [], [], []
+    for r, (a, b) in enumerate(rels):
+        if b == 0:  # target k has relation r when bit r of its place is set, and one to six edges then
+            at = np.repeat(live[((np.arange(live.size) % (1 << into)) >> r) & 1 == 1], 3)
+            at = np.concatenate([at, rng.choice(at, 2 * at.size)])
+        else:
+            at = offs[1] + rng.integers(0, nr, 400)
+        src.append(offs[a] + rng.integers(0, sizes[a], at.size))
+        dst.append(at)
+        rel.append(np.full(at.size, r))
+    hub = live[(1 << into) - 1]  # has every relation
+    for r, runs in ((0, 700), (1, 120), (2, 97)):
+        k = min(runs, sizes[rels[r][0]])
+        src.append(offs[rels[r][0]] + rng.permutation(sizes[rels[r][0]])[:k])
+        dst.append(np.full(k, hub))
+        rel.append(np.full(k, r))
+    g = {"src": np.concatenate(src).astype(np.int32), "dst": np.concatenate(dst).astype(np.int32),
+         "rel": np.concatenate(rel).astype(np.int32), "type_offsets": offs, "rels": rels}
+    assert np.unique(g["dst"][g["dst"] < nu]).size % 4
+    st = hgsynth.bf16_round if dtype == "bf16" else (lambda x: x)
+    w = SimpleNamespace(spec=sp, graph=g, X=st(rng.standard_normal((nu + nr, d)).astype(np.float32)),
+                        dH_top=st(rng.standard_normal((nu + nr, d)).astype(np.float32)))
+    p = hgsynth.make_hgt_params(sp, heads, bias_margin=BF16_RELU_MARGIN if dtype == "bf16" else None)
+    out, dH, gr = run_gpu(hg, w, p, heads, True, w.dH_top)
+    args = (g["src"], g["dst"], g["rel"], offs, rels, p, w.X)
+    ref, _ = OH.hgt_forward(*args, heads, layernorm=True)
+    dref, gref = OH.hgt_backward(*args, w.dH_top, heads, layernorm=True)
+    assert relerr(out, ref) <= TOL[dtype], relerr(out, ref)
+    assert relerr(dH, dref) <= TOL[dtype], relerr(dH, dref)
+    for k in KEYS:
+        assert relerr(gr[k], gref[k]) <= TOL[dtype], (k, relerr(gr[k], gref[k]))
+    assert hg.hg_device_status() == 0
