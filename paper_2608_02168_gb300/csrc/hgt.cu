@@ -320,13 +320,12 @@ struct HgtArgs {
 //  - the bounds of everything claimed are loaded at once, one (node, relation) or row per lane;
 //  - a row's run entries are loaded 32 at a time, one per lane, and handed out by shuffles, and the
 //    first window is loaded together with the row's own slices;
-//  - hub chunks are a whole CTA each, a warp per eighth, merged in warp order.
-// 1M nodes, 20M edges (3.2M runs), d = 128 bf16: fwd nodes 2.01 -> 0.61 ms, target pass 2.32 -> 0.49 ms, source
-// pass 1.77 -> 0.58 ms, the three chunk passes 1.31 -> 0.65 ms; the layer forward + backward 11.05 -> 6.60 ms.
+//  - a hub chunk is a whole CTA, an even share of its runs per warp, merged in warp order.
+// 1M nodes, 20M edges (3.2M runs), d = 128 bf16, against a warp per node and per chunk: forward nodes 1.98 ->
+// 0.37 ms, target pass 2.28 -> 0.31 ms, source pass 1.73 -> 0.40 ms, the three chunk passes 1.28 -> 0.96 ms.
 constexpr int kBatch = 4;        // runs of a row in flight per warp
 constexpr int kEdgeWarps = 4;    // warps per CTA of the node and row kernels
 constexpr int kChunkWarps = 8;   // warps per hub chunk
-constexpr int kChunkPart = kChunkEdges / kChunkWarps;
 constexpr unsigned kAll = 0xffffffffu;
 
 // One window of run entries: lane l holds entry base + l.
@@ -339,6 +338,57 @@ struct RunWindow {
     cnt = e < end ? __ldg(n + e) : 0;
   }
 };
+
+// Runs per warp of a chunk of n runs: an even share in whole batches.  (With 64 runs per warp a chunk of
+// 110 left six of eight warps idle: 50k nodes with 110 distinct in-neighbours each, d = 64 fp32, forward +
+// backward 7.14 ms, with even shares 3.12 ms; the 1M-node graph above, 1.06 -> 0.96 ms for the chunk passes.)
+__device__ __forceinline__ int64_t chunk_share(int64_t n) {
+  return (n + kChunkWarps * kBatch - 1) / (kChunkWarps * kBatch) * kBatch;
+}
+
+// Rows of more runs than this go through the chunk kernels; nchunks = the chunks of all rows above kHubDegree
+// runs.  Up to kManyChunks of them the hub rows are the exception that would hold a warp while the others are
+// done.  From there on they are the work itself, enough of it to keep every warp busy, and a warp per row saves
+// the CTA's barriers and the partials: degrees around 110 on 50k nodes, chunks / warps 2.96 / 2.13 ms; on
+// 5k nodes of skewed degrees (zipf 0.8, 100 edges per node) 0.87 / 0.98 ms.  Rows of one chunk (at most
+// kChunkEdges runs) can go either way.  With the line at 256 / 384 / 512 runs: degrees around 300 6.11 / 4.73 /
+// 4.74 ms, around 450 8.10 / 8.56 / 6.96 ms, but 100k nodes of zipf 0.8, 100 edges per node, 5.31 / 5.44 / 5.70 ms (5.13
+// with all in chunks): a late claim of long rows is that kernel's tail.
+constexpr int kManyChunks = 16384, kHubMany = 384;
+static_assert(kHubMany <= kChunkEdges, "rows of one chunk only");
+__device__ __forceinline__ int hub_runs(int nchunks) { return nchunks < kManyChunks ? kHubDegree : kHubMany; }
+
+// Calls f(c, row, beg, end) for this CTA's chunks of the rows above hub_runs runs, the whole CTA together.
+template <typename F>
+__device__ __forceinline__ void for_chunks(const int32_t* __restrict__ ptr, const int32_t* __restrict__ chunk_ofs,
+                                           const int32_t* __restrict__ chunk_row, int nchunks, F f) {
+  const int lane = threadIdx.x & 31, hub = hub_runs(nchunks);
+  for (int64_t w0 = blockIdx.x; w0 < nchunks; w0 += 32 * (int64_t)gridDim.x) {
+    const int64_t x = w0 + lane * (int64_t)gridDim.x;  // a chunk per lane
+    int row = 0, beg = 0, end = 0;
+    bool take = false;
+    if (x < nchunks) {
+      row = chunk_row[x];
+      const int b = ptr[row], e = ptr[row + 1];
+      take = e - b > hub;
+      beg = b + (int)(x - chunk_ofs[row]) * kChunkEdges;
+      end = e - beg < kChunkEdges ? e : beg + kChunkEdges;
+    }
+    for (unsigned todo = __ballot_sync(kAll, take); todo; todo &= todo - 1) {
+      const int i = __ffs(todo) - 1;
+      f((int)(w0 + i * (int64_t)gridDim.x), __shfl_sync(kAll, row, i), (int64_t)__shfl_sync(kAll, beg, i),
+        (int64_t)__shfl_sync(kAll, end, i));
+    }
+  }
+}
+
+// Items per claim: `most`, or fewer when every warp would not get four claims of them (1000 nodes with 110
+// in-neighbours each, d = 64 fp32: 629 -> 344 us; two claims instead of four cost 5 % at 50k nodes).
+__device__ __forceinline__ int claim_size(int64_t total, int most) {
+  const int64_t nwarps = (int64_t)gridDim.x * kEdgeWarps;
+  while (most > 1 && total < 4 * nwarps * most) most >>= 1;
+  return most;
+}
 
 // claims `n` consecutive items
 __device__ __forceinline__ int64_t claim(int32_t* counter, int n) {
@@ -449,8 +499,8 @@ __device__ __forceinline__ void merge_part(float pm, float pl, const float (&pv)
       for (int e = 0; e < E; ++e) acc[k][e] = fmaf(sp, pv[e], acc[k][e]);
 }
 
-// One CTA per chunk of a hub row: (m, l, unnormalised value sum) of the chunk's runs.  Warp w takes
-// runs [64 w, 64 w + 64) of the chunk; warp 0 merges the warps' parts in order.
+// One CTA per chunk of a hub row: (m, l, unnormalised value sum) of the chunk's runs, an even share per
+// warp; warp 0 merges the warps' parts in order.
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kChunkWarps) hgt_fwd_chunks(HgtArgs a) {
   pdl_begin();
@@ -459,11 +509,8 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_fwd_chunks(HgtArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S;
   const int nchunks = a.dchunk_ofs[a.csr_rows];
   const int stride = 2 * a.S + D;
-  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const int row = a.dchunk_row[c];
-    const int64_t cb = (int64_t)a.dptr[row] + (int64_t)(c - a.dchunk_ofs[row]) * kChunkEdges;
-    const int64_t ce = min((int64_t)a.dptr[row + 1], cb + kChunkEdges);
-    const int64_t beg = cb + warp * kChunkPart, end = min(ce, beg + kChunkPart);
+  for_chunks(a.dptr, a.dchunk_ofs, a.dchunk_row, nchunks, [&](int c, int row, int64_t cb, int64_t ce) {
+    const int64_t share = chunk_share(ce - cb), beg = cb + warp * share, end = min(ce, beg + share);
     float q[E], m = -INFINITY, l = 0.f, acc[1][E];
     load_slice<T, E>((const T*)a.Qp + (int64_t)a.mrow[row] * D + lane * E, q);
 #pragma unroll
@@ -477,7 +524,7 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_fwd_chunks(HgtArgs a) {
     part[warp][lane][E + 1] = l;
     __syncthreads();
     if (warp == 0) {
-      for (int w = 1; w < kChunkWarps && cb + w * kChunkPart < ce; ++w) {
+      for (int w = 1; w < kChunkWarps && cb + w * share < ce; ++w) {
         float pv[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) pv[e] = part[w][lane][e];
@@ -492,7 +539,7 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_fwd_chunks(HgtArgs a) {
       for (int e = 0; e < E; ++e) p[2 * a.S + lane * E + e] = acc[0][e];
     }
     __syncthreads();
-  }
+  });
 }
 
 // nodes with at least one in-edge
@@ -530,10 +577,11 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
   const int64_t total = live_nodes(a);
   const int stride = 2 * a.S + D;
-  for (int64_t x0 = claim(a.work, NC); x0 < total; x0 = claim(a.work, NC)) {
+  const int nc = claim_size(total, NC), hub = hub_runs(a.dchunk_ofs[a.csr_rows]);
+  for (int64_t x0 = claim(a.work, nc); x0 < total; x0 = claim(a.work, nc)) {
     int t = -1, mrow = -1, eb = 0, ee = 0, cb = 0, ce = 0;
     int64_t jl = 0;
-    if (x0 + lane / KS < total) live_node(a, x0 + lane / KS, t, jl);
+    if (lane / KS < nc && x0 + lane / KS < total) live_node(a, x0 + lane / KS, t, jl);
     const int r = t >= 0 ? a.rslot[t][lane % KS] : -1;
     if (r >= 0) {
       const int64_t cr = a.meta.row_base[r] + jl;
@@ -547,7 +595,7 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1
       }
     }
     const int64_t node = t >= 0 ? a.meta.type_off[t] + jl : 0;
-    const int nn = (int)min((int64_t)NC, total - x0);
+    const int nn = (int)min((int64_t)nc, total - x0);
     for (int n = 0; n < nn; ++n) {
       int row[KS];
       RawSlice<T, E> q[KS];
@@ -571,7 +619,7 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, (D <= 128 && KS <= 4) ? 6 : 1
         const int b = __shfl_sync(kAll, eb, n * KS + k), e = __shfl_sync(kAll, ee, n * KS + k);
         const int c0 = __shfl_sync(kAll, cb, n * KS + k), c1 = __shfl_sync(kAll, ce, n * KS + k);
         if (row[k] < 0) continue;
-        if (c1 > c0) {
+        if (e - b > hub) {
           for (int c = c0; c < c1; c += kBatch) {  // kBatch partials loaded before the first is merged
             float pm[kBatch], pl[kBatch], pv[kBatch][E];
 #pragma unroll
@@ -716,11 +764,8 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_dst_chunks(HgtArgs a
   __shared__ float part[kChunkWarps][32][E];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S, h = lane / lph;
   const int nchunks = a.dchunk_ofs[a.csr_rows];
-  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const int row = a.dchunk_row[c];
-    const int64_t cb = (int64_t)a.dptr[row] + (int64_t)(c - a.dchunk_ofs[row]) * kChunkEdges;
-    const int64_t ce = min((int64_t)a.dptr[row + 1], cb + kChunkEdges);
-    const int64_t beg = cb + warp * kChunkPart, end = min(ce, beg + kChunkPart);
+  for_chunks(a.dptr, a.dchunk_ofs, a.dchunk_row, nchunks, [&](int c, int row, int64_t cb, int64_t ce) {
+    const int64_t share = chunk_share(ce - cb), beg = cb + warp * share, end = min(ce, beg + share);
     const int64_t mr = a.mrow[row];
     const float4 st = a.rstat[mr * a.S + h];
     float q[E], g[E], acc[E];
@@ -736,7 +781,7 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_dst_chunks(HgtArgs a
 #pragma unroll
       for (int e = 0; e < E; ++e) a.part[(int64_t)c * D + lane * E + e] = acc[e];
     __syncthreads();
-  }
+  });
 }
 
 // acc += the partials [c0, c1) of one row in order, N floats per lane at p + c * stride; kBatch
@@ -768,8 +813,9 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_dst
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S, h = lane / lph;
   const int64_t total = *a.mcount;
-  for (int64_t x0 = claim(a.work + 1, kRowClaim); x0 < total; x0 = claim(a.work + 1, kRowClaim)) {
-    const int nn = (int)min((int64_t)kRowClaim, total - x0);
+  const int nc = claim_size(total, kRowClaim), hub = hub_runs(a.dchunk_ofs[a.csr_rows]);
+  for (int64_t x0 = claim(a.work + 1, nc); x0 < total; x0 = claim(a.work + 1, nc)) {
+    const int nn = (int)min((int64_t)nc, total - x0);
     int eb = 0, ee = 0, cb = 0, ce = 0;
     if (lane < nn) {
       const int64_t cr = a.mlist[x0 + lane];
@@ -800,7 +846,7 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_dst
       float acc[E];
 #pragma unroll
       for (int e = 0; e < E; ++e) acc[e] = 0.f;
-      if (c1 > c0) {
+      if (e1 - b > hub) {
         add_parts<E>(a.part + lane * E, D, c0, c1, acc);
       } else {
         float qf[E], gf[E];
@@ -875,11 +921,8 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_src_chunks(HgtArgs a
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lph = 32 / a.S;
   const int nchunks = a.schunk_ofs[a.N];
   const T* KV = (const T*)a.KV;
-  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const int i = a.schunk_row[c];
-    const int64_t cb = (int64_t)a.sptr[i] + (int64_t)(c - a.schunk_ofs[i]) * kChunkEdges;
-    const int64_t ce = min((int64_t)a.sptr[i + 1], cb + kChunkEdges);
-    const int64_t beg = cb + warp * kChunkPart, end = min(ce, beg + kChunkPart);
+  for_chunks(a.sptr, a.schunk_ofs, a.schunk_row, nchunks, [&](int c, int i, int64_t cb, int64_t ce) {
+    const int64_t share = chunk_share(ce - cb), beg = cb + warp * share, end = min(ce, beg + share);
     float k[E], v[E], acc[2 * E];
     load_slice<T, E>(KV + (int64_t)i * 2 * D + lane * E, k);
     load_slice<T, E>(KV + (int64_t)i * 2 * D + D + lane * E, v);
@@ -893,7 +936,7 @@ __global__ void __launch_bounds__(32 * kChunkWarps) hgt_bwd_src_chunks(HgtArgs a
 #pragma unroll
       for (int e = 0; e < 2 * E; ++e) a.part[((int64_t)c * 32 + lane) * 2 * E + e] = acc[e];
     __syncthreads();
-  }
+  });
 }
 
 // dK(i), dV(i) of every node (zeros without out-edges); claims and prefetch as in hgt_bwd_dst_rows.
@@ -903,8 +946,9 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_src
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31, lph = 32 / a.S;
   const T* KV = (const T*)a.KV;
-  for (int64_t x0 = claim(a.work + 2, kRowClaim); x0 < a.N; x0 = claim(a.work + 2, kRowClaim)) {
-    const int nn = (int)min((int64_t)kRowClaim, a.N - x0);
+  const int nc = claim_size(a.N, kRowClaim), hub = hub_runs(a.schunk_ofs[a.N]);
+  for (int64_t x0 = claim(a.work + 2, nc); x0 < a.N; x0 = claim(a.work + 2, nc)) {
+    const int nn = (int)min((int64_t)nc, a.N - x0);
     int eb = 0, ee = 0, cb = 0, ce = 0;
     if (lane < nn) {
       eb = a.sptr[x0 + lane];
@@ -932,7 +976,7 @@ __global__ void __launch_bounds__(32 * kEdgeWarps, D <= 128 ? 6 : 1) hgt_bwd_src
       float acc[2 * E];
 #pragma unroll
       for (int e = 0; e < 2 * E; ++e) acc[e] = 0.f;
-      if (c1 > c0) {
+      if (e1 - b > hub) {
         add_parts<2 * E>(a.part + lane * 2 * E, 2 * D, c0, c1, acc);
       } else if (e1 > b) {
         float kf[E], vf[E];
@@ -1130,7 +1174,7 @@ unsigned grid_of(int64_t threads) { return (unsigned)std::max<int64_t>(1, ceil_d
 unsigned chunk_blocks(int64_t cap) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(cap, 152 * 8)); }
 // CTAs of a claiming kernel over at most n items: what the SMs hold, or fewer for few items
 unsigned claim_blocks(int64_t n) {
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, kRowClaim * kEdgeWarps), 152 * 6));
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, kEdgeWarps), 152 * 6));
 }
 
 template <typename T, int D>

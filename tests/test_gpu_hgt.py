@@ -200,3 +200,46 @@ def test_more_than_four_relations_into_a_type(into, dtype, d, heads):
     for k in KEYS:
         assert relerr(gr[k], gref[k]) <= TOL[dtype], (k, relerr(gr[k], gref[k]))
     assert hg.hg_device_status() == 0
+
+
+@pytest.mark.parametrize("dtype,d,many", [("f32", 64, False), ("bf16", 128, False), ("f32", 64, True), ("bf16", 64, True)])
+def test_rows_around_the_hub_limits(dtype, d, many):
+    """Rows and out-lists of 95 to 1025 runs, at the edges of a warp's share of a chunk and of a chunk; with many
+    (above 16384 chunks) rows of up to 384 runs leave the chunks for a warp."""
+    need_gpu()
+    hg = lib()
+    runs = [95, 96, 97, 124, 128, 129, 160, 161, 383, 384, 385, 511, 512, 513, 1024, 1025]
+    fill = 17_000 if many else 0  # more rows of 97 runs
+    nu, heads = 1100 + fill, 4
+    rng = np.random.default_rng(d)
+    src, dst = [], []
+    for k, n in enumerate(runs):  # into risk k from n users, and from risk 20 + k into n users
+        at = rng.permutation(1100)[:n]
+        src += [at, np.full(n, nu + 20 + k)]
+        dst += [np.full(n, nu + k), at]
+    rel = np.concatenate([np.full(x.size, k % 2) for k, x in enumerate(src)])
+    if many:  # hubs on both sides: the users from 1100 on have 97 in-edges each from 97 other users, and as many out-edges
+        a = 1100 + np.repeat(np.arange(fill), 97)
+        b = 1100 + (a - 1100 + 1 + np.tile(np.arange(97) * 3, fill)) % fill
+        src.append(b), dst.append(a)
+        rel = np.concatenate([rel, np.full(a.size, 2)])
+    rels = ((0, 1), (1, 0), (0, 0))
+    sp = hgsynth.spec("tiny-10k", n_user=nu, n_risk=40, num_rels=3, d=d, dtype=dtype)
+    st = hgsynth.bf16_round if dtype == "bf16" else (lambda x: x)
+    g = {"src": np.concatenate(src).astype(np.int32), "dst": np.concatenate(dst).astype(np.int32),
+         "rel": rel.astype(np.int32), "type_offsets": np.array([0, nu, nu + 40], np.int64), "rels": rels}
+    w = SimpleNamespace(spec=sp, graph=g, X=st(rng.standard_normal((nu + 40, d)).astype(np.float32)),
+                        dH_top=st(rng.standard_normal((nu + 40, d)).astype(np.float32)))
+    p = hgsynth.make_hgt_params(sp, heads, bias_margin=BF16_RELU_MARGIN)
+    out, dH, gr = run_gpu(hg, w, p, heads, True, w.dH_top)
+    args = (g["src"], g["dst"], g["rel"], g["type_offsets"], rels, p, w.X)
+    ref, _ = OH.hgt_forward(*args, heads, layernorm=True)
+    dref, gref = OH.hgt_backward(*args, w.dH_top, heads, layernorm=True)
+    assert relerr(out, ref) <= TOL[dtype] and relerr(dH, dref) <= TOL[dtype]
+    for k in KEYS:
+        # every target has one relation, so b_K shifts all scores of a softmax alike: its gradient is zero
+        scale = np.abs(gref["W_K" if k == "b_K" else k]).max()
+        if k == "mu":  # <W_att, dW_att> / mu, a sum of cancelling terms
+            scale = max(np.linalg.norm(p["W_att"][r]) * np.linalg.norm(gref["W_att"][r]) for r in range(3))
+        assert np.abs(gr[k] - gref[k]).max() <= TOL[dtype] * scale, k
+    assert hg.hg_device_status() == 0
