@@ -369,9 +369,11 @@ __global__ void __launch_bounds__(1024) align_loss_finish(const float* __restric
 }
 
 // Backward, row tiles of 64 for one view (blockIdx.y): G = dloss (+-2 (z_a - z_b) + 4 lambda z (C - I)),
-// stored in fp32 scratch; per-block column partials of g = G / sqrt(n) and g * x_hat.
+// stored in fp32 scratch; per-block column partials of g = G / sqrt(n) and g * x_hat.  Both views' blocks (2
+// x kAlignBlocks) are four per SM: with 75 registers at d = 64 three were resident and the rest a second wave
+// (200k rows: 283 -> 450 us).
 template <typename T, int D>
-__global__ void __launch_bounds__(256) align_bwd_rows(const T* __restrict__ Ha, int64_t rows_a,
+__global__ void __launch_bounds__(256, D == 64 ? 4 : 1) align_bwd_rows(const T* __restrict__ Ha, int64_t rows_a,
                                                       const int32_t* __restrict__ ia, const T* __restrict__ Hb,
                                                       int64_t rows_b, const int32_t* __restrict__ ib,
                                                       int64_t n_max, const int64_t* __restrict__ n_dev,
