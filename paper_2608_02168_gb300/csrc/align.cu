@@ -369,11 +369,12 @@ __global__ void __launch_bounds__(1024) align_loss_finish(const float* __restric
 }
 
 // Backward, row tiles of 64 for one view (blockIdx.y): G = dloss (+-2 (z_a - z_b) + 4 lambda z (C - I)),
-// stored in fp32 scratch; per-block column partials of g = G / sqrt(n) and g * x_hat.  Both views' blocks (2
-// x kAlignBlocks) are four per SM: with 75 registers at d = 64 three were resident and the rest a second wave
-// (200k rows: 283 -> 450 us).
+// stored in fp32 scratch; per-block column partials of g = G / sqrt(n) and g * x_hat.  The two views' blocks (2
+// x kAlignBlocks) are four per SM, so the launch bound is a bound on the waves: at d = 64, 75 registers left room for
+// three blocks and a second wave for the rest (200k rows 450 us, with 64 registers 282 us); at d = 128, 128 registers
+// for two (1.19 ms, with 167 for one 1.88 ms).
 template <typename T, int D>
-__global__ void __launch_bounds__(256, D == 64 ? 4 : 1) align_bwd_rows(const T* __restrict__ Ha, int64_t rows_a,
+__global__ void __launch_bounds__(256, D == 64 ? 4 : (D == 128 ? 2 : 1)) align_bwd_rows(const T* __restrict__ Ha, int64_t rows_a,
                                                       const int32_t* __restrict__ ia, const T* __restrict__ Hb,
                                                       int64_t rows_b, const int32_t* __restrict__ ib,
                                                       int64_t n_max, const int64_t* __restrict__ n_dev,

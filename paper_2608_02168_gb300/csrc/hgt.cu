@@ -350,7 +350,7 @@ __device__ __forceinline__ int64_t chunk_share(int64_t n) {
 // runs.  Up to kManyChunks of them the hub rows are the exception that would hold a warp while the others are
 // done.  From there on they are the work itself, enough of it to keep every warp busy, and a warp per row saves
 // the CTA's barriers and the partials: degrees around 110 on 50k nodes, chunks / warps 2.96 / 2.13 ms; on
-// 5k nodes of skewed degrees (zipf 0.8, 100 edges per node) 0.87 / 0.98 ms.  Rows of one chunk (at most
+// 5k nodes of skewed degrees (zipf 0.8, 100 edges per node) 0.87 / 0.99 ms.  Rows of one chunk (at most
 // kChunkEdges runs) can go either way.  With the line at 256 / 384 / 512 runs: degrees around 300 6.11 / 4.73 /
 // 4.74 ms, around 450 8.10 / 8.56 / 6.96 ms, but 100k nodes of zipf 0.8, 100 edges per node, 5.31 / 5.44 / 5.70 ms (5.13
 // with all in chunks): a late claim of long rows is that kernel's tail.
