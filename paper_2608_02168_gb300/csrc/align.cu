@@ -42,9 +42,10 @@ __device__ __forceinline__ int64_t warp_lower_bound(const int64_t* __restrict__ 
   return lo;
 }
 
-// flag[i] = 1 and pos[i] = k where a[i] == b[k].  A CTA takes 1024 consecutive entries of a: one warp
-// finds where the first of them would stand in b, another the last, and each entry is then searched in
-// that stretch only, from shared memory when it fits (lists of a like density: it holds about as many
+// flag[i] = 1 and pos[i] = k where a[i] == b[k].  A CTA takes 1024 consecutive entries of a (256 where the grid
+// covers a with them: 100k against 5M ids 31.7 -> 23.2 us for the call; 1M against 10M would lose 13 %):
+// one warp finds where the first of them would stand in b, another the last, and each entry is then searched
+// in that stretch only, from shared memory when it fits (lists of a like density: it holds about as many
 // entries).  A search of all of b per entry took 262 us for two lists of 10M ids, this 151 us.
 constexpr int kIsectItems = 1024, kIsectStage = 2048;
 __global__ void __launch_bounds__(256) intersect_flags(const int64_t* __restrict__ a, int64_t na,
@@ -55,8 +56,9 @@ __global__ void __launch_bounds__(256) intersect_flags(const int64_t* __restrict
   __shared__ int64_t stage[kIsectStage];
   __shared__ int64_t range[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int64_t i0 = (int64_t)blockIdx.x * kIsectItems; i0 < na; i0 += (int64_t)gridDim.x * kIsectItems) {
-    const int64_t i1 = min(i0 + kIsectItems, na);
+  const int64_t items = na <= (int64_t)gridDim.x * 256 ? 256 : kIsectItems;
+  for (int64_t i0 = (int64_t)blockIdx.x * items; i0 < na; i0 += (int64_t)gridDim.x * items) {
+    const int64_t i1 = min(i0 + items, na);
     if (warp < 2) {
       const int64_t k = warp_lower_bound(b, 0, nb, a[warp ? i1 - 1 : i0]);
       if (lane == 0) range[warp] = k;
