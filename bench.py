@@ -372,8 +372,9 @@ def kernel_models(st: dict, sp) -> dict:
     m["proj_fwd_gather_tc"] = (L * (tf - row * NNZ + fuse_in), L * tfl)
     m["wgrad_gather_tc"] = (L * ((row + 4) * NNZ + fuse_in), L * 2 * d * d * NNZ)
     m["gathered"].update({"proj_fwd_gather_tc": L * f["R_short"] * (8 + row), "wgrad_gather_tc": L * f["R_short"] * (8 + row)})
-    # per 8-bit pass over the keys: read and write of key, edge id and endpoint; three stable sorts
-    # (by source id, then CSR row: (row, source, edge id); that order by CSC row)
+    # per pass over 8 key bits: read and write of key, edge id and endpoint; three stable sorts of the edges
+    # (by source id, then CSR row: (row, source, edge id); that order by CSC row).  The sort as built makes
+    # fewer passes and sorts runs last (`moved` below)
     passes = lambda rows: max(1, -(-int(rows).bit_length() // 8))  # noqa: E731
     m["radix_scatter"] = (2 * 12 * st["E"] * (passes(N) + passes(RR) + passes(CC)), 0)
     # what the kernels as built move where that differs from the terms above (used for rates): the sorts
@@ -701,13 +702,12 @@ def measure_hgt(w: dict, steps: int, warmup: int, dev, with_cpu: bool) -> dict:
     ms = statistics.median(times)
     # no-reuse model per layer: the forward and the two backward edge passes each read a run entry
     # (8 bytes: column and multiplicity) and gather two rows per run of parallel edges (K and V; K
-    # and V; Q' and dS), plus the dense rows (K, V, Q', S written and read, the projection's and
-    # the backward products' rows)
+    # and V; Q' and dS), plus the rows of the dense products: Q' and S of the non-empty (relation, target)
+    # rows written and read, K, V, the projection's and the backward products' rows per node
     b = 4 if sp.dtype == "f32" else 2
-    offs = [int(x) for x in g["type_offsets"]]
-    RR = sum(offs[t + 1] - offs[t] for _, t in g["rels"])
-    runs = int(torch.unique((g["rel"].long() * N + g["dst"].long()) * N + g["src"].long()).numel())
-    per_layer = 3 * runs * (8 + 2 * sp.d * b) + (2 * RR + 10 * sp.num_nodes) * sp.d * b
+    rows = g["rel"].long() * N + g["dst"].long()
+    runs, stored = int(torch.unique(rows * N + g["src"].long()).numel()), int(torch.unique(rows).numel())
+    per_layer = 3 * runs * (8 + 2 * sp.d * b) + (2 * stored + 10 * sp.num_nodes) * sp.d * b
     peaks, psrc = load_peaks()
     ach = sp.layers * per_layer / (ms / 1e3) / 1e9
     res = {"workload": workload_desc(sp), "ms": round(ms, 4), "layers": sp.layers, "heads": HGT_HEADS,
@@ -715,8 +715,8 @@ def measure_hgt(w: dict, steps: int, warmup: int, dev, with_cpu: bool) -> dict:
            "roofline": {"bound": "hbm", "achieved": round(ach, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
                         "peak_source": f"{psrc} hbm_gbs", "frac": round(ach / peaks["hbm_gbs"], 4),
                         "frac_of_nominal": round(ach / NOMINAL_HBM_GBS, 4),
-                        "model": "no-reuse: 3 edge passes x (8 + 2 d b) per run of parallel edges + (2 csr_rows + 10 N) d b per layer",
-                        "runs": runs,
+                        "model": "no-reuse: 3 edge passes x (8 + 2 d b) per run of parallel edges + (2 stored rows + 10 N) d b per layer",
+                        "runs": runs, "stored_rows": stored,
                         "algorithmic_bytes_per_call": int(sp.layers * per_layer)},
            "kernel_time_share": {k: round(v / tot, 4) for k, (_, v) in sorted(rep.items(), key=lambda kv: -kv[1][1])},
            "cpu_baseline": None}

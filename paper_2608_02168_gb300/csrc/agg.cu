@@ -262,8 +262,8 @@ struct Slice {
   }
 };
 
-// Row kernels, streamed (agg_fwd_rows, agg_bwd_nodes).  A warp takes a chunk of 16 consecutive rows
-// (lane l < 16 holds row l's bounds and scale; every lane owns D / 32 columns) and streams through
+// Row kernels, streamed (agg_fwd_rows, agg_bwd_nodes).  A warp takes a chunk of up to 16 consecutive rows
+// (lane l holds row l's bounds and scale; every lane owns D / 32 columns) and streams through
 // the chunk's runs, which are contiguous, in batches of eight gathered rows that cross row
 // boundaries; a row is written when its last run is added, so the loads of a short row do not wait
 // on those of the row before.  Each row's runs are added one by one, in run order, into an fp32

@@ -376,13 +376,11 @@ __global__ void __launch_bounds__(1024) align_loss_finish(const float* __restric
 // three blocks and a second wave for the rest (200k rows 450 us, with 64 registers 282 us); at d = 128, 128 registers
 // for two (1.19 ms, with 167 for one 1.88 ms).
 template <typename T, int D>
-__global__ void __launch_bounds__(256, D == 64 ? 4 : (D == 128 ? 2 : 1)) align_bwd_rows(const T* __restrict__ Ha, int64_t rows_a,
-                                                      const int32_t* __restrict__ ia, const T* __restrict__ Hb,
-                                                      int64_t rows_b, const int32_t* __restrict__ ib,
-                                                      int64_t n_max, const int64_t* __restrict__ n_dev,
-                                                      const float* __restrict__ stats, const float* __restrict__ C,
-                                                      float lambda_n, float dloss, float* __restrict__ G,
-                                                      float* __restrict__ part) {
+__global__ void __launch_bounds__(256, D == 64 ? 4 : (D == 128 ? 2 : 1))
+    align_bwd_rows(const T* __restrict__ Ha, int64_t rows_a, const int32_t* __restrict__ ia, const T* __restrict__ Hb,
+                   int64_t rows_b, const int32_t* __restrict__ ib, int64_t n_max, const int64_t* __restrict__ n_dev,
+                   const float* __restrict__ stats, const float* __restrict__ C, float lambda_n, float dloss,
+                   float* __restrict__ G, float* __restrict__ part) {
   pdl_begin();
   using TL = Tile<float, D>;
   constexpr int RM = TL::RM, CN = TL::CN;

@@ -25,8 +25,9 @@ constexpr int kProjTileRows = 128;  // output rows per tile of the tensor-core f
 // 512 / 128 / 96 / 64 / 40: 100k nodes fp32 854 / 726 / 717 / 696 / 684 us, 1M-node step 5.89 / 5.47 / 5.50 /
 // 5.43 / 5.44 ms, 10M nodes 11.21 / 10.99 / 11.09 / 11.17 / 11.41 ms; 2M nodes forward 3.05 / 2.65 / 2.67 / 2.69 /
 // 2.92 ms.  Chunks of 128, 256 and 1024 runs were slower on the large graphs (12.30, 11.42, 11.32 ms).
-// The scratch holds a partial for each of E / kChunkEdges + min(E / (kHubDegree + 1), rows) chunks: at 200M edges, d = 128,
-// 1.26 GB for the mean layer (0.40 GB at 512) and 2.51 GB for the attention layer (partials of 2 d; 1.20 GB at 512).
+// The scratch holds a partial for each of E / kChunkEdges + min(E / (kHubDegree + 1), rows) chunks: at 200M
+// edges, d = 128, 1.26 GB for the mean layer (0.40 GB at 512) and 2.51 GB for the attention layer (partials of
+// 2 d; 1.20 GB at 512).  The attention layer moves the line up where hub rows are many (hgt.cu).
 constexpr int kHubDegree = 96;
 constexpr int kChunkEdges = 512;
 // The fused mean layer (gathers into the projection's operand tiles) sums a CSR row in the

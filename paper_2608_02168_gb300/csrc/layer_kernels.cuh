@@ -9,8 +9,8 @@
 namespace hg {
 
 struct FwdArgs {
-  const void* M;                 // saved relation means, concatenated CSR rows (or compact rows)
-  const int32_t* mrow;           // compact index of each CSR row (>= msent: empty); null: M by CSR row
+  const void* M;                 // saved relation rows, compact
+  const int32_t* mrow;           // compact index of each CSR row (>= msent: empty)
   int64_t msent;
   int nrel;
   int64_t mrow0[kMaxRels];       // first CSR row of each relation into this type
@@ -43,8 +43,8 @@ struct BwdArgs {
   void* dY;                      // node rows
   void* dU;                      // node rows
   void* dZ;                      // node rows
-  void* dMs;                     // concatenated CSR rows (scaled by 1/deg), or compact rows
-  const int32_t* mrow;           // compact index of each CSR row (>= msent: empty, not stored); null: CSR rows
+  void* dMs;                     // compact rows (scaled by 1/deg)
+  const int32_t* mrow;           // compact index of each CSR row (>= msent: empty, not stored)
   int64_t msent;
   float* part;                   // [blocks][3][D]: db, dgamma, dbeta partials
   int64_t off, n;
@@ -89,7 +89,7 @@ struct TcBwdArgs {
   int rel[kMaxRels];
   int64_t mrow0[kMaxRels];
   const int32_t* mlist;       // CSR row of each compact row; mbase[r] .. mbase[r + 1] = relation r's
-  const int32_t* mbase;       // compact rows (device).  null: every CSR row, dMs indexed by CSR row
+  const int32_t* mbase;       // compact rows (device)
   int type;
   const __nv_bfloat16* dH_out;
   const __nv_bfloat16* H_in;

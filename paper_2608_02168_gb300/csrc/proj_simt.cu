@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(256) proj_bwd_simt(BwdArgs a) {
       const int m = ty * RM + i;
       if (m >= nv) continue;
       const int64_t row = a.mrow0[r] + m0 + m;
-      const int64_t out = a.mrow ? (int64_t)a.mrow[row] : row;  // compact rows: empty rows are not stored
-      if (a.mrow && out >= a.msent) continue;
+      const int64_t out = a.mrow[row];  // compact rows: empty rows are not stored
+      if (out >= a.msent) continue;
       const int deg = a.csr_ptr ? a.csr_ptr[row + 1] - a.csr_ptr[row] : 0;
       const float sc = !a.csr_ptr ? 1.f : (deg > 0 ? __fdiv_rn(1.0f, (float)deg) : 0.f);
       float v[CN];
@@ -246,9 +246,10 @@ __global__ void __launch_bounds__(256) proj_bwd_simt(BwdArgs a) {
 // ---------------------------------------------------------------------------------------------
 // With a map, over a relation's stored rows: X rows are compact rows, Y rows the rows' nodes (their count
 // is a device value, split over the grid on the device).  At d = 64 the next step's rows are loaded
-// while a step is multiplied (at 128 and 256 that left one CTA on an SM and lost 1 %).  Bound by fp32 FMA on large graphs and by the steps' latency on small ones, so a split is
-// 64 rows (256 before) until there are two CTAs per SM.  Per launch on 8000 nodes, d = 64: 18.1 -> 4.1 us (a
-// scan of all rows before, empty ones as zeros); 100k nodes, six launches: 183 -> 67 us.
+// while a step is multiplied (at 128 and 256 that left one CTA on an SM and lost 1 %).  Bound by fp32 FMA
+// on large graphs and by the steps' latency on small ones, so a split is 64 rows (256 before) until there
+// are two CTAs per SM.  Per launch on 8000 nodes, d = 64: 18.1 -> 4.1 us (a scan of all rows before, empty
+// ones as zeros); 100k nodes, six launches: 183 -> 67 us.
 constexpr int kWT = 128;  // output tile edge (D >= 128) or D
 constexpr int kWR = 32;   // rows per step
 

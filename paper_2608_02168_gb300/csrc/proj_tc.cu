@@ -1147,15 +1147,15 @@ struct RelMaps {
 // The jobs of proj_bwd_tc: 128 rows of one relation's stored rows each, relation by relation.
 struct BwdJobs {
   int nrel;
-  int64_t base[kMaxRels];   // first stored row of relation j (compact index, or 0 by CSR row)
+  int64_t base[kMaxRels];   // first stored row of relation j (compact index)
   int64_t count[kMaxRels];  // its stored rows
   int64_t first[kMaxRels + 1];  // first job of relation j; first[nrel] = the number of jobs
   __device__ __forceinline__ void init(const TcBwdArgs& a) {  // one thread
     nrel = a.nrel;
     first[0] = 0;
     for (int j = 0; j < a.nrel; ++j) {
-      base[j] = a.mlist ? (int64_t)a.mbase[a.rel[j]] : 0;
-      count[j] = a.mlist ? (int64_t)a.mbase[a.rel[j] + 1] - base[j] : a.n;
+      base[j] = a.mbase[a.rel[j]];
+      count[j] = (int64_t)a.mbase[a.rel[j] + 1] - base[j];
       first[j + 1] = first[j] + (count[j] + kTileRows - 1) / kTileRows;
     }
   }
@@ -1234,7 +1234,7 @@ __global__ void __launch_bounds__(BwdCfg<D>::kThreads, 1)
       for (int i = 0; i < 4; ++i) {
         const int64_t k = i0 + 4 * lane + i;
         int64_t local = a.n;  // past the relation's rows: zeros
-        if (k < J.count[j]) local = a.mlist ? (int64_t)__ldg(a.mlist + J.base[j] + k) - a.mrow0[j] : k;
+        if (k < J.count[j]) local = (int64_t)__ldg(a.mlist + J.base[j] + k) - a.mrow0[j];
         c[i] = (int)local;
       }
       const int ab = it % NA;
@@ -1318,8 +1318,8 @@ __global__ void __launch_bounds__(BwdCfg<D>::kThreads, 1)
       const int j = J.rel_of(job);
       const int64_t kr = (job - J.first[j]) * kTileRows + row;  // row within the relation's stored rows
       const bool live = kr < J.count[j];
-      const int64_t crow = !live ? 0 : (a.mlist ? (int64_t)a.mlist[J.base[j] + kr] : a.mrow0[j] + kr);
-      const int64_t out = a.mlist ? J.base[j] + kr : crow;  // compact row, or CSR row
+      const int64_t crow = live ? (int64_t)a.mlist[J.base[j] + kr] : 0;
+      const int64_t out = J.base[j] + kr;
       const int deg = live && a.csr_ptr ? a.csr_ptr[crow + 1] - a.csr_ptr[crow] : 0;
       const float sc = !a.csr_ptr ? 1.f : (deg > 0 ? __fdiv_rn(1.0f, (float)deg) : 0.f);
       const uint32_t k = jb % NB;

@@ -86,9 +86,9 @@ __device__ __forceinline__ void stage_b(float* Bs, const T* __restrict__ B, int 
 // acc[i][j] += sum_k A(ty*RM+i, k) * B(k, tx*CN + j) for k in [0, KC), in order of k; A from an fp32 smem
 // tile with row stride lda and column offset kofs (both multiples of four), B from Bs (columns at b_pos).
 // A is read four k at a time: with one read per row and k the products waited for shared memory (1.5
-// times the FMA cycles at d = 64, 2.2 times at 256, where B's bank conflicts came on top).  223k nodes fp32, layer forward + backward at d = 256: 16.5 -> 10.7 ms;
-// temporal module, 60k nodes, d = 256: 17.5 -> 12.4 ms, 90k nodes, d = 128: 6.09 -> 5.42 ms; at d = 64 the layer of
-// 112k nodes 518 -> 509 us.
+// times the FMA cycles at d = 64, 2.2 times at 256, where B's bank conflicts came on top).  223k nodes fp32,
+// layer forward + backward at d = 256: 16.5 -> 10.7 ms; temporal module, 60k nodes, d = 256: 17.5 -> 12.4 ms, 90k
+// nodes, d = 128: 6.09 -> 5.42 ms; at d = 64 the layer of 112k nodes 518 -> 509 us.
 template <int D, int RM, int CN>
 __device__ __forceinline__ void mma_chunk(const float* A, int lda, int kofs, const float* Bs, float (&acc)[RM][CN]) {
   static_assert(CN == D / 16 && CN % 4 == 0, "columns per thread");
