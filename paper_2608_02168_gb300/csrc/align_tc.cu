@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         tmem_ld16(trow + c0p + c, v);
         float* dst = Ps + ((warp & 3) * 32 + (threadIdx.x & 31)) * C::kPLd + c;
 #pragma unroll
-        for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        for (int i = 0; i < 16; i += 4)
+          *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
       }
       __syncthreads();
       const int c0 = c0p + pg * 8;

@@ -319,7 +319,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter(
 #pragma unroll
   for (int r = 0; r < kItems; ++r) {
     old[r] = 0;
-    if (j0 + 32 * r < cnt && lane == __ffs(peers[r]) - 1) old[r] = atomicAdd(&wh[(k[r] >> shift) & mask], __popc(peers[r]));
+    if (j0 + 32 * r < cnt && lane == __ffs(peers[r]) - 1)
+      old[r] = atomicAdd(&wh[(k[r] >> shift) & mask], __popc(peers[r]));
     __syncwarp();  // the next round's adds come after
   }
 #pragma unroll
@@ -716,9 +717,8 @@ __global__ void __launch_bounds__(256) row_pack(const int32_t* __restrict__ mrow
 // The runs in CSC order (sorted keys, uval and destination of each; cptr: CSC row pointers over
 // runs).  Writes the node-major list of out-runs used by the backward aggregation -- node i's row holds,
 // relation by relation (ascending) and in CSC order within a relation, the compact row of each run's
-// target and its multiplicity -- and, per run, its length, its
-// first CSR position (or uval, for one edge), and
-// 1 / deg_r(destination).
+// target and its multiplicity -- and, per run, its length, its first CSR position (or uval, for one
+// edge), and 1 / deg_r(destination).
 __global__ void __launch_bounds__(256) csc_runs(
     const uint32_t* __restrict__ skey, const uint32_t* __restrict__ srun, const uint32_t* __restrict__ sdst,
     const int32_t* __restrict__ n_dev, const int32_t* __restrict__ cptr, GraphMeta m,
@@ -1150,14 +1150,14 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     HG_TRY(launch("edge_keys", edge_keys, dim3(g), dim3(256), 0, s, src, dst, rel, E, m, rows, L.sort.keys[0],
                   L.sort.ckeys));
     int r1 = 0;
-    HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)N), (const uint32_t*)L.sort.keys[0], (const uint32_t*)nullptr,
-                      (const uint32_t*)L.sort.ckeys, 0, s, &r1));
+    HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)N), (const uint32_t*)L.sort.keys[0],
+                      (const uint32_t*)nullptr, (const uint32_t*)L.sort.ckeys, 0, s, &r1));
     // the last pass writes the edge ids and source ids straight into csr_eid and csr_col
     HG_TRY(radix_sort(L.sort, E, nullptr, bit_width((uint64_t)rows), (const uint32_t*)L.sort.vals2[r1],
                       (const uint32_t*)L.sort.vals[r1], (const uint32_t*)L.sort.keys[r1], r1, s, &res,
                       (uint32_t*)L.csr_eid, (uint32_t*)L.csr_col));
-    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, (const uint32_t*)L.sort.keys[res],
-                  E, (const int32_t*)nullptr, rows, L.csr_ptr, L.invalid));
+    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s,
+                  (const uint32_t*)L.sort.keys[res], E, (const int32_t*)nullptr, rows, L.csr_ptr, L.invalid));
   }
   // non-empty CSR rows (the rows the mean layer stores) and their compact numbering
   HG_TRY(launch("nonempty_flags", nonempty_flags, dim3(grid_for(rows)), dim3(256), 0, s, (const int32_t*)L.csr_ptr,
@@ -1176,8 +1176,8 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
                   (const int32_t*)L.csr_ptr, rows, E, flag));
     HG_TRY(exclusive_scan(flag, u, E, L.sort.scan_scratch, s));
     HG_TRY(launch("run_write", run_write, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, (const int32_t*)u,
-                  (const int32_t*)L.csr_col, rkey, (const int32_t*)L.csr_ptr, rows, m, (const int32_t*)L.csr_eid, L.agg_col, L.run_pos,
-                  L.sort.ckeys, L.sort.vals2[res], L.sort.vals[res]));
+                  (const int32_t*)L.csr_col, rkey, (const int32_t*)L.csr_ptr, rows, m, (const int32_t*)L.csr_eid,
+                  L.agg_col, L.run_pos, L.sort.ckeys, L.sort.vals2[res], L.sort.vals[res]));
     HG_TRY(launch("run_finish", run_finish, dim3(grid_for(std::max(E, rows + 1))), dim3(256), 0, s, (const int32_t*)u,
                   (const int32_t*)L.run_pos, (const int32_t*)L.csr_ptr, rows, L.agg_cnt, L.agg_ptr));
     // the runs by CSC row
@@ -1186,8 +1186,8 @@ extern "C" hg_status hg_build_csr(const int32_t* src, const int32_t* dst, const 
     HG_TRY(radix_sort(L.sort, E, nruns, bit_width((uint64_t)crows), (const uint32_t*)L.sort.ckeys,
                       (const uint32_t*)L.sort.vals[res], (const uint32_t*)L.sort.vals2[res], res, s, &x));
     const uint32_t *skey = L.sort.keys[x], *srun = L.sort.vals[x], *sdst = L.sort.vals2[x];
-    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, skey, E, nruns, crows, L.csc_ptr,
-                  (int32_t*)nullptr));
+    HG_TRY(launch("row_ptr_from_keys", row_ptr_from_keys, dim3(grid_for(E / 4 + 1)), dim3(256), 0, s, skey, E, nruns,
+                  crows, L.csc_ptr, (int32_t*)nullptr));
     // node-major rows: out-runs per node over its relations, their scan, then the runs
     HG_TRY(launch("node_out_counts", node_out_counts, dim3(grid_for(N)), dim3(256), 0, s, (const int32_t*)L.csc_ptr,
                   m, L.cnt));
